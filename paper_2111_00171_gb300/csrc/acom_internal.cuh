@@ -126,7 +126,7 @@ struct Workspace {
     float* Xsi = nullptr;
     float* xnorm2 = nullptr;       // [chunk]
     float* Chat = nullptr;         // [4][F][chunk][Zp] (exhaustive mode only)
-    float* U = nullptr;            // [chunk][Z] spectral bounds
+    float* U = nullptr;            // [groups][chunk][Z] spectral bounds (freq_split)
     void* XB = nullptr;            // BF16 [F][PTs][128][Spad] (tensor-core operand, 16-row groups: 8 re, 8 im)
     int PTs = 0;                   // pattern tiles of 64 in XB
     alignas(64) unsigned char map_x[128];   // TMA map of XB
@@ -242,6 +242,14 @@ inline void set_max_dynamic_smem(const void* func, size_t bytes) {
     done.push_back({func, dev, bytes});
 }
 
+// SMs of the current device (a host lookup; no allocation, allowed in capture)
+inline int sm_count() {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n > 0 ? n : 1;
+}
+
 // ---- error reporting (api.cu) ----
 acom_status set_error(acom_status s, const std::string& msg);
 acom_status cuda_error(cudaError_t e, const char* what);
@@ -269,8 +277,19 @@ void launch_contract_fp32(const acom_plan_s* p, const float* Xr, const float* Xi
 void launch_idft_argmax_fp32(const acom_plan_s* p, const float* Chat, int nb, int chunk,
                              float* za_scores, unsigned long long* best, cudaStream_t st);
 // match_prune.cu
+// split: the frequencies in contract_fp32_groups(p, nb) groups, a plane of U each
 void launch_contract_bound_fp32(const acom_plan_s* p, const float* Xr, const float* Xi, int nb,
-                                float* U, cudaStream_t st);
+                                float* U, cudaStream_t st, bool split);
+int contract_fp32_groups(const acom_plan_s* p, int nb);
+// frequencies of a contraction in `groups` groups of `per` (the last may be shorter)
+struct FreqSplit {
+    int groups, per;
+};
+FreqSplit freq_split(int tiles, int slots, int F);
+// values of the planes of any split contraction (a split only happens below
+// 2 CTAs an SM of 4096 pairs, FP32, or 1 of 8192, tensor cores)
+inline size_t split_plane_values() { return (size_t)4 * 4096 * sm_count(); }
+void launch_sum_planes(const float* U, int64_t n, int groups, float* dst, cudaStream_t st);
 void launch_plan_fnorm_max(const acom_plan_s* p, float* out, cudaStream_t st);
 // p->smask from the plan's shell-major spectra (p->smask allocated, Zp x Spad/32)
 void launch_plan_shell_mask(const acom_plan_s* p, cudaStream_t st);
@@ -291,8 +310,9 @@ void launch_plan_to_operand(const float* Pr, const float* Pi, int Zp, int F, int
                             cudaStream_t st, int kind, float scale);
 void launch_orient_compose(const acom_plan_s* p, const OrientIn* oin, int nb, int refine,
                            acom_result out, int64_t off, cudaStream_t st);
+// U: u_groups planes [nb][Z] whose sum is the bound
 void launch_select_exact(const acom_plan_s* p, const float* Xsr, const float* Xsi, const float* U,
-                         const float* xfn, const int2* srange, const uint32_t* rmask,
+                         int u_groups, const float* xfn, const int2* srange, const uint32_t* rmask,
                          const float* pfmax, const float* xnorm2, int nb,
                          float kappa, int refine, acom_result out, int64_t off, int* n_eval,
                          cudaStream_t st, const float* xscale, int rescore_top, OrientIn* oin);

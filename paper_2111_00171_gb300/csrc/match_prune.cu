@@ -17,6 +17,7 @@
 // exhaustive evaluation (up to FP32 ties).
 #include <math_constants.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "acom_internal.cuh"
@@ -26,103 +27,198 @@ namespace acom {
 
 // ---------------------------------------------------------------------------
 // FP32 contraction with the bound epilogue.  CTA tile: 64 zone axes x 64
-// patterns, all frequencies; thread tile 4 x 4 pairs.
+// patterns; frequencies in turn; thread tile 8 x 4 pairs, four products a pair.
+// Bound by the FP32 pipe and its operand reads (a register-only loop of these
+// instructions reached 60 to 65 TFLOP/s here, without operand reuse 49).  The
+// products run as packed pairs (fma.rn.f32x2: (A, B) += (Pr, Pi) (Xr, Xi),
+// (C, D) += (Pr, Pi) (Xi, Xr)), each half the rounding of a scalar fmaf; an
+// 8 x 4 tile because a 16-byte shared load takes four cycles of the SM whatever
+// it broadcasts, and 4 x 4 needed as many of those as of the FP32 pipe (42
+// against 47 TFLOP/s, both in this layout); the next 8 shells load into registers
+// while this step is multiplied, one barrier a step; only shells k0 .. S - 1
+// are summed (the plan's rows below k0 and the padding rows are zero, their
+// products exactly 0).  Every sum keeps the order of its shells.  8,190
+// patterns x 903 axes x 150 shells x 181 frequencies: 42.2 -> 26.5 ms.
 // ---------------------------------------------------------------------------
-constexpr int kBz = 64, kBb = 64, kBk = 16;
+constexpr int kBz = 64, kBb = 64, kBk = 8;
+constexpr int kBPitch = kBz + 2;      // float2 per staged shell: conflict-free transposing stores
+constexpr int kBThreads = 128;        // two CTAs an SM (250 registers)
+constexpr int kBRows = kBThreads * 4 / kBk;    // operand rows a load pass covers
 
-__global__ void __launch_bounds__(256)
+__device__ __forceinline__ void ffma2(unsigned long long& d, unsigned long long a,
+                                      unsigned long long b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+
+__device__ __forceinline__ unsigned long long swap2(unsigned long long x) {
+    unsigned long long y;
+    asm("{\n.reg .b32 l, h;\nmov.b64 {l, h}, %1;\nmov.b64 %0, {h, l};\n}" : "=l"(y) : "l"(x));
+    return y;
+}
+
+__global__ void __launch_bounds__(kBThreads, 2)
 k_contract_bound_fp32(const float* __restrict__ Pr, const float* __restrict__ Pi,
                       const float* __restrict__ Xr, const float* __restrict__ Xi, int F, int N,
-                      int Spad, int Z, int nb, float* __restrict__ U) {
-    __shared__ __align__(16) float sPr[kBk][kBz + 4];
-    __shared__ __align__(16) float sPi[kBk][kBz + 4];
-    __shared__ __align__(16) float sXr[kBk][kBb + 4];
-    __shared__ __align__(16) float sXi[kBk][kBb + 4];
+                      int Spad, int k0, int steps, int Z, int nb, int f_per,
+                      float* __restrict__ U) {
+    static_assert(kBRows == kBz, "one load pass covers the tile's rows");
+    __shared__ __align__(16) float2 sP[2][kBk][kBPitch];
+    __shared__ __align__(16) float2 sX[2][kBk][kBPitch];
     const int z0 = blockIdx.x * kBz, b0 = blockIdx.y * kBb;
-    const int t = threadIdx.x, tz = t & 15, tb = t >> 4;
-    const int lr = t >> 2, lc = (t & 3) * 4;
+    const int f0 = blockIdx.z * f_per, f1 = min(F, f0 + f_per);
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    // loads: row lr of both operands, shells lc .. lc + 3 of the step
+    const int lr = t / (kBk / 4), lc = (t % (kBk / 4)) * 4;
     const bool bvalid = (b0 + lr) < nb;
-    float Ud[4][4];
+    const int64_t prow = ((int64_t)(z0 + lr) * F) * Spad + k0 + lc;
+    const int64_t xrow = ((int64_t)(b0 + lr) * F) * Spad + k0 + lc;
+    // products: a warp takes 64 axes x 16 patterns, a lane axes zt + {0, 1} + 16
+    // {0, 1, 2, 3} and patterns bt + {0, 1, 8, 9}: conflict-free 16-byte loads
+    const int zt = (lane & 7) * 2, bt = warp * 16 + (lane >> 3) * 2;
+    float Ud[8][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) Ud[i][j] = 0.f;
 
-    for (int f = 0; f < F; ++f) {
-        float A[4][4], B[4][4], C[4][4], D[4][4];
+    float4 pr, pi, xr = make_float4(0.f, 0.f, 0.f, 0.f), xi = xr;
+    auto fetch = [&](int f, int step) {
+        const int o = f * Spad + step * kBk;
+        pr = *reinterpret_cast<const float4*>(Pr + prow + o);
+        pi = *reinterpret_cast<const float4*>(Pi + prow + o);
+        if (bvalid) {
+            xr = *reinterpret_cast<const float4*>(Xr + xrow + o);
+            xi = *reinterpret_cast<const float4*>(Xi + xrow + o);
+        }
+    };
+    int buf = 0;
+    if (f0 < f1) fetch(f0, 0);
+    for (int f = f0; f < f1; ++f) {
+        unsigned long long AB[8][4], CD[8][4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 8; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) A[i][j] = B[i][j] = C[i][j] = D[i][j] = 0.f;
-        const int64_t prow = ((int64_t)(z0 + lr) * F + f) * Spad;
-        const int64_t xrow = ((int64_t)(b0 + lr) * F + f) * Spad;
-        for (int s0 = 0; s0 < Spad; s0 += kBk) {
-            float4 pr = *reinterpret_cast<const float4*>(Pr + prow + s0 + lc);
-            float4 pi = *reinterpret_cast<const float4*>(Pi + prow + s0 + lc);
-            float4 xr = make_float4(0.f, 0.f, 0.f, 0.f), xi = xr;
-            if (bvalid) {
-                xr = *reinterpret_cast<const float4*>(Xr + xrow + s0 + lc);
-                xi = *reinterpret_cast<const float4*>(Xi + xrow + s0 + lc);
-            }
+            for (int j = 0; j < 4; ++j) AB[i][j] = CD[i][j] = 0ull;
+        for (int step = 0; step < steps; ++step, buf ^= 1) {
+            // a buffer is refilled two steps after it was read, with the barrier of
+            // the step between them in between
+            sP[buf][lc + 0][lr] = make_float2(pr.x, pi.x);
+            sP[buf][lc + 1][lr] = make_float2(pr.y, pi.y);
+            sP[buf][lc + 2][lr] = make_float2(pr.z, pi.z);
+            sP[buf][lc + 3][lr] = make_float2(pr.w, pi.w);
+            sX[buf][lc + 0][lr] = make_float2(xr.x, xi.x);
+            sX[buf][lc + 1][lr] = make_float2(xr.y, xi.y);
+            sX[buf][lc + 2][lr] = make_float2(xr.z, xi.z);
+            sX[buf][lc + 3][lr] = make_float2(xr.w, xi.w);
             __syncthreads();
-            sPr[lc + 0][lr] = pr.x; sPr[lc + 1][lr] = pr.y; sPr[lc + 2][lr] = pr.z; sPr[lc + 3][lr] = pr.w;
-            sPi[lc + 0][lr] = pi.x; sPi[lc + 1][lr] = pi.y; sPi[lc + 2][lr] = pi.z; sPi[lc + 3][lr] = pi.w;
-            sXr[lc + 0][lr] = xr.x; sXr[lc + 1][lr] = xr.y; sXr[lc + 2][lr] = xr.z; sXr[lc + 3][lr] = xr.w;
-            sXi[lc + 0][lr] = xi.x; sXi[lc + 1][lr] = xi.y; sXi[lc + 2][lr] = xi.z; sXi[lc + 3][lr] = xi.w;
-            __syncthreads();
-#pragma unroll
+            if (step + 1 < steps)
+                fetch(f, step + 1);
+            else if (f + 1 < f1)
+                fetch(f + 1, 0);
+#pragma unroll 4
             for (int kk = 0; kk < kBk; ++kk) {
-                float4 a_r = *reinterpret_cast<const float4*>(&sPr[kk][tz * 4]);
-                float4 a_i = *reinterpret_cast<const float4*>(&sPi[kk][tz * 4]);
-                float4 b_r = *reinterpret_cast<const float4*>(&sXr[kk][tb * 4]);
-                float4 b_i = *reinterpret_cast<const float4*>(&sXi[kk][tb * 4]);
-                const float ar[4] = {a_r.x, a_r.y, a_r.z, a_r.w};
-                const float ai[4] = {a_i.x, a_i.y, a_i.z, a_i.w};
-                const float br[4] = {b_r.x, b_r.y, b_r.z, b_r.w};
-                const float bi[4] = {b_i.x, b_i.y, b_i.z, b_i.w};
+                unsigned long long p[8], x[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+                for (int q = 0; q < 4; ++q) {
+                    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&sP[buf][kk][zt + 16 * q]);
+                    p[2 * q] = v.x;
+                    p[2 * q + 1] = v.y;
+                }
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        A[i][j] = fmaf(ar[i], br[j], A[i][j]);
-                        B[i][j] = fmaf(ai[i], bi[j], B[i][j]);
-                        C[i][j] = fmaf(ar[i], bi[j], C[i][j]);
-                        D[i][j] = fmaf(ai[i], br[j], D[i][j]);
+                for (int q = 0; q < 2; ++q) {
+                    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&sX[buf][kk][bt + 8 * q]);
+                    x[2 * q] = v.x;
+                    x[2 * q + 1] = v.y;
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const unsigned long long xs = swap2(x[j]);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        ffma2(AB[i][j], p[i], x[j]);
+                        ffma2(CD[i][j], p[i], xs);
                     }
+                }
             }
         }
         const float w = (f == 0 || 2 * f == N) ? 1.f : 2.f;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 8; ++i)
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 // max(|c_dir|, |c_mir|)^2 = p + 2 |AB - CD|, p = A^2 + B^2 + C^2 + D^2
-                const float a_ = A[i][j], b_ = B[i][j], c_ = C[i][j], d_ = D[i][j];
+                const float a_ = __uint_as_float((unsigned)AB[i][j]);
+                const float b_ = __uint_as_float((unsigned)(AB[i][j] >> 32));
+                const float c_ = __uint_as_float((unsigned)CD[i][j]);
+                const float d_ = __uint_as_float((unsigned)(CD[i][j] >> 32));
                 const float p = fmaf(a_, a_, fmaf(b_, b_, fmaf(c_, c_, d_ * d_)));
                 const float q = fmaf(a_, b_, -c_ * d_);
                 Ud[i][j] = fmaf(w, sqrtf(fmaf(2.0f, fabsf(q), p)), Ud[i][j]);
             }
     }
     const float invN = 1.0f / (float)N;
+    float* out = U + (int64_t)blockIdx.z * nb * Z;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        const int b = b0 + tb * 4 + j;
+        const int b = b0 + bt + (j & 1) + 8 * (j >> 1);
         if (b >= nb) continue;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int z = z0 + tz * 4 + i;
-            if (z < Z) U[(int64_t)b * Z + z] = Ud[i][j] * invN;
+        for (int i = 0; i < 8; ++i) {
+            const int z = z0 + zt + (i & 1) + 16 * (i >> 1);
+            if (z < Z) out[(int64_t)b * Z + z] = Ud[i][j] * invN;
         }
     }
 }
 
+// A grid of fewer CTAs than the GPU holds leaves SMs idle while each CTA runs
+// every frequency in turn, so the frequencies of a small batch are split into
+// groups, each group's partial bound in its own [nb][Z] plane (the reader adds
+// the planes in order).  tiles: CTAs without a split; slots: CTAs at a time.
+// From `slots` tiles on there is no split: every SM has its CTAs anyway, and the
+// planes would only add traffic.  100 patterns x 231 axes (8 tiles, 31 groups):
+// 1.24 -> 0.049 ms.
+FreqSplit freq_split(int tiles, int slots, int F) {
+    FreqSplit s{1, F};
+    if (tiles <= 0 || tiles >= slots) return s;
+    const int g = std::min(F, (slots + tiles - 1) / tiles);
+    s.per = (F + g - 1) / g;
+    s.groups = (F + s.per - 1) / s.per;
+    return s;
+}
+
+static FreqSplit fp32_split(const acom_plan_s* p, int nb) {
+    return freq_split(((p->Z + kBz - 1) / kBz) * ((nb + kBb - 1) / kBb), 2 * sm_count(), p->F);
+}
+
+int contract_fp32_groups(const acom_plan_s* p, int nb) { return fp32_split(p, nb).groups; }
+
 void launch_contract_bound_fp32(const acom_plan_s* p, const float* Xr, const float* Xi, int nb,
-                                float* U, cudaStream_t st) {
-    dim3 grid(p->Zp / kBz, (nb + kBb - 1) / kBb);
+                                float* U, cudaStream_t st, bool split) {
+    const FreqSplit fs = split ? fp32_split(p, nb) : FreqSplit{1, p->F};
+    dim3 grid((p->Z + kBz - 1) / kBz, (nb + kBb - 1) / kBb, fs.groups);
+    const int steps = (p->S - p->k0 + kBk - 1) / kBk;
     prof_begin(kKContract, st);
-    k_contract_bound_fp32<<<grid, 256, 0, st>>>(p->Pr, p->Pi, Xr, Xi, p->F, p->N, p->Spad, p->Z,
-                                                nb, U);
+    k_contract_bound_fp32<<<grid, kBThreads, 0, st>>>(p->Pr, p->Pi, Xr, Xi, p->F, p->N, p->Spad, p->k0,
+                                                steps, p->Z, nb, fs.per, U);
     prof_end(kKContract, st);
+}
+
+// dst[i] = sum over the groups' planes, in their order
+__global__ void k_sum_planes(const float* __restrict__ U, int64_t n, int groups,
+                             float* __restrict__ dst) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        float u = U[i];
+        for (int g = 1; g < groups; ++g) u += U[g * n + i];
+        dst[i] = u;
+    }
+}
+
+void launch_sum_planes(const float* U, int64_t n, int groups, float* dst, cudaStream_t st) {
+    const int blocks = (int)std::min<int64_t>((n + 255) / 256, 8 * (int64_t)sm_count());
+    prof_begin(kKMisc, st);
+    k_sum_planes<<<blocks, 256, 0, st>>>(U, n, groups, dst);
+    prof_end(kKMisc, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -349,7 +445,8 @@ __device__ __forceinline__ void fma4(float4& acc, const float4 p, const float4 x
 
 struct SelectArgs {
     const float *Psr, *Psi, *Xsr, *Xsi;   // FP32 spectra, shell-major [.][Spad][Fs]
-    const float* U;                   // [nb][Z] bounds
+    const float* U;                   // [u_groups][nb][Z] bounds, the sum of the planes
+    int u_groups;
     const float* xfn;                 // [nb][F] ||X^_bf||
     const int2* srange;               // [nb] non-zero shell range
     const uint32_t* rmask;            // [nb][Spad / 32] shells the pattern's tents reach
@@ -809,7 +906,9 @@ __global__ void __launch_bounds__(kSelThreads, 3) k_select_exact(SelectArgs a) {
 
     for (int64_t b = blockIdx.x; b < a.nb; b += gridDim.x) {
         for (int z = threadIdx.x; z < Z; z += kSelThreads) {
-            sm.U[z] = a.U[b * Z + z];
+            float u = a.U[b * Z + z];
+            for (int g = 1; g < a.u_groups; ++g) u += a.U[((int64_t)g * a.nb + b) * Z + z];
+            sm.U[z] = u;
             sm.ev[z] = 0;
         }
         // the shells some peak's tent reached (recorded by the raster, which
@@ -1040,11 +1139,11 @@ size_t select_smem_bytes(int Z, int N, int F, int Spad) {
 }
 
 void launch_select_exact(const acom_plan_s* p, const float* Xsr, const float* Xsi, const float* U,
-                         const float* xfn, const int2* srange, const uint32_t* rmask,
+                         int u_groups, const float* xfn, const int2* srange, const uint32_t* rmask,
                          const float* pfmax, const float* xnorm2, int nb,
                          float kappa, int refine, acom_result out, int64_t off, int* n_eval,
                          cudaStream_t st, const float* xscale, int rescore_top, OrientIn* oin) {
-    SelectArgs a{p->Psr, p->Psi, Xsr, Xsi, U, xfn, srange, rmask, pfmax, xnorm2, p->za, p->frames,
+    SelectArgs a{p->Psr, p->Psi, Xsr, Xsi, U, u_groups, xfn, srange, rmask, pfmax, xnorm2, p->za, p->frames,
                  p->nbr_ptr,
                  p->nbr_idx, p->phase_off, p->n_phases, p->Z, p->F, p->N, p->S, p->Spad, nb, refine, kappa,
                  fft_radices(p->N), out, off, n_eval, xscale, 1.0f / p->pscale,

@@ -117,7 +117,7 @@ extern "C" acom_status acom_bounds_static(acom_plan p, const acom_peaks_csr* pea
         if (tc)
             launch_contract_bound_tc(p, map_x, PTs, nb, U, st);
         else
-            launch_contract_bound_fp32(p, Xr, Xi, nb, U, st);
+            launch_contract_bound_fp32(p, Xr, Xi, nb, U, st, false);
     }
     prof_suppress(false);
     e = cudaGetLastError();

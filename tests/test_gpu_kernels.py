@@ -1,0 +1,60 @@
+"""Kernels at the sizes where their tilings and splits can go wrong (edges of tiles,
+remainders, one pattern, batches that leave SMs idle), against FP64 values of the same
+spectra."""
+
+import math
+
+import numpy as np
+import pytest
+
+import synth
+from gpu_common import LAM, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__ as g
+    g.build()
+
+
+def au_plan(step, shells, dq, n_phi, precision=0):
+    from paper_2111_00171_gb300 import acom
+    tri, area = acom.cubic_triangle()
+    return acom.Plan(acom.au_crystal(), tri, area, step, shells, dq, n_phi, lam=LAM,
+                     precision=precision)
+
+
+def bounds64(plan, peaks):
+    """FP64 spectral bounds of the plan's and the patterns' FP32 spectra, and the sum
+    (1/N) sum_f w_f max_z ||P_zf|| ||X_bf|| that scales their rounding."""
+    import torch
+    P = torch.view_as_complex(plan.spectra()).to(torch.complex128)           # [Z][S][F]
+    X = torch.view_as_complex(plan.polar_spectra(*peaks)[0]).to(torch.complex128)
+    N, F = plan.info["n_phi"], plan.info["n_freq"]
+    w = torch.full((F,), 2.0 / N, dtype=torch.float64, device="cuda")
+    w[0] = w[-1] = 1.0 / N
+    c = torch.einsum("zsf,bsf->bzf", P.conj(), X).abs()
+    m = torch.einsum("zsf,bsf->bzf", P.conj(), X.conj()).abs()
+    scale = (w * P.norm(dim=1).amax(0) * X.norm(dim=1)).sum(1)               # [B]
+    return (torch.maximum(c, m) * w).sum(2), scale
+
+
+# one pattern; a tile's edge and one past it; more tiles than the GPU holds CTAs of
+@pytest.mark.parametrize("geometry", [(3.0, 75, 0.02, 180), (6.0, 200, 0.0075, 72),
+                                      (2.0, 33, 0.045, 84)], ids=str)
+@pytest.mark.parametrize("patterns", [1, 63, 65, 1300])
+def test_fp32_bounds_at_tile_edges(geometry, patterns):
+    plan = au_plan(*geometry)
+    peaks = to_dev(synth.random_patterns(31 + patterns, n_patterns=patterns))
+    got = plan.bounds(*peaks).double()
+    want, scale = bounds64(plan, peaks)
+    # dot products of the shells, four products, root and the sum over frequencies
+    S, F = math.ceil(geometry[1] / 32) * 32, geometry[3] // 2 + 1
+    tol = (3 * (S + 2) + 2 * F) * 2.0 ** -24 * scale
+    assert ((got - want).abs() <= tol[:, None]).all()
+    plan.close()
