@@ -126,7 +126,8 @@ struct Workspace {
     float* Xsi = nullptr;
     float* xnorm2 = nullptr;       // [chunk]
     float* Chat = nullptr;         // [4][F][chunk][Zp] (exhaustive mode only)
-    float* U = nullptr;            // [groups][chunk][Z] spectral bounds (freq_split)
+    float* U = nullptr;            // [chunk][Z] spectral bounds
+    float* extra = nullptr;        // later groups' bounds of split tiles (TileSplit)
     void* XB = nullptr;            // BF16 [F][PTs][128][Spad] (tensor-core operand, 16-row groups: 8 re, 8 im)
     int PTs = 0;                   // pattern tiles of 64 in XB
     alignas(64) unsigned char map_x[128];   // TMA map of XB
@@ -250,6 +251,44 @@ inline int sm_count() {
     return n > 0 ? n : 1;
 }
 
+// How a contraction's tiles (ZT axis tiles x PTu pattern tiles, 2^lz axes x 2^lb
+// patterns) are cut into units: tile t < first is one unit; each later tile is
+// `groups` units of `per` frequencies (the last may be shorter).  Group 0 of a
+// split tile writes its partial bound to U, group g > 0 to plane g - 1 of
+// `extra` (tile-local), and the reader adds them in order.
+struct TileSplit {
+    int first = 0, groups = 1, per = 0;
+    int ZT = 0, PTu = 0, zmajor = 0, lb = 0, lz = 0;
+    __host__ __device__ int all() const { return ZT * PTu; }
+    __host__ __device__ int tiles() const { return all() - first; }        // split tiles
+    __host__ __device__ int units() const { return first + tiles() * groups; }
+    __host__ __device__ int64_t extra_at(int g, int t, int b, int z) const {
+        return ((((int64_t)(g - 1) * tiles() + (t - first)) << (lb + lz)) |
+                ((int64_t)(b & ((1 << lb) - 1)) << lz)) | (z & ((1 << lz) - 1));
+    }
+    // tile t of pattern b, axis z, when it is split; else -1
+    __host__ __device__ int split_tile(int b, int z) const {
+        const int t = zmajor ? (z >> lz) * PTu + (b >> lb) : (b >> lb) * ZT + (z >> lz);
+        return t >= first ? t : -1;
+    }
+    // full waves of `wave` tiles whole; the rest in groups so that about `slots`
+    // units run at a time
+    void set(int wave, int slots, int F, bool split) {
+        const int n = all();
+        first = n;
+        groups = 1;
+        per = F;
+        const int rest = n % wave;
+        if (!split || rest == 0 || slots / rest < 2) return;
+        const int g = slots / rest < F ? slots / rest : F;
+        first = n - rest;
+        per = (F + g - 1) / g;
+        groups = (F + per - 1) / per;
+    }
+};
+// floats of `extra` for any split: (groups - 1) tiles <= slots
+inline size_t split_extra_floats() { return (size_t)sm_count() << 14; }
+
 // ---- error reporting (api.cu) ----
 acom_status set_error(acom_status s, const std::string& msg);
 acom_status cuda_error(cudaError_t e, const char* what);
@@ -277,19 +316,13 @@ void launch_contract_fp32(const acom_plan_s* p, const float* Xr, const float* Xi
 void launch_idft_argmax_fp32(const acom_plan_s* p, const float* Chat, int nb, int chunk,
                              float* za_scores, unsigned long long* best, cudaStream_t st);
 // match_prune.cu
-// split: the frequencies in contract_fp32_groups(p, nb) groups, a plane of U each
+// ts from fp32_split; extra: the later groups' bounds of split tiles
+TileSplit fp32_split(const acom_plan_s* p, int nb, bool split);
 void launch_contract_bound_fp32(const acom_plan_s* p, const float* Xr, const float* Xi, int nb,
-                                float* U, cudaStream_t st, bool split);
-int contract_fp32_groups(const acom_plan_s* p, int nb);
-// frequencies of a contraction in `groups` groups of `per` (the last may be shorter)
-struct FreqSplit {
-    int groups, per;
-};
-FreqSplit freq_split(int tiles, int slots, int F);
-// values of the planes of any split contraction (a split only happens below
-// 2 CTAs an SM of 4096 pairs, FP32, or 1 of 8192, tensor cores)
-inline size_t split_plane_values() { return (size_t)4 * 4096 * sm_count(); }
-void launch_sum_planes(const float* U, int64_t n, int groups, float* dst, cudaStream_t st);
+                                const TileSplit& ts, float* U, float* extra, cudaStream_t st);
+// adds the later groups' bounds of the split tiles to U [nb][Z]
+void launch_sum_groups(const TileSplit& ts, float* U, const float* extra, int nb, int Z,
+                       cudaStream_t st);
 void launch_plan_fnorm_max(const acom_plan_s* p, float* out, cudaStream_t st);
 // p->smask from the plan's shell-major spectra (p->smask allocated, Zp x Spad/32)
 void launch_plan_shell_mask(const acom_plan_s* p, cudaStream_t st);
@@ -301,18 +334,19 @@ void launch_half_to_e4m3(const void* src, void* dst, int64_t n, float mul, cudaS
 void set_wait_cycles(long long cycles);
 // xscale: per-pattern 2^e of FP16 pattern spectra (nullptr: BF16, no scale)
 // cta_pairs: 0 one CTA per MMA (cta_group::1), 1 CTA pairs (cta_group::2)
+TileSplit tc_split(const acom_plan_s* p, int nb, int tile_order, bool split);
 void launch_contract_bound_tc(const acom_plan_s* p, const void* map_x, int pt_stride, int nb,
-                              float* U, cudaStream_t st, const float* xscale = nullptr,
-                              int tile_order = 0, int cta_pairs = 0);
+                              const TileSplit& ts, float* U, float* extra, cudaStream_t st,
+                              const float* xscale = nullptr, int cta_pairs = 0);
 // the plan's FP32 spectra Pr, Pi [Zp][F][Spad] -> the merged operand p->Pb:
 // BF16 of P^ (kind 0), FP16 (1) or E4M3 (2) of scale * P^
 void launch_plan_to_operand(const float* Pr, const float* Pi, int Zp, int F, int Spad, void* dst,
                             cudaStream_t st, int kind, float scale);
 void launch_orient_compose(const acom_plan_s* p, const OrientIn* oin, int nb, int refine,
                            acom_result out, int64_t off, cudaStream_t st);
-// U: u_groups planes [nb][Z] whose sum is the bound
+// U: bounds, `extra` the later groups' of split tiles (TileSplit)
 void launch_select_exact(const acom_plan_s* p, const float* Xsr, const float* Xsi, const float* U,
-                         int u_groups, const float* xfn, const int2* srange, const uint32_t* rmask,
+                         const float* extra, const TileSplit& ts, const float* xfn, const int2* srange, const uint32_t* rmask,
                          const float* pfmax, const float* xnorm2, int nb,
                          float kappa, int refine, acom_result out, int64_t off, int* n_eval,
                          cudaStream_t st, const float* xscale, int rescore_top, OrientIn* oin);

@@ -148,6 +148,7 @@ static void free_workspace(Workspace& ws, cudaStream_t st) {
     pool_free(ws.xnorm2, st);
     pool_free(ws.Chat, st);
     pool_free(ws.U, st);
+    pool_free(ws.extra, st);
     pool_free(ws.xfn, st);
     pool_free(ws.n_eval, st);
     pool_free(ws.srange, st);
@@ -187,12 +188,8 @@ static acom_status ensure_ws(acom_plan_s* p, Workspace& ws, int chunk, bool need
     if (need_chat &&
         (e = dalloc(&ws.Chat, (size_t)4 * p->F * chunk * p->Zp, &acc, st)) != cudaSuccess)
         goto fail;
-    // room for the planes of a split contraction (at most one a frequency)
-    if ((e = dalloc(&ws.U,
-                    std::max((size_t)chunk * p->Z,
-                             std::min((size_t)chunk * p->Z * p->F, split_plane_values())),
-                    &acc, st)) != cudaSuccess)
-        goto fail;
+    if ((e = dalloc(&ws.U, (size_t)chunk * p->Z, &acc, st)) != cudaSuccess) goto fail;
+    if ((e = dalloc(&ws.extra, split_extra_floats(), &acc, st)) != cudaSuccess) goto fail;
     if ((e = dalloc(&ws.xfn, (size_t)chunk * p->F, &acc, st)) != cudaSuccess) goto fail;
     if ((e = dalloc(&ws.n_eval, (size_t)1, &acc, st)) != cudaSuccess) goto fail;
     if ((e = dalloc(&ws.srange, (size_t)chunk, &acc, st)) != cudaSuccess) goto fail;
@@ -859,16 +856,15 @@ static acom_status match_enqueue(acom_plan p, const acom_peaks_csr* peaks,
             if (out->phase || out->phase_score)
                 launch_phase_outputs(p, w.za_scores, nb, *out, c0, st);
         } else {
-            int groups = 1;
+            const TileSplit ts = tc ? tc_split(p, nb, tile_order, true) : fp32_split(p, nb, true);
             if (tc) {
                 convert_fp8(p, w, st);
-                launch_contract_bound_tc(p, w.map_x, w.PTs, nb, w.U, st, xscale, tile_order,
+                launch_contract_bound_tc(p, w.map_x, w.PTs, nb, ts, w.U, w.extra, st, xscale,
                                          cta_pairs);
             } else {
-                groups = contract_fp32_groups(p, nb);
-                launch_contract_bound_fp32(p, w.Xr, w.Xi, nb, w.U, st, true);
+                launch_contract_bound_fp32(p, w.Xr, w.Xi, nb, ts, w.U, w.extra, st);
             }
-            launch_select_exact(p, w.Xsr, w.Xsi, w.U, groups, w.xfn, w.srange, w.rmask, p->pfmax,
+            launch_select_exact(p, w.Xsr, w.Xsi, w.U, w.extra, ts, w.xfn, w.srange, w.rmask, p->pfmax,
                                 w.xnorm2, nb, tc ? kappa_tc(p) : kappa_fp32(p), refine, *out,
                                 c0, w.n_eval, st, xscale, rescore_top, w.oin);
             if (out->phi3 || out->orient)
@@ -960,15 +956,14 @@ acom_status acom_bounds(acom_plan p, const acom_peaks_csr* peaks, float* dst, vo
         ro.sumsq = p->ws.xnorm2;
         launch_raster_patterns(geo, src, ro, p->err, st);
         float* U = dst + c0 * (int64_t)p->Z;
+        const TileSplit ts = tc ? tc_split(p, nb, 0, true) : fp32_split(p, nb, true);
         if (tc) {
             convert_fp8(p, p->ws, st);
-            launch_contract_bound_tc(p, p->ws.map_x, p->ws.PTs, nb, U, st, xscale);
+            launch_contract_bound_tc(p, p->ws.map_x, p->ws.PTs, nb, ts, U, p->ws.extra, st, xscale);
         } else {
-            const int groups = contract_fp32_groups(p, nb);
-            launch_contract_bound_fp32(p, p->ws.Xr, p->ws.Xi, nb, groups > 1 ? p->ws.U : U, st,
-                                       true);
-            if (groups > 1) launch_sum_planes(p->ws.U, (int64_t)nb * p->Z, groups, U, st);
+            launch_contract_bound_fp32(p, p->ws.Xr, p->ws.Xi, nb, ts, U, p->ws.extra, st);
         }
+        launch_sum_groups(ts, U, p->ws.extra, nb, p->Z, st);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "bounds launch");

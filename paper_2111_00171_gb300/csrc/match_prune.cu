@@ -59,13 +59,13 @@ __device__ __forceinline__ unsigned long long swap2(unsigned long long x) {
 __global__ void __launch_bounds__(kBThreads, 2)
 k_contract_bound_fp32(const float* __restrict__ Pr, const float* __restrict__ Pi,
                       const float* __restrict__ Xr, const float* __restrict__ Xi, int F, int N,
-                      int Spad, int k0, int steps, int Z, int nb, int f_per,
-                      float* __restrict__ U) {
+                      int Spad, int k0, int steps, int Z, int nb, TileSplit ts,
+                      float* __restrict__ U, float* __restrict__ extra) {
     static_assert(kBRows == kBz, "one load pass covers the tile's rows");
     __shared__ __align__(16) float2 sP[2][kBk][kBPitch];
     __shared__ __align__(16) float2 sX[2][kBk][kBPitch];
     const int z0 = blockIdx.x * kBz, b0 = blockIdx.y * kBb;
-    const int f0 = blockIdx.z * f_per, f1 = min(F, f0 + f_per);
+    const int g = blockIdx.z, f0 = g * ts.per, f1 = min(F, f0 + ts.per);
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     // loads: row lr of both operands, shells lc .. lc + 3 of the step
     const int lr = t / (kBk / 4), lc = (t % (kBk / 4)) * 4;
@@ -157,7 +157,6 @@ k_contract_bound_fp32(const float* __restrict__ Pr, const float* __restrict__ Pi
             }
     }
     const float invN = 1.0f / (float)N;
-    float* out = U + (int64_t)blockIdx.z * nb * Z;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const int b = b0 + bt + (j & 1) + 8 * (j >> 1);
@@ -165,59 +164,63 @@ k_contract_bound_fp32(const float* __restrict__ Pr, const float* __restrict__ Pi
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int z = z0 + zt + (i & 1) + 16 * (i >> 1);
-            if (z < Z) out[(int64_t)b * Z + z] = Ud[i][j] * invN;
+            if (z < Z)
+                *(g == 0 ? U + (int64_t)b * Z + z
+                         : extra + ts.extra_at(g, ts.split_tile(b, z), b, z)) = Ud[i][j] * invN;
         }
     }
 }
 
-// A grid of fewer CTAs than the GPU holds leaves SMs idle while each CTA runs
-// every frequency in turn, so the frequencies of a small batch are split into
-// groups, each group's partial bound in its own [nb][Z] plane (the reader adds
-// the planes in order).  tiles: CTAs without a split; slots: CTAs at a time.
-// From `slots` tiles on there is no split: every SM has its CTAs anyway, and the
-// planes would only add traffic.  100 patterns x 231 axes (8 tiles, 31 groups):
-// 1.24 -> 0.049 ms.
-FreqSplit freq_split(int tiles, int slots, int F) {
-    FreqSplit s{1, F};
-    if (tiles <= 0 || tiles >= slots) return s;
-    const int g = std::min(F, (slots + tiles - 1) / tiles);
-    s.per = (F + g - 1) / g;
-    s.groups = (F + s.per - 1) / s.per;
-    return s;
+// A grid of fewer CTAs than the GPU holds (two an SM) leaves SMs idle while each
+// CTA runs every frequency in turn, so a small batch's frequencies are split
+// into groups.  From two CTAs an SM on there is no split: every SM has its CTAs
+// anyway, and the partial bounds would only add traffic.  100 patterns x 231
+// axes (8 tiles, 31 groups): 1.24 -> 0.049 ms.
+TileSplit fp32_split(const acom_plan_s* p, int nb, bool split) {
+    TileSplit ts;
+    ts.ZT = (p->Z + kBz - 1) / kBz;
+    ts.PTu = (nb + kBb - 1) / kBb;
+    ts.lb = ts.lz = 6;
+    const int slots = 2 * sm_count();
+    ts.set(ts.all() < slots ? slots : 1, slots, p->F, split);
+    return ts;
 }
-
-static FreqSplit fp32_split(const acom_plan_s* p, int nb) {
-    return freq_split(((p->Z + kBz - 1) / kBz) * ((nb + kBb - 1) / kBb), 2 * sm_count(), p->F);
-}
-
-int contract_fp32_groups(const acom_plan_s* p, int nb) { return fp32_split(p, nb).groups; }
 
 void launch_contract_bound_fp32(const acom_plan_s* p, const float* Xr, const float* Xi, int nb,
-                                float* U, cudaStream_t st, bool split) {
-    const FreqSplit fs = split ? fp32_split(p, nb) : FreqSplit{1, p->F};
-    dim3 grid((p->Z + kBz - 1) / kBz, (nb + kBb - 1) / kBb, fs.groups);
+                                const TileSplit& ts, float* U, float* extra, cudaStream_t st) {
+    dim3 grid(ts.ZT, ts.PTu, ts.groups);
     const int steps = (p->S - p->k0 + kBk - 1) / kBk;
     prof_begin(kKContract, st);
-    k_contract_bound_fp32<<<grid, kBThreads, 0, st>>>(p->Pr, p->Pi, Xr, Xi, p->F, p->N, p->Spad, p->k0,
-                                                steps, p->Z, nb, fs.per, U);
+    k_contract_bound_fp32<<<grid, kBThreads, 0, st>>>(p->Pr, p->Pi, Xr, Xi, p->F, p->N, p->Spad,
+                                                      p->k0, steps, p->Z, nb, ts, U, extra);
     prof_end(kKContract, st);
 }
 
-// dst[i] = sum over the groups' planes, in their order
-__global__ void k_sum_planes(const float* __restrict__ U, int64_t n, int groups,
-                             float* __restrict__ dst) {
+// a split tile's later groups, in their order
+__device__ __forceinline__ float later_groups(const TileSplit& ts, const float* __restrict__ extra,
+                                              int b, int z, float u) {
+    const int t = ts.groups > 1 ? ts.split_tile(b, z) : -1;
+    if (t >= 0)
+        for (int g = 1; g < ts.groups; ++g) u += extra[ts.extra_at(g, t, b, z)];
+    return u;
+}
+
+__global__ void k_sum_groups(TileSplit ts, float* __restrict__ U, const float* __restrict__ extra,
+                             int64_t n, int Z) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
-        float u = U[i];
-        for (int g = 1; g < groups; ++g) u += U[g * n + i];
-        dst[i] = u;
+        const int b = (int)(i / Z);
+        U[i] = later_groups(ts, extra, b, (int)(i - (int64_t)b * Z), U[i]);
     }
 }
 
-void launch_sum_planes(const float* U, int64_t n, int groups, float* dst, cudaStream_t st) {
+void launch_sum_groups(const TileSplit& ts, float* U, const float* extra, int nb, int Z,
+                       cudaStream_t st) {
+    if (ts.groups <= 1) return;
+    const int64_t n = (int64_t)nb * Z;
     const int blocks = (int)std::min<int64_t>((n + 255) / 256, 8 * (int64_t)sm_count());
     prof_begin(kKMisc, st);
-    k_sum_planes<<<blocks, 256, 0, st>>>(U, n, groups, dst);
+    k_sum_groups<<<blocks, 256, 0, st>>>(ts, U, extra, n, Z);
     prof_end(kKMisc, st);
 }
 
@@ -445,8 +448,9 @@ __device__ __forceinline__ void fma4(float4& acc, const float4 p, const float4 x
 
 struct SelectArgs {
     const float *Psr, *Psi, *Xsr, *Xsi;   // FP32 spectra, shell-major [.][Spad][Fs]
-    const float* U;                   // [u_groups][nb][Z] bounds, the sum of the planes
-    int u_groups;
+    const float* U;                   // [nb][Z] bounds
+    const float* extra;               // their later groups (TileSplit)
+    TileSplit ts;
     const float* xfn;                 // [nb][F] ||X^_bf||
     const int2* srange;               // [nb] non-zero shell range
     const uint32_t* rmask;            // [nb][Spad / 32] shells the pattern's tents reach
@@ -906,9 +910,7 @@ __global__ void __launch_bounds__(kSelThreads, 3) k_select_exact(SelectArgs a) {
 
     for (int64_t b = blockIdx.x; b < a.nb; b += gridDim.x) {
         for (int z = threadIdx.x; z < Z; z += kSelThreads) {
-            float u = a.U[b * Z + z];
-            for (int g = 1; g < a.u_groups; ++g) u += a.U[((int64_t)g * a.nb + b) * Z + z];
-            sm.U[z] = u;
+            sm.U[z] = later_groups(a.ts, a.extra, (int)b, z, a.U[b * Z + z]);
             sm.ev[z] = 0;
         }
         // the shells some peak's tent reached (recorded by the raster, which
@@ -1139,11 +1141,11 @@ size_t select_smem_bytes(int Z, int N, int F, int Spad) {
 }
 
 void launch_select_exact(const acom_plan_s* p, const float* Xsr, const float* Xsi, const float* U,
-                         int u_groups, const float* xfn, const int2* srange, const uint32_t* rmask,
+                         const float* extra, const TileSplit& ts, const float* xfn, const int2* srange, const uint32_t* rmask,
                          const float* pfmax, const float* xnorm2, int nb,
                          float kappa, int refine, acom_result out, int64_t off, int* n_eval,
                          cudaStream_t st, const float* xscale, int rescore_top, OrientIn* oin) {
-    SelectArgs a{p->Psr, p->Psi, Xsr, Xsi, U, u_groups, xfn, srange, rmask, pfmax, xnorm2, p->za, p->frames,
+    SelectArgs a{p->Psr, p->Psi, Xsr, Xsi, U, extra, ts, xfn, srange, rmask, pfmax, xnorm2, p->za, p->frames,
                  p->nbr_ptr,
                  p->nbr_idx, p->phase_off, p->n_phases, p->Z, p->F, p->N, p->S, p->Spad, nb, refine, kappa,
                  fft_radices(p->N), out, off, n_eval, xscale, 1.0f / p->pscale,

@@ -16,31 +16,29 @@
 // w_f max(|(A+B) + i(C-D)|, |(A-B) - i(C+D)|) over f.  The spectra never leave
 // the chip; only U is written.
 //
-// A thread issues one tcgen05.mma per ~120 cycles whatever its size, about the
-// time an M = 128, N = 256, K = 16 MMA takes on the tensor core, and every
-// barrier round trip and commit between MMAs leaves the tensor core idle.  So
-// one N = 256 MMA per 16 shells, and two issuing warps: warp 1 takes the even
-// frequencies into TMEM buffer 0, warp 2 the odd ones into buffer 1, and their
-// MMAs interleave in the tensor pipe.  Both consume stages of one operand ring
-// in the producer's order; each issuer has its own full barrier per ring slot
-// (the producer signals the stage's owner), so every full barrier has one
-// consumer and its phases are consumed in order.  A slot's empty barrier is
-// committed by the owner of each use; the producer issues the next use only
-// after that commit, so those phases are ordered too.
+// CTA tile: 128 patterns (two MMA tiles of 64) x 128 axes.  Per frequency the plan
+// operand (64 KB on the 1-degree plan) is loaded once and multiplied with both
+// pattern tiles: 128 KB of L2 reads per 16 MMAs instead of 192 with one pattern
+// tile, whose loads alone took 6.2 of its 9.0 ms on 65,536 patterns x 903 axes.
+// That scan: 9.06 -> 7.14 ms (1,810 TFLOP/s of 8 Z S F algorithmic flops); 16,000
+// patterns x 3,486 axes: 8.04 -> 6.34 ms.  What bounds it now, from timed copies of the
+// kernel: an MMA reads 12 KB of shared memory in its 128 cycles and the copies
+// write 62 bytes a cycle, 1.2 times the 128 bytes a cycle there are; and the epilogue
+// is as long as the MMAs it runs under (without its arithmetic 6.3 ms, without the
+// copies 6.6, without both 5.9).  The two pattern tiles alternate between two TMEM
+// accumulators, so a tile's epilogue has the other tile's MMAs to run under.
 //
-// CTA: two TMA producer warps (warp 0 loads the pattern operand X, warp 3 the
-// plan operand: one box of 256 rows, the axis tile's real rows followed by its
-// imaginary rows), two MMA-issuing warps, sixteen epilogue warps; persistent
-// over (64-pattern x 128-axis) tiles; with 16-bit operands a ring stage holds
-// two K tiles of 64 elements (128-byte rows, 128-byte swizzle), the whole K
-// range of a frequency on the 1-degree plan, in two stages of 96 KB, and each
-// K tile completes on its own full barrier, so the first K tile's MMAs start
-// while the second K tile lands; accumulators are double-buffered over f in
-// 512 TMEM columns.  Issuing a TMA copy costs the
-// issuing thread a few hundred cycles whatever the box (measured: one thread
-// issuing three boxes per stage was busy 80 % of the time, and halving the
-// boxes' rows or bytes changed nothing), so the copies of a stage are
-// issued by two threads and the plan operand is one box.
+// Warps: 0 loads the pattern operand (three 32 KB slots of two K tiles), 3 the plan
+// operand (two 64 KB slots; one box of 256 rows, the axis tile's real rows followed
+// by its imaginary rows), 1 issues every MMA, 2 hands slots back, 4 to 19 are the
+// epilogue.  Issuing costs the thread about 50 cycles an MMA, whatever its size, and
+// a commit 220 (measured; 380 under a `lane == 0` branch instead of elect.sync), and
+// the M = 128, N = 256, K = 16 MMA takes 128: one thread keeps the tensor pipe
+// busy as long as it commits about once per 8 MMAs.  So the issuer commits once per
+// accumulation, and warp 2, which waits for that, releases its operand slots; only
+// the earlier K stages of plans of more than 128 shells commit their own slots.
+// Each K tile has its own full barrier, so MMAs start on the first K tile while
+// the second lands.
 // Every mbarrier wait is bounded: a timeout sets the device error word, stops
 // all roles, drains copies and MMAs in flight, frees TMEM and returns.
 #include <cuda.h>
@@ -61,8 +59,8 @@ constexpr int kKT = 64;               // 16-bit operands per K tile row (128 byt
 constexpr int kKT8 = 128;             // 8-bit operands per K tile row (128 bytes)
 constexpr int kTileBytes = 128 * kKT * 2;      // 16 KB
 constexpr int kEpiWarps = 16;
-constexpr int kIssuers = 2;                    // MMA-issuing warps, one per TMEM buffer
-constexpr int kProdP = 1 + kIssuers;           // warp of the plan-operand producer
+constexpr int kIssuers = 2;                    // MMA-issuing warps of a CTA pair, one per TMEM buffer
+constexpr int kProdP = 3;                      // warp of the plan-operand producer
 constexpr int kEpi0 = kProdP + 1;               // first epilogue warp
 constexpr int kThreads = (kEpi0 + kEpiWarps) * 32;
 constexpr uint32_t kTmemCols = 512;
@@ -119,6 +117,19 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
             return false;
         }
     }
+}
+
+// one lane of the (converged) warp, known to the compiler to be one
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "elect.sync _|p, 0xffffffff;\n"
+        "selp.u32 %0, 1, 0, p;\n"
+        "}\n"
+        : "=r"(p));
+    return p != 0;
 }
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y,
@@ -303,8 +314,8 @@ __device__ __forceinline__ void accumulate_pair2(uint32_t a0, uint32_t a1, uint3
         "mul.rn.f32x2 R, A, B;\n"
         "sub.rn.f32x2 Q, R, Q;\n"
         "and.b64 Q, Q, 0x7FFFFFFF7FFFFFFF;\n"
-        "add.rn.f32x2 Q, Q, Q;\n"
-        "add.rn.f32x2 P, P, Q;\n"
+        "mov.b64 R, 0x4000000040000000;\n"
+        "fma.rn.f32x2 P, Q, R, P;\n"
         "mov.b64 {%0, %1}, P;\n"
         "}\n"
         : "=f"(t0), "=f"(t1)
@@ -314,73 +325,390 @@ __device__ __forceinline__ void accumulate_pair2(uint32_t a0, uint32_t a1, uint3
 }
 
 struct TcArgs {
-    int F, N, Z, nb, ZT, PT, KT;   // frequencies, bins, axes, patterns, axis tiles, pattern tiles, K tiles
+    int F, N, Z, nb, ZT, PT, KT;   // frequencies, bins, axes, patterns, axis tiles, pattern tiles, K stages
+    TileSplit ts;                  // tiles (axis tile x two pattern tiles) and their frequency groups
     int PTs;                       // pattern tiles per frequency in the pattern map (row stride)
     int Spad;                      // shells (K) in the operand rows
     int k0;                        // first shell of the contraction's K range (the
                                    // plan's rows below it are zero for every axis)
     int Zrows;                     // rows per frequency in the plan map (ZT * 256)
     float* U;                      // [nb][Z]
+    float* extra;                  // the later groups' bounds of split tiles (TileSplit)
     int* err;
     uint32_t idesc;                // MMA instruction descriptor (operand format)
     const float* xscale;           // [nb] 2^e of FP16 pattern spectra, or nullptr
     float xs_mul;                  // the operands hold xscale * xs_mul times X^
     float inv_pscale;              // 2^-k of the plan operand's scale (1 for BF16)
-    int zmajor;                    // tile order: 0 consecutive tiles share a pattern
-                                   // tile, 1 they share an axis tile
     long long wait_cycles;         // budget of each pipeline wait (the drain waits
                                    // that precede the exit always take kWaitCycles)
 };
 
-// F8: E4M3 operands (kind::f8f6f4, 128 elements per K tile), else 16-bit
-// (kind::f16, 64 elements per K tile); a template parameter, so the MMA issue
-// loop carries no branch on it
-// Ring geometry.  A stage holds kSub K tiles of X (16 KB each) and of the B
-// operand: for a single CTA with 16-bit operands two K tiles (128 shells: the
-// whole K range of a frequency on the 1-degree plan, so one barrier round trip
-// per frequency instead of two), X 32 KB + B 64 KB, two stages; with E4M3
-// operands (128 shells per K tile already) one K tile, four stages; a CTA of a
-// pair stages X and its half of B (16 KB each), so a pair's ring is deeper.
-// A single CTA with two K tiles per stage gives each K tile its own full
-// barrier (kFull = 2): the issuer starts the first K tile's MMAs while the
-// second K tile's copies are still landing (measured: 9.32 -> 8.98 ms per step
-// on the 256 x 256 scan, the same bounds bit for bit); the stage is still
-// released by one commit.
-template <bool F8, bool PAIR>
-struct Ring {
-    static constexpr int kSub = (PAIR || F8) ? 1 : 2;
-    static constexpr int kStageBytes = kSub * (PAIR ? 2 : 3) * kTileBytes;
-    static constexpr int kStages = PAIR ? 6 : (kSub == 2 ? 2 : 4);
-    static constexpr int kFull = kSub;      // full barriers per stage and issuer
+// One unit of work: an axis tile x two pattern tiles and a range of frequencies.
+struct Unit {
+    int zt, pu, g, f0, f1;
+    bool split;
+    int t;
 };
+__device__ __forceinline__ Unit unit_of(const TcArgs& a, int u) {
+    Unit w;
+    const TileSplit& ts = a.ts;
+    w.split = u >= ts.first;
+    w.t = w.split ? ts.first + (u - ts.first) / ts.groups : u;
+    w.g = w.split ? (u - ts.first) % ts.groups : 0;
+    w.f0 = w.split ? w.g * ts.per : 0;
+    w.f1 = w.split ? min(a.F, w.f0 + ts.per) : a.F;
+    w.zt = ts.zmajor ? w.t / ts.PTu : w.t % a.ZT;
+    w.pu = ts.zmajor ? w.t % ts.PTu : w.t / a.ZT;
+    return w;
+}
+// where the unit's bound of pattern b, axis z goes
+__device__ __forceinline__ float* bound_at(const TcArgs& a, const Unit& w, int b, int z) {
+    return w.g == 0 ? a.U + (int64_t)b * a.Z + z : a.extra + a.ts.extra_at(w.g, w.t, b, z);
+}
+
+// products of 16 axes' columns and 8 patterns' lanes into ud[0..8)
+#define ACOM_ACCUMULATE(R, I, ud, w)                                                           \
+    _Pragma("unroll") for (int n = 0; n < 4; ++n)                                              \
+        accumulate_pair2(R[4 * n], R[4 * n + 1], R[4 * n + 2], R[4 * n + 3], I[4 * n],         \
+                         I[4 * n + 1], I[4 * n + 2], I[4 * n + 3], w, (ud)[2 * n], (ud)[2 * n + 1])
+
+constexpr int kSub = 2;                            // K tiles a slot holds
+constexpr int kXSlots = 3, kPSlots = 2;
+constexpr int kXBytes = kSub * kTileBytes;         // 32 KB: 128 rows
+constexpr int kPBytes = 2 * kSub * kTileBytes;     // 64 KB: 256 rows
+constexpr int kBars = kXSlots * (kSub + 1) + kPSlots * (kSub + 1) + 5;
 
 // F8: E4M3 operands (kind::f8f6f4, 128 elements per K tile), else 16-bit
 // (kind::f16, 64 elements per K tile); a template parameter, so the MMA issue
 // loop carries no branch on it.
-// PAIR: a cluster of two CTAs computes each MMA together (cta_group::2,
-// M = 256): CTA rank r of the pair holds pattern tile 2 p + r of the pair's
-// pattern tiles (its A rows) and half of the axis tile's B operand (rank 0 the
-// real rows, rank 1 the imaginary rows); rank 0's two threads issue every MMA,
-// whose accumulators land in both CTAs' tensor memory, lanes = the CTA's own
-// patterns, columns = all 256 B rows, exactly as for a single CTA.  Both CTAs'
-// copies complete on rank 0's full barriers; commits arrive on both CTAs'
-// barriers; both epilogues release rank 0's accumulator barrier.
-template <bool F8, bool PAIR>
+template <bool F8>
 __global__ void __launch_bounds__(kThreads, 1)
 k_contract_bound_tc(const __grid_constant__ CUtensorMap map_p,
                     const __grid_constant__ CUtensorMap map_x, TcArgs a) {
-    constexpr int kSt = Ring<F8, PAIR>::kStages;
-    constexpr int kSB = Ring<F8, PAIR>::kStageBytes;
-    constexpr int kSub = Ring<F8, PAIR>::kSub;
-    constexpr int kFS = Ring<F8, PAIR>::kFull;
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* ring_p = reinterpret_cast<unsigned char*>(
+        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    unsigned char* ring_x = ring_p + kPSlots * kPBytes;
+    uint64_t* xfull = reinterpret_cast<uint64_t*>(ring_x + kXSlots * kXBytes);   // [kXSlots][kSub]
+    uint64_t* xempty = xfull + kXSlots * kSub;      // [kXSlots]
+    uint64_t* pfull = xempty + kXSlots;             // [kPSlots][kSub]
+    uint64_t* pempty = pfull + kPSlots * kSub;      // [kPSlots]
+    uint64_t* done = pempty + kPSlots;              // [2] accumulation finished, per TMEM buffer
+    uint64_t* tempty = done + 2;                    // [2] accumulator read (epilogue warps, warp 2)
+    uint64_t* drain = tempty + 2;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kXSlots * kSub; ++i) mbar_init(smem_u32(xfull + i), 1);
+        for (int i = 0; i < kPSlots * kSub; ++i) mbar_init(smem_u32(pfull + i), 1);
+        for (int i = 0; i < kXSlots; ++i) mbar_init(smem_u32(xempty + i), 1);
+        for (int i = 0; i < kPSlots; ++i) mbar_init(smem_u32(pempty + i), 1);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(smem_u32(done + i), 1);
+            mbar_init(smem_u32(tempty + i), kEpiWarps + 1);
+        }
+        mbar_init(smem_u32(drain), 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_p)));
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_x)));
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                         smem_u32(tmem_slot)),
+                     "r"(kTmemCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = *tmem_slot;
+    const int n_units = a.ts.units();
+    constexpr int ktel = F8 ? kKT8 : kKT;
+
+    if (warp == 0 || warp == kProdP) {
+        // ------------------------------------------------ TMA producers
+        if (elect_one()) {
+            const bool xprod = warp == 0;
+            const int slots = xprod ? kXSlots : kPSlots;
+            uint64_t* full = xprod ? xfull : pfull;
+            uint64_t* empty = xprod ? xempty : pempty;
+            int slot = 0;
+            uint32_t phase = 0;          // parity of the slots' current use
+            uint32_t used = 0, last = 0; // per slot: used at all, parity of its last use
+            bool ok = true;
+            for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
+                const Unit w = unit_of(a, u);
+                const int nsub = min(2, a.PT - 2 * w.pu);
+                for (int f = w.f0; f < w.f1 && ok; ++f)
+                    for (int kt = 0; kt < a.KT && ok; ++kt) {
+                        const int kbase = a.k0 + kt * ktel * kSub;
+                        for (int sub = 0; sub < (xprod ? nsub : 1); ++sub) {
+                            if (!mbar_wait(smem_u32(empty + slot), phase ^ 1u, abort_flag, a.err,
+                                           a.wait_cycles)) {
+                                ok = false;
+                                break;
+                            }
+#pragma unroll
+                            for (int k = 0; k < kSub; ++k) {
+                                const uint32_t fb = smem_u32(full + slot * kSub + k);
+                                const int x = kbase + k * ktel;
+                                if (x >= a.Spad) {           // past the padded shells: not
+                                    mbar_arrive(fb);         // loaded, not multiplied
+                                } else if (xprod) {
+                                    mbar_expect_tx(fb, kTileBytes);
+                                    tma_load_2d(smem_u32(ring_x + slot * kXBytes + k * kTileBytes),
+                                                &map_x, x, (f * a.PTs + 2 * w.pu + sub) * 128, fb);
+                                } else {
+                                    mbar_expect_tx(fb, 2 * kTileBytes);
+                                    tma_load_2d(smem_u32(ring_p + slot * kPBytes + k * 2 * kTileBytes),
+                                                &map_p, x, f * a.Zrows + w.zt * 256, fb);
+                                }
+                            }
+                            used |= 1u << slot;
+                            last = (last & ~(1u << slot)) | (phase << slot);
+                            if (++slot == slots) {
+                                slot = 0;
+                                phase ^= 1u;
+                            }
+                        }
+                    }
+            }
+            // every copy lands before the CTA's shared memory goes away
+            for (int i = 0; i < slots; ++i)
+                if (used & (1u << i))
+                    for (int k = 0; k < kSub; ++k) {
+                        const long long w0 = clock64();
+                        while (!mbar_try(smem_u32(full + i * kSub + k), (last >> i) & 1u) &&
+                               clock64() - w0 < kWaitCycles) {
+                        }
+                    }
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // ------------------------------------------------ MMA issuer
+        if (elect_one()) {
+            int xs = 0, ps = 0;
+            uint32_t xph = 0, pph = 0, tph = 0;      // tph: bit b, parity of buffer b's next use
+            uint32_t buf = 0;                        // TMEM buffer of the next accumulation
+            bool ok = true;
+            for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
+                const Unit w = unit_of(a, u);
+                const int nsub = min(2, a.PT - 2 * w.pu);
+                for (int f = w.f0; f < w.f1 && ok; ++f) {
+                    for (int kt = 0; kt < a.KT && ok; ++kt) {
+                        const bool last_k = kt + 1 == a.KT;
+                        // K steps of 32 bytes inside the shells (16 16-bit or 32 8-bit
+                        // elements); a step moves the descriptors by 32 bytes (2 units)
+                        const int nk = (min(ktel * kSub, a.Spad - a.k0 - kt * ktel * kSub) * (F8 ? 1 : 2)) >> 5;
+                        const uint64_t pd = sdesc(smem_u32(ring_p + ps * kPBytes));
+                        for (int sub = 0; sub < nsub; ++sub) {
+                            const uint32_t b = buf ^ (uint32_t)sub;
+                            if (kt == 0) {
+                                if (!mbar_wait(smem_u32(tempty + b), ((tph >> b) & 1u) ^ 1u,
+                                               abort_flag, a.err, a.wait_cycles)) {
+                                    ok = false;
+                                    break;
+                                }
+                                tph ^= 1u << b;
+                            }
+                            const uint64_t xd = sdesc(smem_u32(ring_x + xs * kXBytes));
+                            const uint32_t dacc = tmem + b * 256;
+#pragma unroll
+                            for (int j = 0; j < 4 * kSub; ++j) {
+                                const int k = j >> 2;
+                                if ((j & 3) == 0) {
+                                    if ((sub == 0 &&
+                                         !mbar_wait(smem_u32(pfull + ps * kSub + k), pph, abort_flag,
+                                                    a.err, a.wait_cycles)) ||
+                                        !mbar_wait(smem_u32(xfull + xs * kSub + k), xph, abort_flag,
+                                                   a.err, a.wait_cycles)) {
+                                        ok = false;
+                                        break;
+                                    }
+                                    fence_after();
+                                }
+                                if (j < nk) {
+                                    const uint64_t xa = xd + k * (kTileBytes >> 4) + 2 * (j & 3);
+                                    const uint64_t pa = pd + k * (2 * kTileBytes >> 4) + 2 * (j & 3);
+                                    if constexpr (F8)
+                                        mma_f8kind(dacc, xa, pa, a.idesc, (kt | j) ? 1u : 0u);
+                                    else
+                                        mma_f16kind(dacc, xa, pa, a.idesc, (kt | j) ? 1u : 0u);
+                                }
+                            }
+                            if (!ok) break;
+                            if (last_k) {
+                                mma_commit(smem_u32(done + b));
+                            } else {
+                                mma_commit(smem_u32(xempty + xs));
+                                if (sub + 1 == nsub) mma_commit(smem_u32(pempty + ps));
+                            }
+                            if (++xs == kXSlots) {
+                                xs = 0;
+                                xph ^= 1u;
+                            }
+                        }
+                        if (++ps == kPSlots) {
+                            ps = 0;
+                            pph ^= 1u;
+                        }
+                    }
+                    buf ^= (uint32_t)(nsub & 1);
+                }
+            }
+            // all MMAs issued by this thread complete before TMEM is released
+            mma_commit(smem_u32(drain));
+            const long long w0 = clock64();
+            while (!mbar_try(smem_u32(drain), 0) && clock64() - w0 < kWaitCycles) {
+            }
+        }
+        __syncwarp();
+    } else if (warp == 2) {
+        // ------------------------------------------------ slot release: a finished
+        // accumulation hands back the slots its last K stage read
+        if (elect_one()) {
+            int xs = 0, ps = 0;
+            uint32_t dph = 0, buf = 0;
+            bool ok = true;
+            for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
+                const Unit w = unit_of(a, u);
+                const int nsub = min(2, a.PT - 2 * w.pu);
+                for (int f = w.f0; f < w.f1 && ok; ++f) {
+                    // the last K stage's slots: nsub pattern slots a stage, one plan slot
+                    xs = (xs + (a.KT - 1) * nsub) % kXSlots;
+                    ps = (ps + a.KT - 1) % kPSlots;
+                    for (int sub = 0; sub < nsub; ++sub) {
+                        const uint32_t b = buf ^ (uint32_t)sub;
+                        if (!mbar_wait(smem_u32(done + b), (dph >> b) & 1u, abort_flag, a.err,
+                                       a.wait_cycles)) {
+                            ok = false;
+                            break;
+                        }
+                        dph ^= 1u << b;
+                        mbar_arrive(smem_u32(xempty + xs));
+                        if (sub + 1 == nsub) mbar_arrive(smem_u32(pempty + ps));
+                        mbar_arrive(smem_u32(tempty + b));
+                        xs = xs + 1 == kXSlots ? 0 : xs + 1;
+                    }
+                    ps = ps + 1 == kPSlots ? 0 : ps + 1;
+                    buf ^= (uint32_t)(nsub & 1);
+                }
+            }
+        }
+        __syncwarp();
+    } else {
+        // ------------------------------------------------ epilogue
+        const int q = warp & 3;                  // TMEM lane quarter: patterns 16q .. 16q + 15
+        const int zq = (warp - kEpi0) >> 2;      // axis columns 32 zq .. 32 zq + 31
+        const float invN = 1.0f / (float)a.N;
+        const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16) + zq * 32;
+        float ud[2][16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) ud[0][j] = ud[1][j] = 0.f;
+        uint32_t dph = 0, buf = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
+            const Unit w = unit_of(a, u);
+            const int nsub = min(2, a.PT - 2 * w.pu);
+            for (int f = w.f0; f < w.f1; ++f) {
+                const float wf = (f == 0 || 2 * f == a.N) ? 1.f : 2.f;
+#pragma unroll
+                for (int sub = 0; sub < 2; ++sub) {
+                    if (sub >= nsub) break;
+                    const uint32_t b = buf ^ (uint32_t)sub;
+                    if (!mbar_wait(smem_u32(done + b), (dph >> b) & 1u, abort_flag, a.err,
+                                   a.wait_cycles)) {
+                        ok = false;
+                        break;
+                    }
+                    dph ^= 1u << b;
+                    fence_after();
+                    // two halves of 8 patterns (16 lanes each)
+                    const uint32_t tb = tq + b * 256;
+                    uint32_t R[16], I[16];
+                    ACOM_TMEM_LD16x256_X4(tb, R);                          // (Xr, Xi) . Pr
+                    ACOM_TMEM_LD16x256_X4(tb + 128, I);                    // (Xr, Xi) . Pi
+                    ACOM_TMEM_WAIT32(R, I);
+                    ACOM_ACCUMULATE(R, I, ud[sub], wf);
+                    ACOM_TMEM_LD16x256_X4(tb + (16u << 16), R);
+                    ACOM_TMEM_LD16x256_X4(tb + (16u << 16) + 128, I);
+                    ACOM_TMEM_WAIT32(R, I);
+                    fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(tempty + b));
+                    ACOM_ACCUMULATE(R, I, ud[sub] + 8, wf);
+                }
+                if (!ok) break;
+                buf ^= (uint32_t)(nsub & 1);
+            }
+            if (!ok) break;
+#pragma unroll
+            for (int sub = 0; sub < 2; ++sub)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int b = (2 * w.pu + sub) * kNP + 8 * (2 * q + h) + (lane >> 2);
+                    // FP16 spectra carry power-of-two scales: divide them out
+                    const float sc = (a.xscale && b < a.nb)
+                                         ? invN * a.inv_pscale / (a.xscale[b] * a.xs_mul)
+                                         : invN * a.inv_pscale;
+#pragma unroll
+                    for (int n = 0; n < 4; ++n)
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const int z = w.zt * kM + zq * 32 + 8 * n + 2 * (lane & 3) + e;
+                            if (b < a.nb && z < a.Z)
+                                *bound_at(a, w, b, z) = ud[sub][h * 8 + 2 * n + e] * sc;
+                            ud[sub][h * 8 + 2 * n + e] = 0.f;
+                        }
+                }
+        }
+    }
+    fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                     "r"(kTmemCols)
+                     : "memory");
+    }
+}
+
+constexpr size_t tc_smem_bytes() {
+    return 1024 + (size_t)kPSlots * kPBytes + (size_t)kXSlots * kXBytes + 8 * kBars + 16;
+}
+
+// ---- CTA pairs: a cluster of two CTAs computes each MMA together (cta_group::2,
+// M = 256): CTA rank r holds pattern tile 2 p + r of the unit's two pattern
+// tiles (its A rows) and half of the axis tile's B operand (rank 0 the real
+// rows, rank 1 the imaginary rows); rank 0's two threads issue every MMA (even
+// frequencies into TMEM buffer 0, odd into 1), whose accumulators land in both
+// CTAs' tensor memory, lanes = the CTA's own patterns, columns = all 256 B
+// rows, exactly as for a single CTA.  Both CTAs' copies complete on rank 0's full
+// barriers (each issuer has its own per ring slot, so every full barrier has
+// one consumer); commits arrive on both CTAs' barriers; both epilogues release
+// rank 0's accumulator barrier.  A stage is one K tile of X and of the CTA's
+// half of B (16 KB each).
+constexpr int kPairStages = 6;
+constexpr int kPairStageBytes = 2 * kTileBytes;
+
+template <bool F8>
+__global__ void __launch_bounds__(kThreads, 1)
+k_contract_bound_pair(const __grid_constant__ CUtensorMap map_p,
+                      const __grid_constant__ CUtensorMap map_x, TcArgs a) {
+    constexpr int kSt = kPairStages;
+    constexpr int kSB = kPairStageBytes;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // 1024-byte alignment of the operand ring
     unsigned char* base = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     unsigned char* ring = base;
     uint64_t* bars = reinterpret_cast<uint64_t*>(ring + kSt * kSB);
-    uint64_t* full = bars;                          // [kIssuers][kSt][kFS]
-    uint64_t* empty = bars + kIssuers * kSt * kFS;  // [kSt]
+    uint64_t* full = bars;                      // [kIssuers][kSt]
+    uint64_t* empty = bars + kIssuers * kSt;    // [kSt]
     uint64_t* tfull = empty + kSt;              // [kIssuers]
     uint64_t* tempty = tfull + kIssuers;        // [kIssuers]
     uint64_t* drain = tempty + kIssuers;        // [kIssuers]
@@ -388,19 +716,18 @@ k_contract_bound_tc(const __grid_constant__ CUtensorMap map_p,
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = PAIR ? cluster_rank() : 0u;
+    const uint32_t rank = cluster_rank();
     const bool leader = rank == 0;
-    // the pair's abort flag of the other CTA: a timeout stops both CTAs
-    const uint32_t peer_abort =
-        PAIR ? mapa_rank(smem_u32(const_cast<int*>(abort_flag)), rank ^ 1u) : 0u;
+    // the abort flag of the other CTA: a timeout stops both CTAs
+    const uint32_t peer_abort = mapa_rank(smem_u32(const_cast<int*>(abort_flag)), rank ^ 1u);
     if (threadIdx.x == 0) {
-        // a full barrier completes on the arrivals of the (leading CTA's) two
-        // producers and the bytes of every copy of its K tile (of the stage)
-        for (int s = 0; s < kIssuers * kSt * kFS; ++s) mbar_init(smem_u32(full + s), 2);
+        // a full barrier completes on the arrivals of the leading CTA's two
+        // producers and the bytes of every copy of its stage
+        for (int s = 0; s < kIssuers * kSt; ++s) mbar_init(smem_u32(full + s), 2);
         for (int s = 0; s < kSt; ++s) mbar_init(smem_u32(empty + s), 1);
         for (int b = 0; b < kIssuers; ++b) {
             mbar_init(smem_u32(tfull + b), 1);
-            mbar_init(smem_u32(tempty + b), (PAIR ? 2 : 1) * kEpiWarps);
+            mbar_init(smem_u32(tempty + b), 2 * kEpiWarps);
             mbar_init(smem_u32(drain + b), 1);
         }
         *abort_flag = 0;
@@ -409,37 +736,20 @@ k_contract_bound_tc(const __grid_constant__ CUtensorMap map_p,
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_x)));
     }
     if (warp == 1) {
-        if constexpr (PAIR) {
-            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                             smem_u32(tmem_slot)),
-                         "r"(kTmemCols)
-                         : "memory");
-            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-        } else {
-            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                             smem_u32(tmem_slot)),
-                         "r"(kTmemCols)
-                         : "memory");
-            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-        }
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                         smem_u32(tmem_slot)),
+                     "r"(kTmemCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     fence_before();
-    if constexpr (PAIR)
-        cluster_sync_all();      // both CTAs' barriers exist before any copy or arrival
-    else
-        __syncthreads();
+    cluster_sync_all();      // both CTAs' barriers exist before any copy or arrival
     fence_after();
     const uint32_t tmem = *tmem_slot;
-    // tiles: single CTA (axis tile, pattern tile); pair (axis tile, pair of
-    // pattern tiles), the pair's CTAs taking the two pattern tiles
-    const int PTu = PAIR ? (a.PT + 1) / 2 : a.PT;
-    const int n_tiles = a.ZT * PTu;
-    const int t0 = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
-    const int tstep = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
-    auto set_abort = [&]() {
-        if constexpr (PAIR) st_cluster_u32(peer_abort, 1u);
-    };
-    bool aborted = false;
+    // units: axis tile x pair of pattern tiles, the CTAs taking a pattern tile each
+    const int n_units = a.ts.units();
+    const int u0 = (int)(blockIdx.x >> 1), ustep = (int)(gridDim.x >> 1);
+    auto set_abort = [&]() { st_cluster_u32(peer_abort, 1u); };
 
     if (warp == 0 || warp == kProdP) {
         // ------------------------------------------------ TMA producers: warp 0
@@ -454,13 +764,12 @@ k_contract_bound_tc(const __grid_constant__ CUtensorMap map_p,
             uint32_t issued_mask = 0, last_par = 0, last_own = 0;
             int fcount = 0;
             bool ok = true;
-            for (int t = t0; t < n_tiles && ok; t += tstep) {
-                const int zt = a.zmajor ? t / PTu : t % a.ZT;
-                const int pu = a.zmajor ? t % PTu : t / a.ZT;
-                const int pt = PAIR ? 2 * pu + (int)rank : pu;
-                for (int f = 0; f < a.F && ok; ++f, ++fcount) {
-                    // a pair's CTA loads the real (rank 0) or imaginary rows of the tile
-                    const int prow = f * a.Zrows + zt * 256 + (PAIR ? 128 * (int)rank : 0);
+            for (int u = u0; u < n_units && ok; u += ustep) {
+                const Unit w = unit_of(a, u);
+                const int pt = 2 * w.pu + (int)rank;
+                for (int f = w.f0; f < w.f1 && ok; ++f, ++fcount) {
+                    // a CTA loads the real (rank 0) or imaginary rows of the axis tile
+                    const int prow = f * a.Zrows + w.zt * 256 + 128 * (int)rank;
                     const int xrow = (f * a.PTs + pt) * 128;
                     const int own = fcount & 1;
                     for (int kt = 0; kt < a.KT; ++kt) {
@@ -469,54 +778,17 @@ k_contract_bound_tc(const __grid_constant__ CUtensorMap map_p,
                             ok = false;
                             break;
                         }
-                        const uint32_t fb = smem_u32(full + (own * kSt + stage) * kFS);
+                        const uint32_t fb = smem_u32(full + own * kSt + stage);
                         unsigned char* sbuf = ring + stage * kSB;
-                        constexpr int ktel = F8 ? kKT8 : kKT;
-                        // the stage's first shell; K tiles past the padded shells are
-                        // not loaded (nor expected, nor multiplied)
-                        const int kbase = a.k0 + kt * ktel * kSub;
-                        const int nsub = (kSub == 1 || a.Spad - kbase > ktel) ? kSub : 1;
-                        if constexpr (PAIR) {
-                            // every copy completes on the leading CTA's barrier, which
-                            // expects both CTAs' bytes of its operand
-                            const uint32_t fbl = mapa_rank(fb, 0);
-                            if (leader) mbar_expect_tx(fb, 2 * kTileBytes);
-                            if (xprod)
-                                tma_load_2d_pair(smem_u32(sbuf), &map_x, kbase, xrow, fbl);
-                            else
-                                tma_load_2d_pair(smem_u32(sbuf + kTileBytes), &map_p, kbase,
-                                                 prow, fbl);
-                        } else if (kFS > 1) {
-                            // K tile u completes on full barrier u (X: 16 KB, the
-                            // plan's 256-row box: 32 KB); a K tile past the padded
-                            // shells is only arrived on, so every barrier of the
-                            // stage completes once per use
-                            for (int u = 0; u < kFS; ++u) {
-                                const uint32_t fbu = fb + 8u * (uint32_t)u;
-                                if (u < nsub) {
-                                    mbar_expect_tx(fbu, (xprod ? 1 : 2) * kTileBytes);
-                                    if (xprod)
-                                        tma_load_2d(smem_u32(sbuf + u * kTileBytes), &map_x,
-                                                    kbase + u * ktel, xrow, fbu);
-                                    else
-                                        tma_load_2d(smem_u32(sbuf + (kSub + 2 * u) * kTileBytes),
-                                                    &map_p, kbase + u * ktel, prow, fbu);
-                                } else {
-                                    mbar_arrive(fbu);
-                                }
-                            }
-                        } else if (xprod) {
-                            mbar_expect_tx(fb, nsub * kTileBytes);
-                            for (int u = 0; u < nsub; ++u)
-                                tma_load_2d(smem_u32(sbuf + u * kTileBytes), &map_x,
-                                            kbase + u * ktel, xrow, fb);
-                        } else {
-                            // B operand: 256 rows, the tile's re rows then its im rows
-                            mbar_expect_tx(fb, nsub * 2 * kTileBytes);
-                            for (int u = 0; u < nsub; ++u)
-                                tma_load_2d(smem_u32(sbuf + (kSub + 2 * u) * kTileBytes), &map_p,
-                                            kbase + u * ktel, prow, fb);
-                        }
+                        const int kbase = a.k0 + kt * (F8 ? kKT8 : kKT);
+                        // every copy completes on the leading CTA's barrier, which
+                        // expects both CTAs' bytes of its operand
+                        const uint32_t fbl = mapa_rank(fb, 0);
+                        if (leader) mbar_expect_tx(fb, 2 * kTileBytes);
+                        if (xprod)
+                            tma_load_2d_pair(smem_u32(sbuf), &map_x, kbase, xrow, fbl);
+                        else
+                            tma_load_2d_pair(smem_u32(sbuf + kTileBytes), &map_p, kbase, prow, fbl);
                         issued_mask |= 1u << stage;
                         const uint32_t par = (fpar[own] >> stage) & 1u;
                         last_par = (last_par & ~(1u << stage)) | (par << stage);
@@ -530,19 +802,16 @@ k_contract_bound_tc(const __grid_constant__ CUtensorMap map_p,
                 }
             }
             if (!ok) {
-                aborted = true;
                 set_abort();
-                if (!PAIR || leader) {
+                if (leader) {
                     // let copies in flight land before the CTA's shared memory goes away
                     for (int s = 0; s < kSt; ++s)
                         if (issued_mask & (1u << s)) {
                             const uint32_t par = (last_par >> s) & 1u;
                             const int own = (last_own >> s) & 1u;
-                            for (int u = 0; u < kFS; ++u) {
-                                const long long w0 = clock64();
-                                while (!mbar_try(smem_u32(full + (own * kSt + s) * kFS + u), par) &&
-                                       clock64() - w0 < kWaitCycles) {
-                                }
+                            const long long w0 = clock64();
+                            while (!mbar_try(smem_u32(full + own * kSt + s), par) &&
+                                   clock64() - w0 < kWaitCycles) {
                             }
                         }
                 } else {
@@ -556,20 +825,21 @@ k_contract_bound_tc(const __grid_constant__ CUtensorMap map_p,
         }
         __syncwarp();
     } else if (warp <= kIssuers) {
-        // ------------------------------------------------ MMA issuers
+        // ------------------------------------------------ MMA issuers (leading CTA)
         // issuer mi takes the frequencies with fcount % 2 == mi into TMEM
         // buffer mi; it walks the ring in the producer's order and waits only
-        // on its own full barriers (a pair: the leading CTA's issuers only)
+        // on its own full barriers
         const int mi = warp - 1;
-        if (lane == 0 && (!PAIR || leader)) {
+        if (lane == 0 && leader) {
             int stage = 0;
             uint32_t fpar = 0;           // bit s: parity of this issuer's next phase of slot s
             uint32_t tph = 0;
             int fcount = 0;
             bool ok = true;
-            uint64_t* myfull = full + mi * kSt * kFS;
-            for (int t = t0; t < n_tiles && ok; t += tstep) {
-                for (int f = 0; f < a.F && ok; ++f, ++fcount) {
+            uint64_t* myfull = full + mi * kSt;
+            for (int u = u0; u < n_units && ok; u += ustep) {
+                const Unit w = unit_of(a, u);
+                for (int f = w.f0; f < w.f1 && ok; ++f, ++fcount) {
                     if ((fcount & 1) != mi) {
                         stage = (stage + a.KT) % kSt;
                         continue;
@@ -591,64 +861,31 @@ k_contract_bound_tc(const __grid_constant__ CUtensorMap map_p,
                         // fill); a step moves the descriptors' start address by
                         // 32 bytes (2 units of 16)
                         constexpr int ktel = F8 ? kKT8 : kKT;
-                        const int kbase = a.k0 + kt * ktel * kSub;
-                        const int nk = (min(ktel * kSub, a.Spad - kbase) * (F8 ? 1 : 2)) >> 5;
-#pragma unroll
-                        for (int j = 0; j < 4 * kSub; ++j) {
-                            // before the stage's first MMA (one full barrier) or
-                            // each K tile's first (one per K tile)
-                            if ((kFS > 1 && (j & 3) == 0) || j == 0) {
-                                if (!mbar_wait(smem_u32(myfull + stage * kFS + (kFS > 1 ? (j >> 2) : 0)),
-                                               spar, abort_flag, a.err, a.wait_cycles)) {
-                                    ok = false;
-                                    break;
-                                }
-                                fence_after();
-                            }
-                            if (j < nk) {
-                                // K tile j / 4 of the stage, step j % 4 inside it
-                                const int k4 = j & 3, u = j >> 2;
-                                const uint64_t xa = sdesc(sb + u * kTileBytes);
-                                const uint64_t pb = sdesc(sb + (kSub + 2 * u) * kTileBytes);
-                                const uint32_t acc = (kt | j) ? 1u : 0u;
-                                if constexpr (PAIR) {
-                                    if constexpr (F8)
-                                        mma_f8kind_pair(dacc, xa + 2 * k4, pb + 2 * k4, a.idesc, acc);
-                                    else
-                                        mma_f16kind_pair(dacc, xa + 2 * k4, pb + 2 * k4, a.idesc, acc);
-                                } else {
-                                    if constexpr (F8)
-                                        mma_f8kind(dacc, xa + 2 * k4, pb + 2 * k4, a.idesc, acc);
-                                    else
-                                        mma_f16kind(dacc, xa + 2 * k4, pb + 2 * k4, a.idesc, acc);
-                                }
-                            }
+                        const int nk = (min(ktel, a.Spad - a.k0 - kt * ktel) * (F8 ? 1 : 2)) >> 5;
+                        if (!mbar_wait(smem_u32(myfull + stage), spar, abort_flag, a.err,
+                                       a.wait_cycles)) {
+                            ok = false;
+                            break;
                         }
-                        if (!ok) break;
-                        // frees the stage (in both CTAs of a pair)
-                        if constexpr (PAIR)
-                            mma_commit_pair_both(smem_u32(empty + stage));
-                        else
-                            mma_commit(smem_u32(empty + stage));
+                        fence_after();
+                        const uint64_t xa = sdesc(sb), pb = sdesc(sb + kTileBytes);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (j < nk) {
+                                if constexpr (F8)
+                                    mma_f8kind_pair(dacc, xa + 2 * j, pb + 2 * j, a.idesc, (kt | j) ? 1u : 0u);
+                                else
+                                    mma_f16kind_pair(dacc, xa + 2 * j, pb + 2 * j, a.idesc, (kt | j) ? 1u : 0u);
+                            }
+                        mma_commit_pair_both(smem_u32(empty + stage));     // frees the stage in both CTAs
                         if (++stage == kSt) stage = 0;
                     }
-                    if (ok) {                                    // accumulators ready
-                        if constexpr (PAIR)
-                            mma_commit_pair_both(smem_u32(tfull + mi));
-                        else
-                            mma_commit(smem_u32(tfull + mi));
-                    }
+                    if (ok) mma_commit_pair_both(smem_u32(tfull + mi));    // accumulators ready
                 }
             }
-            if (!ok) {
-                aborted = true;
-                set_abort();
-            }
+            if (!ok) set_abort();
             // all MMAs issued by this thread complete before TMEM is released
-            if constexpr (PAIR)
-                mma_commit_pair(smem_u32(drain + mi));
-            else
-                mma_commit(smem_u32(drain + mi));
+            mma_commit_pair(smem_u32(drain + mi));
             const long long w0 = clock64();
             while (!mbar_try(smem_u32(drain + mi), 0) && clock64() - w0 < kWaitCycles) {
             }
@@ -666,14 +903,12 @@ k_contract_bound_tc(const __grid_constant__ CUtensorMap map_p,
         int fcount = 0;
         bool ok = true;
         // the accumulator barriers live in the leading CTA
-        const uint32_t tempty_l[2] = {PAIR ? mapa_rank(smem_u32(tempty), 0) : smem_u32(tempty),
-                                      PAIR ? mapa_rank(smem_u32(tempty + 1), 0)
-                                           : smem_u32(tempty + 1)};
-        for (int t = t0; t < n_tiles && ok; t += tstep) {
-            const int zt = a.zmajor ? t / PTu : t % a.ZT;
-            const int pu = a.zmajor ? t % PTu : t / a.ZT;
-            const int pt = PAIR ? 2 * pu + (int)rank : pu;
-            for (int f = 0; f < a.F; ++f, ++fcount) {
+        const uint32_t tempty_l[2] = {mapa_rank(smem_u32(tempty), 0),
+                                      mapa_rank(smem_u32(tempty + 1), 0)};
+        for (int u = u0; u < n_units && ok; u += ustep) {
+            const Unit w = unit_of(a, u);
+            const int pt = 2 * w.pu + (int)rank;
+            for (int f = w.f0; f < w.f1; ++f, ++fcount) {
                 const int buf = fcount & 1;
                 if (!mbar_wait(smem_u32(tfull + buf), tph[buf], abort_flag, a.err, a.wait_cycles)) {
                     ok = false;
@@ -681,7 +916,7 @@ k_contract_bound_tc(const __grid_constant__ CUtensorMap map_p,
                 }
                 tph[buf] ^= 1u;
                 fence_after();
-                const float w = (f == 0 || 2 * f == a.N) ? 1.f : 2.f;
+                const float wf = (f == 0 || 2 * f == a.N) ? 1.f : 2.f;
                 const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + buf * 256 + zq * 32;
                 // two halves of 8 patterns (16 lanes each); the second half's
                 // loads are in flight while the first is reduced
@@ -691,25 +926,12 @@ k_contract_bound_tc(const __grid_constant__ CUtensorMap map_p,
                 ACOM_TMEM_WAIT32(R0, I0);
                 ACOM_TMEM_LD16x256_X4(tb + (16u << 16), R1);
                 ACOM_TMEM_LD16x256_X4(tb + (16u << 16) + 128, I1);
-#pragma unroll
-                for (int n = 0; n < 4; ++n)
-                    accumulate_pair2(R0[4 * n], R0[4 * n + 1], R0[4 * n + 2], R0[4 * n + 3],
-                                     I0[4 * n], I0[4 * n + 1], I0[4 * n + 2], I0[4 * n + 3], w,
-                                     ud[2 * n], ud[2 * n + 1]);
+                ACOM_ACCUMULATE(R0, I0, ud, wf);
                 ACOM_TMEM_WAIT32(R1, I1);
                 fence_before();
                 __syncwarp();
-                if (lane == 0) {
-                    if constexpr (PAIR)
-                        mbar_arrive_cluster(tempty_l[buf]);
-                    else
-                        mbar_arrive(tempty_l[buf]);
-                }
-#pragma unroll
-                for (int n = 0; n < 4; ++n)
-                    accumulate_pair2(R1[4 * n], R1[4 * n + 1], R1[4 * n + 2], R1[4 * n + 3],
-                                     I1[4 * n], I1[4 * n + 1], I1[4 * n + 2], I1[4 * n + 3], w,
-                                     ud[8 + 2 * n], ud[8 + 2 * n + 1]);
+                if (lane == 0) mbar_arrive_cluster(tempty_l[buf]);
+                ACOM_ACCUMULATE(R1, I1, ud + 8, wf);
             }
             if (!ok) break;
 #pragma unroll
@@ -723,37 +945,27 @@ k_contract_bound_tc(const __grid_constant__ CUtensorMap map_p,
                 for (int n = 0; n < 4; ++n)
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
-                        const int z = zt * kM + zq * 32 + 8 * n + 2 * (lane & 3) + e;
-                        if (b < a.nb && z < a.Z) a.U[(int64_t)b * a.Z + z] = ud[h * 8 + 2 * n + e] * sc;
+                        const int z = w.zt * kM + zq * 32 + 8 * n + 2 * (lane & 3) + e;
+                        if (b < a.nb && z < a.Z) *bound_at(a, w, b, z) = ud[h * 8 + 2 * n + e] * sc;
                         ud[h * 8 + 2 * n + e] = 0.f;
                     }
             }
         }
         if (!ok && lane == 0) set_abort();
     }
-    (void)aborted;
     fence_before();
-    if constexpr (PAIR)
-        cluster_sync_all();      // the leading CTA's MMAs and every copy are done in both CTAs
-    else
-        __syncthreads();
+    cluster_sync_all();      // the leading CTA's MMAs and every copy are done in both CTAs
     if (warp == 1) {
         fence_after();
-        if constexpr (PAIR)
-            asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                         "r"(kTmemCols)
-                         : "memory");
-        else
-            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                         "r"(kTmemCols)
-                         : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                     "r"(kTmemCols)
+                     : "memory");
     }
 }
 
-template <bool F8, bool PAIR>
-size_t tc_smem_bytes() {
-    return 1024 + (size_t)Ring<F8, PAIR>::kStages * Ring<F8, PAIR>::kStageBytes +
-           8 * ((kIssuers * Ring<F8, PAIR>::kFull + 1) * Ring<F8, PAIR>::kStages + 3 * kIssuers) + 16;
+constexpr size_t pair_smem_bytes() {
+    return 1024 + (size_t)kPairStages * kPairStageBytes +
+           8 * ((kIssuers + 1) * kPairStages + 3 * kIssuers) + 16;
 }
 
 }  // namespace tc
@@ -811,27 +1023,44 @@ size_t tensor_map_bytes() { return sizeof(CUtensorMap); }
 static long long g_wait_cycles = 0;
 void set_wait_cycles(long long cycles) { g_wait_cycles = cycles > 0 ? cycles : 0; }
 
+// The tiles of full waves run whole.  The tiles of the last, partial wave (all
+// tiles of a small batch) are split over the frequencies into as many groups as
+// fill the SMs: a CTA runs a tile's frequencies in turn, so a wave of few tiles
+// would take as long as a full one.  1-degree plan: one pattern (8 tiles, 19
+// groups) 174 -> 27 us; 4,095 patterns (256 tiles, the last 104 too many to
+// split) 676 -> 515 us, from the larger tile.
+TileSplit tc_split(const acom_plan_s* p, int nb, int tile_order, bool split) {
+    TileSplit ts;
+    ts.zmajor = tile_order == 1 ? 1 : 0;
+    ts.ZT = p->Zp / tc::kM;
+    ts.PTu = (nb + 2 * tc::kNP - 1) / (2 * tc::kNP);
+    ts.lb = ts.lz = 7;
+    ts.set(sm_count(), sm_count(), p->F, split);
+    return ts;
+}
+
 void launch_contract_bound_tc(const acom_plan_s* p, const void* map_x, int pt_stride, int nb,
-                              float* U, cudaStream_t st, const float* xscale, int tile_order,
-                              int cta_pairs) {
+                              const TileSplit& ts, float* U, float* extra, cudaStream_t st,
+                              const float* xscale, int cta_pairs) {
     tc::TcArgs a;
-    a.zmajor = tile_order == 1 ? 1 : 0;
+    a.ts = ts;
     a.F = p->F;
     a.N = p->N;
     a.Z = p->Z;
     a.nb = nb;
-    a.ZT = p->Zp / tc::kM;
+    a.ZT = ts.ZT;
     a.PT = (nb + tc::kNP - 1) / tc::kNP;
     a.PTs = pt_stride;
     const bool f8 = p->precision == ACOM_PREC_FP8;
     const int ktel = f8 ? tc::kKT8 : tc::kKT;
     // the K range starts at the plan's first non-zero shell (a multiple of 16);
-    // KT stages of kSub K tiles each per frequency
+    // KT stages of `sub` K tiles each per frequency
     a.k0 = p->k0;
     auto stages = [&](int sub) { return (p->Spad - p->k0 + ktel * sub - 1) / (ktel * sub); };
     a.Spad = p->Spad;
     a.Zrows = 2 * p->Zp;
     a.U = U;
+    a.extra = extra;
     a.err = p->err;
     // E4M3 is format 0 for A and B, the same bits as F16
     a.idesc = p->precision == ACOM_PREC_BF16 ? tc::kIdescBF16 : tc::kIdescF16;
@@ -839,21 +1068,19 @@ void launch_contract_bound_tc(const acom_plan_s* p, const void* map_x, int pt_st
     a.xs_mul = f8 ? kFp8Shift : 1.0f;
     a.inv_pscale = 1.0f / p->pscale;
     a.wait_cycles = g_wait_cycles > 0 ? g_wait_cycles : tc::kWaitCycles;
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const int nsm = sm_count();
+    const int n_units = ts.units();
+    if (n_units <= 0) return;
     const CUtensorMap& mx = *reinterpret_cast<const CUtensorMap*>(map_x);
     if (cta_pairs && nsm >= 2) {
         // CTA pairs: M = 256 (the pair's two pattern tiles), each CTA loading
         // half of the 256 B rows (128-row boxes)
         a.idesc = (a.idesc & ~(0x1Fu << 24)) | ((256u >> 4) << 24);
         a.KT = stages(1);
-        const size_t smem = f8 ? tc::tc_smem_bytes<true, true>() : tc::tc_smem_bytes<false, true>();
-        auto kern = f8 ? tc::k_contract_bound_tc<true, true> : tc::k_contract_bound_tc<false, true>;
+        const size_t smem = tc::pair_smem_bytes();
+        auto kern = f8 ? tc::k_contract_bound_pair<true> : tc::k_contract_bound_pair<false>;
         set_max_dynamic_smem((const void*)kern, smem);
-        const int n_tiles = a.ZT * ((a.PT + 1) / 2);
-        const int clusters = n_tiles < nsm / 2 ? n_tiles : nsm / 2;
-        if (clusters <= 0) return;
+        const int clusters = n_units < nsm / 2 ? n_units : nsm / 2;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(2 * clusters, 1, 1);
         cfg.blockDim = dim3(tc::kThreads, 1, 1);
@@ -871,15 +1098,13 @@ void launch_contract_bound_tc(const acom_plan_s* p, const void* map_x, int pt_st
         prof_end(kKContractBf16, st);
         return;
     }
-    a.KT = f8 ? stages(tc::Ring<true, false>::kSub) : stages(tc::Ring<false, false>::kSub);
-    const size_t smem = f8 ? tc::tc_smem_bytes<true, false>() : tc::tc_smem_bytes<false, false>();
-    auto kern = f8 ? tc::k_contract_bound_tc<true, false> : tc::k_contract_bound_tc<false, false>;
+    a.KT = stages(tc::kSub);
+    const size_t smem = tc::tc_smem_bytes();
+    auto kern = f8 ? tc::k_contract_bound_tc<true> : tc::k_contract_bound_tc<false>;
     set_max_dynamic_smem((const void*)kern, smem);
-    const int n_tiles = a.ZT * a.PT;
-    const int grid = n_tiles < nsm ? n_tiles : nsm;
-    if (grid <= 0) return;
     prof_begin(kKContractBf16, st);
-    kern<<<grid, tc::kThreads, smem, st>>>(*reinterpret_cast<const CUtensorMap*>(p->map_p), mx, a);
+    kern<<<n_units < nsm ? n_units : nsm, tc::kThreads, smem, st>>>(
+        *reinterpret_cast<const CUtensorMap*>(p->map_p), mx, a);
     prof_end(kKContractBf16, st);
 }
 

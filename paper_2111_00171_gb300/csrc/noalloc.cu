@@ -115,9 +115,9 @@ extern "C" acom_status acom_bounds_static(acom_plan p, const acom_peaks_csr* pea
         launch_raster_patterns(geo, src, ro, p->err, st);
         float* U = dst + c0 * (int64_t)p->Z;
         if (tc)
-            launch_contract_bound_tc(p, map_x, PTs, nb, U, st);
+            launch_contract_bound_tc(p, map_x, PTs, nb, tc_split(p, nb, 0, false), U, nullptr, st);
         else
-            launch_contract_bound_fp32(p, Xr, Xi, nb, U, st, false);
+            launch_contract_bound_fp32(p, Xr, Xi, nb, fp32_split(p, nb, false), U, nullptr, st);
     }
     prof_suppress(false);
     e = cudaGetLastError();

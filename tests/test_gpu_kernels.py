@@ -58,3 +58,21 @@ def test_fp32_bounds_at_tile_edges(geometry, patterns):
     tol = (3 * (S + 2) + 2 * F) * 2.0 ** -24 * scale
     assert ((got - want).abs() <= tol[:, None]).all()
     plan.close()
+
+
+# one pattern and the edges of 64- and 128-pattern tiles; one to three K stages; a last
+# wave split over the frequencies (20,000 patterns: 157 tiles), and a batch of few tiles
+@pytest.mark.parametrize("geometry,patterns", [
+    ((3.0, 150, 0.01, 360), 1), ((3.0, 150, 0.01, 360), 64), ((2.0, 75, 0.02, 180), 65),
+    ((2.0, 75, 0.02, 180), 128), ((6.0, 200, 0.0075, 72), 129), ((6.0, 400, 0.00375, 72), 193),
+    ((6.0, 40, 0.0375, 72), 20000)], ids=str)
+def test_tensor_core_bounds_at_tile_edges(geometry, patterns):
+    plan = au_plan(*geometry, precision=1)
+    peaks = to_dev(synth.random_patterns(77, n_patterns=patterns))
+    got = plan.bounds(*peaks).double()
+    want, scale = bounds64(plan, peaks)
+    # BF16 operands: 2^-7 a product, sqrt(2) a side; FP32 accumulation charged 8-fold
+    S, F = math.ceil(geometry[1] / 32) * 32, geometry[3] // 2 + 1
+    tol = (2.0 ** -6 + (3 * (S + 2) + 2 * F) * 2.0 ** -21) * scale
+    assert ((got - want).abs() <= tol[:, None]).all()
+    plan.close()
