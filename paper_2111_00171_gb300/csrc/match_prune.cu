@@ -293,6 +293,7 @@ void launch_plan_fnorm_max(const acom_plan_s* p, float* out, cudaStream_t st) {
 constexpr int kSelThreads = 256;
 constexpr int kSelWarps = kSelThreads / 32;
 constexpr int kBatch = 8;
+constexpr int kOrderCap = 512;          // pending axes sorted once per pattern
 
 struct SelState {
     float T;             // best exact score so far
@@ -303,6 +304,7 @@ struct SelState {
                          // its own: thread 0 fills it right after the main loop's
                          // last barrier, while slower threads may still read nc)
     int q;               // next neighbour to consider (refinement batches)
+    int n_order, at;     // pending axes counted, the next of `order` to consider
     float best3[3];      // winning correlation at bins k - 1, k, k + 1
     float Emax;          // rounding margin of the bounds
     float next_u;        // bound of the best pending axis after a batch's picks
@@ -319,6 +321,7 @@ struct SelSmem {
     float* U;        // [Z] bound, replaced by the exact score once evaluated
     uint8_t* ev;     // [Z] 0 pending, 1 evaluated, 2 in the current batch
     uint16_t* kb;    // [Z] bin + mirror * N of each evaluated axis' maximum
+    uint16_t* order; // [kOrderCap] pending axes in decreasing bound (search_order)
     float* wv;       // [kSelWarps][kBatch] per-warp top-K values
     int* wi;         // [kSelWarps][kBatch] and axes
     int* cand;       // [kBatch]
@@ -359,20 +362,26 @@ __device__ inline void warp_argmax(float& v, unsigned& i) {
     }
 }
 
+// Argmax over the warp of bounds (not negative, so their bit patterns order like
+// their values; -1 marks none), ties to the lowest axis: two warp reductions.
+__device__ __forceinline__ void warp_argmax_bound(float& v, unsigned& i) {
+    const unsigned key = v >= 0.f ? __float_as_uint(v) + 1u : 0u;
+    const unsigned m = __reduce_max_sync(0xffffffffu, key);
+    i = __reduce_min_sync(0xffffffffu, m != 0u && key == m ? i : 0xffffffffu);
+    v = m ? __uint_as_float(m - 1u) : -CUDART_INF_F;
+}
+
 // The up to K pending axes (ev == 0) of largest bound with U rel + Emax >= thr
 // (with per_phase, thr is the best score so far of the axis' own phase), in
 // decreasing bound (ties: lowest axis), into cand and st->nc; marks them
 // ev = 2.  Each warp takes its K best by repeated argmax over entries strictly
 // below its previous pick; warp 0 merges the warps' lists the same way.
 __device__ void block_topk(SelSmem& sm, int Z, int K, float thr, float rel, float Emax,
-                           bool per_phase, int nph, bool want_next = false) {
-    // with want_next, one more round finds the best pending axis after the K
-    // picks (K < kBatch): its bound goes to st->next_u (-inf: none), unpicked
-    const int Kr = K + (want_next ? 1 : 0);
+                           bool per_phase, int nph) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float lv = CUDART_INF_F;
     unsigned li = 0u;                       // previous pick (nothing is above it)
-    for (int r = 0; r < Kr; ++r) {
+    for (int r = 0; r < K; ++r) {
         float v = -CUDART_INF_F;
         unsigned zi = 0xffffffffu;
         for (int z = warp * 32 + lane; z < Z; z += kSelThreads) {
@@ -391,7 +400,7 @@ __device__ void block_topk(SelSmem& sm, int Z, int K, float thr, float rel, floa
             sm.wi[warp * kBatch + r] = (int)zi;
         }
         if (zi == 0xffffffffu) {
-            for (int r2 = r + 1 + lane; r2 < Kr; r2 += 32) sm.wi[warp * kBatch + r2] = -1;
+            for (int r2 = r + 1 + lane; r2 < K; r2 += 32) sm.wi[warp * kBatch + r2] = -1;
             break;
         }
         lv = v;
@@ -399,16 +408,15 @@ __device__ void block_topk(SelSmem& sm, int Z, int K, float thr, float rel, floa
     }
     __syncthreads();
     if (warp == 0) {
-        const int ne = kSelWarps * Kr;
+        const int ne = kSelWarps * K;
         lv = CUDART_INF_F;
         li = 0u;
         int n = 0;
-        float next = -CUDART_INF_F;
-        for (int r = 0; r < Kr; ++r) {
+        for (int r = 0; r < K; ++r) {
             float v = -CUDART_INF_F;
             unsigned zi = 0xffffffffu;
             for (int e = lane; e < ne; e += 32) {
-                const int w = e / Kr, j = e - w * Kr;
+                const int w = e / K, j = e - w * K;
                 const int z = sm.wi[w * kBatch + j];
                 if (z < 0) continue;
                 const float u = sm.wv[w * kBatch + j];
@@ -419,10 +427,6 @@ __device__ void block_topk(SelSmem& sm, int Z, int K, float thr, float rel, floa
             }
             warp_argmax(v, zi);
             if (zi == 0xffffffffu) break;
-            if (r == K) {                    // the best axis after the picks
-                next = v;
-                break;
-            }
             if (lane == 0) {
                 sm.cand[n] = (int)zi;
                 sm.ev[zi] = 2;
@@ -433,7 +437,6 @@ __device__ void block_topk(SelSmem& sm, int Z, int K, float thr, float rel, floa
         }
         if (lane == 0) {
             sm.st->nc = n;
-            sm.st->next_u = next;
         }
     }
     __syncthreads();
@@ -499,20 +502,12 @@ __device__ void batch_spectra(const SelectArgs& a, int64_t b, int nc, int s_lo, 
         for (int c = warp; c < nc; c += kSelWarps) {
             const uint32_t* pm = a.smask + (int64_t)sm.cand[c] * MW;
             const uint32_t m = lane < MW ? (sm.pmask[lane] & pm[lane]) : 0u;
-            const int cnt = __popc(m);
-            int off = cnt;                              // inclusive scan over the lanes
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(0xffffffffu, off, o);
-                if (lane >= o) off += v;
-            }
-            const int tot = __shfl_sync(0xffffffffu, off, 31);
-            off -= cnt;
             uint16_t* L = sm.slist + c * a.Spad;
-            uint32_t mm = m;
-            while (mm) {
-                const int bit = __ffs(mm) - 1;
-                mm &= mm - 1;
-                L[off++] = (uint16_t)(32 * lane + bit);
+            int tot = 0;
+            for (int w = 0; w < MW; ++w) {
+                const uint32_t mw = __shfl_sync(0xffffffffu, m, w);
+                if (mw >> lane & 1u) L[tot + __popc(mw & ((1u << lane) - 1u))] = (uint16_t)(32 * w + lane);
+                tot += __popc(mw);
             }
             if (lane == 0) sm.slen[c] = tot;
         }
@@ -651,31 +646,132 @@ __device__ void batch_transforms(const SelectArgs& a, int nc, SelSmem& sm) {
 }
 
 // Record the batch's exact scores; with update, fold them into the best.
-// Every score also updates its phase's best.
+// Every score also updates its phase's best.  Lane c of warp 0 takes candidate c.
 __device__ void fold_batch(int nc, int N, bool update, int nph, SelSmem& sm) {
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32) {
+        const int c = threadIdx.x;
         SelState& st = *sm.st;
-        for (int c = 0; c < nc; ++c) {
+        float bv = -CUDART_INF_F;
+        unsigned gidx = 0xffffffffu, bi = 0;
+        int ph = -1;
+        if (c < nc) {
             const int z = sm.cand[c];
-            const float* r = sm.res + 5 * c;
-            const float bv = r[0];
-            float& tp = st.Tp[phase_of(sm.poff, nph, z)];
-            tp = bv > tp ? bv : tp;
-            const unsigned bi = __float_as_uint(r[1]);
-            const unsigned gidx = (unsigned)z * 2u * (unsigned)N + bi;
-            if (update && better(bv, gidx, st.T, st.Tidx)) {
-                st.T = bv;
-                st.Tidx = gidx;
-                st.bz = z;
-                st.bm = (int)(bi / (unsigned)N);
-                st.bk = (int)(bi - (unsigned)st.bm * N);
-                st.best3[0] = r[2];
-                st.best3[1] = r[3];
-                st.best3[2] = r[4];
-            }
+            bv = sm.res[5 * c];
+            bi = __float_as_uint(sm.res[5 * c + 1]);
+            gidx = (unsigned)z * 2u * (unsigned)N + bi;
+            ph = phase_of(sm.poff, nph, z);
             sm.U[z] = bv;
             sm.kb[z] = (uint16_t)bi;
             sm.ev[z] = 1;
+        }
+        for (int p = 0; p < nph; ++p) {
+            float v = ph == p ? bv : -CUDART_INF_F;
+            for (int o = kBatch / 2; o > 0; o >>= 1)
+                v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+            if (c == 0 && v > st.Tp[p]) st.Tp[p] = v;
+        }
+        if (update) {
+            float tv = bv;
+            unsigned ti = gidx;
+            for (int o = kBatch / 2; o > 0; o >>= 1) {
+                const float ov = __shfl_xor_sync(0xffffffffu, tv, o);
+                const unsigned oi = __shfl_xor_sync(0xffffffffu, ti, o);
+                if (better(ov, oi, tv, ti)) {
+                    tv = ov;
+                    ti = oi;
+                }
+            }
+            if (c < nc && ti == gidx && better(bv, gidx, st.T, st.Tidx)) {
+                st.T = bv;
+                st.Tidx = gidx;
+                st.bz = sm.cand[c];
+                st.bm = (int)(bi / (unsigned)N);
+                st.bk = (int)(bi - (unsigned)st.bm * N);
+                st.best3[0] = sm.res[5 * c + 2];
+                st.best3[1] = sm.res[5 * c + 3];
+                st.best3[2] = sm.res[5 * c + 4];
+            }
+        }
+    }
+    __syncthreads();
+}
+
+// The bound an axis must reach to be evaluated: the best score so far, of its own
+// phase when every phase is certified.
+__device__ __forceinline__ float search_threshold(const SelSmem& sm, bool per_phase, int nph, int z) {
+    return per_phase ? sm.st->Tp[phase_of(sm.poff, nph, z)] : sm.st->T;
+}
+
+// After the first batch: the pending axes whose bound can reach their threshold, in
+// decreasing bound (ties: lowest axis), into `order`.  The thresholds only rise, so
+// no other axis becomes pending and the later batches take the list in turn: one
+// scan of the axes a pattern instead of kBatch a batch (phases workload, 2,001
+// axes and 17 batches a pattern: 33,000 of a batch's 66,000 cycles).  More than
+// kOrderCap axes: -1, the batch scans (block_topk) and the next tries again.  Returns
+// the length, the same in every thread.
+__device__ int search_order(SelSmem& sm, int Z, float rel, float Emax, bool per_phase, int nph) {
+    float* lu = reinterpret_cast<float*>(sm.part);                    // not in use here
+    uint16_t* lz = reinterpret_cast<uint16_t*>(lu + kOrderCap);
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) sm.st->n_order = 0;
+    __syncthreads();
+    for (int z0 = threadIdx.x - lane; z0 < Z; z0 += kSelThreads) {
+        const int z = z0 + lane;
+        const float u = z < Z ? sm.U[z] : 0.f;
+        const bool in = z < Z && sm.ev[z] == 0 && u == u &&
+                        !(u * rel + Emax < search_threshold(sm, per_phase, nph, z));
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        if (m == 0u) continue;
+        int base = 0;
+        if (lane == 0) base = atomicAdd(&sm.st->n_order, __popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0) + __popc(m & ((1u << lane) - 1u));
+        if (in && base < kOrderCap) {
+            lu[base] = u;
+            lz[base] = (uint16_t)z;
+        }
+    }
+    __syncthreads();
+    const int n = sm.st->n_order;
+    __syncthreads();
+    if (n > kOrderCap) return -1;
+    for (int i = threadIdx.x; i < n; i += kSelThreads) {
+        const float u = lu[i];
+        const unsigned z = lz[i];
+        int rank = 0;
+        for (int j = 0; j < n; ++j) rank += better(lu[j], lz[j], u, z) ? 1 : 0;
+        sm.order[rank] = (uint16_t)z;
+    }
+    if (threadIdx.x == 0) sm.st->at = 0;
+    __syncthreads();
+    return n;
+}
+
+// The next up to K axes of `order` that can still reach their threshold, into cand
+// and st->nc; marks them ev = 2.  The first K of the list in order are the K
+// largest bounds still pending.
+__device__ void next_in_order(SelSmem& sm, int n, int K, float rel, float Emax, bool per_phase,
+                              int nph) {
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        int at = sm.st->at, nc = 0;
+        while (at < n && nc < K) {
+            const int z = at + lane < n ? sm.order[at + lane] : -1;
+            const bool in = z >= 0 &&
+                            !(sm.U[z] * rel + Emax < search_threshold(sm, per_phase, nph, z));
+            const unsigned m = __ballot_sync(0xffffffffu, in);
+            const int r = nc + __popc(m & ((1u << lane) - 1u));
+            if (in && r < K) {
+                sm.cand[r] = z;
+                sm.ev[z] = 2;
+            }
+            // past the K-th taken entry, or the whole group
+            const unsigned kth = __ballot_sync(0xffffffffu, in && r == K - 1);
+            nc = min(K, nc + __popc(m));
+            at += kth ? __ffs(kth) : 32;
+        }
+        if (lane == 0) {
+            sm.st->at = at;
+            sm.st->nc = nc;
         }
     }
     __syncthreads();
@@ -888,6 +984,7 @@ __global__ void __launch_bounds__(kSelThreads, 3) k_select_exact(SelectArgs a) {
     sm.st = reinterpret_cast<SelState*>(take(sizeof(SelState)));
     sm.ev = take(Z);
     sm.kb = reinterpret_cast<uint16_t*>(take(sizeof(uint16_t) * Z));
+    sm.order = reinterpret_cast<uint16_t*>(take(sizeof(uint16_t) * kOrderCap));
     const int nph = a.n_phases;
     for (int i = threadIdx.x; i <= nph; i += kSelThreads) sm.poff[i] = a.phase_off[i];
     // with per-phase scores requested, every phase's best is certified
@@ -909,9 +1006,27 @@ __global__ void __launch_bounds__(kSelThreads, 3) k_select_exact(SelectArgs a) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
     for (int64_t b = blockIdx.x; b < a.nb; b += gridDim.x) {
+        // the bounds, and the three largest of each lane's (ties: lowest axis) for
+        // the first batch
+        float tv[3] = {-1.f, -1.f, -1.f};
+        unsigned tz[3] = {0xffffffffu, 0xffffffffu, 0xffffffffu};
         for (int z = threadIdx.x; z < Z; z += kSelThreads) {
-            sm.U[z] = later_groups(a.ts, a.extra, (int)b, z, a.U[b * Z + z]);
+            const float u = later_groups(a.ts, a.extra, (int)b, z, a.U[b * Z + z]);
+            sm.U[z] = u;
             sm.ev[z] = 0;
+            if (u > tv[2]) {
+                const bool b1 = u > tv[1], b0 = u > tv[0];
+                tv[2] = b1 ? tv[1] : u;
+                tz[2] = b1 ? tz[1] : (unsigned)z;
+                if (b1) {
+                    tv[1] = b0 ? tv[0] : u;
+                    tz[1] = b0 ? tz[0] : (unsigned)z;
+                }
+                if (b0) {
+                    tv[0] = u;
+                    tz[0] = (unsigned)z;
+                }
+            }
         }
         // the shells some peak's tent reached (recorded by the raster, which
         // wrote only those rows; every other row of the pattern is zero)
@@ -941,7 +1056,52 @@ __global__ void __launch_bounds__(kSelThreads, 3) k_select_exact(SelectArgs a) {
             sm.red[warp] = e;
             sm.red[kSelWarps + warp] = ea;
         }
+        for (int r = 0; r < 3; ++r) {
+            float v = tv[0];
+            unsigned zi = tz[0];
+            warp_argmax_bound(v, zi);
+            if (lane == 0) {
+                sm.wv[warp * kBatch + r] = v;
+                sm.wi[warp * kBatch + r] = (int)zi;
+            }
+            if (tz[0] == zi) {               // this lane's: on to its next (none left: -1)
+                tv[0] = tv[1];
+                tz[0] = tz[1];
+                tv[1] = tv[2];
+                tz[1] = tz[2];
+                tv[2] = -1.f;
+                tz[2] = 0xffffffffu;
+            }
+        }
         __syncthreads();
+        if (warp == 1) {
+            // the block's two largest bounds are the first batch; the third's bound
+            // tells whether a second one can follow
+            float v = -1.f;
+            unsigned zi = 0xffffffffu;
+            if (lane < 3 * kSelWarps) {
+                v = sm.wv[(lane / 3) * kBatch + lane % 3];
+                zi = (unsigned)sm.wi[(lane / 3) * kBatch + lane % 3];
+            }
+            int n = 0;
+            for (int r = 0; r < 3; ++r) {
+                float bv = v;
+                unsigned bz = zi;
+                warp_argmax_bound(bv, bz);
+                if (lane == 0) {
+                    if (r == 2) sm.st->next_u = bv;
+                    else if (bz != 0xffffffffu && rescore_top == 0) {
+                        sm.cand[n++] = (int)bz;
+                        sm.ev[bz] = 2;
+                    }
+                }
+                if (zi == bz) {
+                    v = -1.f;
+                    zi = 0xffffffffu;
+                }
+            }
+            if (lane == 0) sm.st->nc = n;
+        }
         if (threadIdx.x == 0) {
             float t = 0.f, ta = 0.f;
             for (int w = 0; w < kSelWarps; ++w) {
@@ -973,23 +1133,27 @@ __global__ void __launch_bounds__(kSelThreads, 3) k_select_exact(SelectArgs a) {
         //    winner.
         const bool single = !per_phase && rescore_top == 0;
         const bool want_ru = FULL && (a.out.runner_za || a.out.runner_score || a.out.runner_orient);
-        int stage = 0, batch = 0;
+        int stage = 0, batch = 0, n_order = -1;     // n_order: axes in `order` (-1: not sorted)
         for (;;) {
             int nc = 0;
             bool update = false;
             if (stage == 0) {
-                const int left = rescore_top - evals;
-                if (rescore_top == 0 || left > 0) {
-                    const float thr =
-                        (batch == 0 || rescore_top > 0) ? -CUDART_INF_F : sm.st->T;
-                    const int K = rescore_top > 0 ? (left < kBatch ? left : kBatch)
-                                                  : (batch == 0 ? 2 : kBatch);
-                    // the first batch also finds the best bound after its picks:
-                    // when that cannot reach the batch's best score, no later batch
-                    // would find a candidate and the search ends without a scan
-                    block_topk(sm, Z, K, thr, rel, Emax,
-                               per_phase && batch > 0 && rescore_top == 0, nph,
-                               single && batch == 0);
+                if (rescore_top > 0) {
+                    const int left = rescore_top - evals;
+                    if (left > 0) {
+                        block_topk(sm, Z, left < kBatch ? left : kBatch, -CUDART_INF_F, rel, Emax,
+                                   false, nph);
+                        nc = sm.st->nc;
+                    }
+                } else {
+                    // the first batch (two largest bounds) was picked as they loaded
+                    if (batch > 0) {
+                        if (n_order < 0) n_order = search_order(sm, Z, rel, Emax, per_phase, nph);
+                        if (n_order >= 0)
+                            next_in_order(sm, n_order, kBatch, rel, Emax, per_phase, nph);
+                        else
+                            block_topk(sm, Z, kBatch, sm.st->T, rel, Emax, per_phase, nph);
+                    }
                     nc = sm.st->nc;
                 }
                 update = true;
@@ -1137,7 +1301,8 @@ size_t select_smem_bytes(int Z, int N, int F, int Spad) {
            r16(sizeof(uint32_t) * (Spad >> 5)) + r16(sizeof(uint16_t) * kBatch * Spad) +
            r16(sizeof(int) * kBatch) +
            (N == 360 ? 2 * r16(sizeof(uint16_t) * 360) : 0) +
-           r16(sizeof(SelState)) + r16(Z) + r16(sizeof(uint16_t) * Z);
+           r16(sizeof(SelState)) + r16(Z) + r16(sizeof(uint16_t) * Z) +
+           r16(sizeof(uint16_t) * kOrderCap);
 }
 
 void launch_select_exact(const acom_plan_s* p, const float* Xsr, const float* Xsi, const float* U,
