@@ -110,11 +110,12 @@ inline float fp16_plan_scale(int N) {
 
 // What the select kernel hands the orientation kernel for one pattern: the
 // winner (axis z, bin + mirror * N), the correlation at bins k - 1, k, k + 1
-// and the score-weighted sum of the neighbour axes within 0.9 of the best.
+// and the number of neighbour axes within 0.9 of the best (or their
+// score-weighted sum).
 struct OrientIn {
     double w[3];
     float c3[3];
-    int z, km, pad;
+    int z, km, n;                  // n: neighbours handed on in onbr (-1: summed in w)
 };
 
 // Workspace for one chunk of patterns.
@@ -132,7 +133,7 @@ struct Workspace {
     int PTs = 0;                   // pattern tiles of 64 in XB
     alignas(64) unsigned char map_x[128];   // TMA map of XB
     float* xfn = nullptr;          // [chunk][F] ||X^_bf|| over shells
-    int* n_eval = nullptr;         // axes evaluated exactly in the last match
+    int* n_eval = nullptr;         // [2] axes evaluated exactly in the last match, patterns taken
     int2* srange = nullptr;        // [chunk] non-zero shell range of each pattern
     uint32_t* rmask = nullptr;     // [chunk][Spad / 32] shells each pattern's tents reach
     unsigned long long* best = nullptr;  // [chunk] packed (score, index)
@@ -140,6 +141,7 @@ struct Workspace {
     float* xscale = nullptr;       // [chunk] 2^e of each pattern's FP16 spectrum
     void* XB8 = nullptr;           // E4M3 copy of XB (FP8 plans)
     OrientIn* oin = nullptr;       // [chunk] winners for the orientation kernel
+    float2* onbr = nullptr;        // [chunk][32] their neighbours' (score, axis)
     size_t bytes = 0;
 };
 
@@ -342,14 +344,17 @@ void launch_contract_bound_tc(const acom_plan_s* p, const void* map_x, int pt_st
 // BF16 of P^ (kind 0), FP16 (1) or E4M3 (2) of scale * P^
 void launch_plan_to_operand(const float* Pr, const float* Pi, int Zp, int F, int Spad, void* dst,
                             cudaStream_t st, int kind, float scale);
-void launch_orient_compose(const acom_plan_s* p, const OrientIn* oin, int nb, int refine,
+void launch_orient_compose(const acom_plan_s* p, const OrientIn* oin, const float2* onbr, int nb,
+                           int refine,
                            acom_result out, int64_t off, cudaStream_t st);
-// U: bounds, `extra` the later groups' of split tiles (TileSplit)
+// U: bounds, `extra` the later groups' of split tiles (TileSplit); n_eval: axes
+// evaluated and patterns taken so far, *taken the latter on the host
 void launch_select_exact(const acom_plan_s* p, const float* Xsr, const float* Xsi, const float* U,
                          const float* extra, const TileSplit& ts, const float* xfn, const int2* srange, const uint32_t* rmask,
                          const float* pfmax, const float* xnorm2, int nb,
                          float kappa, int refine, acom_result out, int64_t off, int* n_eval,
-                         cudaStream_t st, const float* xscale, int rescore_top, OrientIn* oin);
+                         cudaStream_t st, const float* xscale, int rescore_top, OrientIn* oin,
+                         float2* onbr, int* taken);
 // refine.cu: continuous refinement on the plan's reflections
 acom_status refine_table(acom_plan_s* p, cudaStream_t st);
 void launch_refine_orient(const acom_plan_s* p, const acom_peaks_csr* pk, int steps,

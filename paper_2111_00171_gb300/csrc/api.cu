@@ -159,6 +159,7 @@ static void free_workspace(Workspace& ws, cudaStream_t st) {
     pool_free(ws.xscale, st);
     pool_free(ws.XB8, st);
     pool_free(ws.oin, st);
+    pool_free(ws.onbr, st);
     ws = Workspace{};
 }
 
@@ -191,12 +192,13 @@ static acom_status ensure_ws(acom_plan_s* p, Workspace& ws, int chunk, bool need
     if ((e = dalloc(&ws.U, (size_t)chunk * p->Z, &acc, st)) != cudaSuccess) goto fail;
     if ((e = dalloc(&ws.extra, split_extra_floats(), &acc, st)) != cudaSuccess) goto fail;
     if ((e = dalloc(&ws.xfn, (size_t)chunk * p->F, &acc, st)) != cudaSuccess) goto fail;
-    if ((e = dalloc(&ws.n_eval, (size_t)1, &acc, st)) != cudaSuccess) goto fail;
+    if ((e = dalloc(&ws.n_eval, (size_t)2, &acc, st)) != cudaSuccess) goto fail;
     if ((e = dalloc(&ws.srange, (size_t)chunk, &acc, st)) != cudaSuccess) goto fail;
     if ((e = dalloc(&ws.rmask, (size_t)chunk * (p->Spad / 32), &acc, st)) != cudaSuccess) goto fail;
     if ((e = dalloc(&ws.best, (size_t)chunk, &acc, st)) != cudaSuccess) goto fail;
     if ((e = dalloc(&ws.za_scores, (size_t)chunk * p->Z, &acc, st)) != cudaSuccess) goto fail;
     if ((e = dalloc(&ws.oin, (size_t)chunk, &acc, st)) != cudaSuccess) goto fail;
+    if ((e = dalloc(&ws.onbr, (size_t)chunk * 32, &acc, st)) != cudaSuccess) goto fail;
     if (tc_precision(p->precision)) {
         // the raster writes BF16, or FP16 with a per-pattern scale; E4M3
         // operands are converted from the FP16 rows
@@ -821,7 +823,8 @@ static acom_status match_enqueue(acom_plan p, const acom_peaks_csr* peaks,
     s = ensure_workspace(p, chunk, exhaustive, fp32_contraction, st);
     if (s != ACOM_OK) return s;
     cudaMemsetAsync(p->err, 0, sizeof(int), st);
-    cudaMemsetAsync(p->ws.n_eval, 0, sizeof(int), st);
+    cudaMemsetAsync(p->ws.n_eval, 0, 2 * sizeof(int), st);
+    int taken = 0;
     launch_check_row0(peaks->row_ptr, p->err, st);
     RasterGeom geo{p->S, p->Spad, p->N, p->F, (float)p->dq, (float)p->delta, (float)p->gamma_pow, 0};
     const int wchunk = p->ws.chunk;
@@ -866,9 +869,10 @@ static acom_status match_enqueue(acom_plan p, const acom_peaks_csr* peaks,
             }
             launch_select_exact(p, w.Xsr, w.Xsi, w.U, w.extra, ts, w.xfn, w.srange, w.rmask, p->pfmax,
                                 w.xnorm2, nb, tc ? kappa_tc(p) : kappa_fp32(p), refine, *out,
-                                c0, w.n_eval, st, xscale, rescore_top, w.oin);
+                                c0, w.n_eval, st, xscale, rescore_top, w.oin, w.onbr,
+                                &taken);
             if (out->phi3 || out->orient)
-                launch_orient_compose(p, w.oin, nb, refine, *out, c0, st);
+                launch_orient_compose(p, w.oin, w.onbr, nb, refine, *out, c0, st);
         }
     }
     cudaError_t e = cudaGetLastError();

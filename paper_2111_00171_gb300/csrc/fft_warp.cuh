@@ -245,44 +245,53 @@ __device__ __forceinline__ void dft9(float2* v) {
     }
 }
 
-// In-place forward transform of the permuted row z (360 complex values, z +
-// zz when zz is given: the two rows are summed as the first stage loads them).
-// One warp; z must not be read by other warps meanwhile.
-__device__ __forceinline__ void warp_pfa360(float2* z, const float2* zz, int lane) {
-    for (int d = lane; d < 45; d += 32) {           // length 8 along n1: stride 45
-        float2 v[8];
+// The small DFTs of the three stages, in place: d = 0 .. 44 of length 8 along n1
+// (stride 45; z + zz when zz is given, summed as they load), d = 0 .. 39 of length 9
+// along n2 (stride 5), d = 0 .. 71 of length 5 along n3 (stride 1).  Each stage after
+// every DFT of the one before.
+__device__ __forceinline__ void pfa360_stage8(float2* z, const float2* zz, int d) {
+    float2 v[8];
 #pragma unroll
-        for (int n1 = 0; n1 < 8; ++n1) {
-            v[n1] = z[45 * n1 + d];
-            if (zz) {
-                const float2 u = zz[45 * n1 + d];
-                v[n1].x += u.x;
-                v[n1].y += u.y;
-            }
+    for (int n1 = 0; n1 < 8; ++n1) {
+        v[n1] = z[45 * n1 + d];
+        if (zz) {
+            const float2 u = zz[45 * n1 + d];
+            v[n1].x += u.x;
+            v[n1].y += u.y;
         }
-        dft8(v);
-#pragma unroll
-        for (int k1 = 0; k1 < 8; ++k1) z[45 * k1 + d] = v[k1];
     }
+    dft8(v);
+#pragma unroll
+    for (int k1 = 0; k1 < 8; ++k1) z[45 * k1 + d] = v[k1];
+}
+
+__device__ __forceinline__ void pfa360_stage9(float2* z, int d) {
+    const int base = 45 * (d / 5) + d % 5;
+    float2 v[9];
+#pragma unroll
+    for (int n2 = 0; n2 < 9; ++n2) v[n2] = z[base + 5 * n2];
+    dft9(v);
+#pragma unroll
+    for (int k2 = 0; k2 < 9; ++k2) z[base + 5 * k2] = v[k2];
+}
+
+__device__ __forceinline__ void pfa360_stage5(float2* z, int d) {
+    float2 v[5];
+#pragma unroll
+    for (int n3 = 0; n3 < 5; ++n3) v[n3] = z[5 * d + n3];
+    dft_small<5>(v);
+#pragma unroll
+    for (int k3 = 0; k3 < 5; ++k3) z[5 * d + k3] = v[k3];
+}
+
+// In-place forward transform of the permuted row z (360 complex values, z +
+// zz when zz is given).  One warp; z must not be read by other warps meanwhile.
+__device__ __forceinline__ void warp_pfa360(float2* z, const float2* zz, int lane) {
+    for (int d = lane; d < 45; d += 32) pfa360_stage8(z, zz, d);
     __syncwarp();
-    for (int d = lane; d < 40; d += 32) {           // length 9 along n2: stride 5
-        const int base = 45 * (d / 5) + d % 5;
-        float2 v[9];
-#pragma unroll
-        for (int n2 = 0; n2 < 9; ++n2) v[n2] = z[base + 5 * n2];
-        dft9(v);
-#pragma unroll
-        for (int k2 = 0; k2 < 9; ++k2) z[base + 5 * k2] = v[k2];
-    }
+    for (int d = lane; d < 40; d += 32) pfa360_stage9(z, d);
     __syncwarp();
-    for (int d = lane; d < 72; d += 32) {           // length 5 along n3: stride 1
-        float2 v[5];
-#pragma unroll
-        for (int n3 = 0; n3 < 5; ++n3) v[n3] = z[5 * d + n3];
-        dft_small<5>(v);
-#pragma unroll
-        for (int k3 = 0; k3 < 5; ++k3) z[5 * d + k3] = v[k3];
-    }
+    for (int d = lane; d < 72; d += 32) pfa360_stage5(z, d);
     __syncwarp();
 }
 

@@ -293,6 +293,9 @@ void launch_plan_fnorm_max(const acom_plan_s* p, float* out, cudaStream_t st) {
 constexpr int kSelThreads = 256;
 constexpr int kSelWarps = kSelThreads / 32;
 constexpr int kBatch = 8;
+constexpr int kStateBit = 11;           // 2 N <= 1440 < 2^11
+constexpr int kNbrCap = 32;             // neighbours kept in shared memory and handed on
+static_assert(2 * kMaxPhi <= 1 << kStateBit, "bin and mirror below the state bits");
 constexpr int kOrderCap = 512;          // pending axes sorted once per pattern
 
 struct SelState {
@@ -300,10 +303,11 @@ struct SelState {
     unsigned Tidx;       // (z * 2 + mirror) * N + k of the best
     int bz, bk, bm;      // its axis, bin and mirror flag
     int nc;              // candidates of the current main batch
+    int64_t next;        // the CTA's next pattern
     int nref;            // candidates of the current refinement batch (a field of
                          // its own: thread 0 fills it right after the main loop's
                          // last barrier, while slower threads may still read nc)
-    int q;               // next neighbour to consider (refinement batches)
+    int q0, q, qe;       // the winner's neighbours: first, next to consider, end
     int n_order, at;     // pending axes counted, the next of `order` to consider
     float best3[3];      // winning correlation at bins k - 1, k, k + 1
     float Emax;          // rounding margin of the bounds
@@ -317,10 +321,13 @@ struct SelSmem {
     float2* tw;      // [N] (cos, sin)(2 pi i / N)
     float2* y;       // [kBatch][N] spectra of the batch, transformed in place
     float2* yt;      // [kBatch][N] transform ping-pong (shares space with part)
-    float4* part;    // [items][4] partial (A, B, C, D) of a shell part
+    float4* part;    // [4][sel_items(F)] partial A, B, C, D of a shell part
     float* U;        // [Z] bound, replaced by the exact score once evaluated
-    uint8_t* ev;     // [Z] 0 pending, 1 evaluated, 2 in the current batch
-    uint16_t* kb;    // [Z] bin + mirror * N of each evaluated axis' maximum
+    // [Z] bin + mirror * N of an evaluated axis' maximum, and above kStateBit its
+    // state: 0 pending, 1 evaluated, 2 in the current batch (4: of the winner's
+    // neighbourhood, while the runner-up is searched)
+    uint16_t* ax;
+    int* nbr;        // [kNbrCap] the winner's first neighbours
     uint16_t* order; // [kOrderCap] pending axes in decreasing bound (search_order)
     float* wv;       // [kSelWarps][kBatch] per-warp top-K values
     int* wi;         // [kSelWarps][kBatch] and axes
@@ -339,6 +346,11 @@ struct SelSmem {
     uint16_t* pout;
     SelState* st;
 };
+
+__device__ __forceinline__ int state_of(const SelSmem& sm, int z) { return sm.ax[z] >> kStateBit; }
+__device__ __forceinline__ void set_state(SelSmem& sm, int z, int v) {
+    sm.ax[z] = (uint16_t)((sm.ax[z] & ((1 << kStateBit) - 1)) | (v << kStateBit));
+}
 
 // Phase of axis z: the last p with poff[p] <= z.
 __device__ __forceinline__ int phase_of(const int* poff, int nph, int z) {
@@ -371,10 +383,10 @@ __device__ __forceinline__ void warp_argmax_bound(float& v, unsigned& i) {
     v = m ? __uint_as_float(m - 1u) : -CUDART_INF_F;
 }
 
-// The up to K pending axes (ev == 0) of largest bound with U rel + Emax >= thr
+// The up to K pending axes of largest bound with U rel + Emax >= thr
 // (with per_phase, thr is the best score so far of the axis' own phase), in
 // decreasing bound (ties: lowest axis), into cand and st->nc; marks them
-// ev = 2.  Each warp takes its K best by repeated argmax over entries strictly
+// in the batch.  Each warp takes its K best by repeated argmax over entries strictly
 // below its previous pick; warp 0 merges the warps' lists the same way.
 __device__ void block_topk(SelSmem& sm, int Z, int K, float thr, float rel, float Emax,
                            bool per_phase, int nph) {
@@ -385,7 +397,7 @@ __device__ void block_topk(SelSmem& sm, int Z, int K, float thr, float rel, floa
         float v = -CUDART_INF_F;
         unsigned zi = 0xffffffffu;
         for (int z = warp * 32 + lane; z < Z; z += kSelThreads) {
-            if (sm.ev[z] != 0) continue;
+            if (state_of(sm, z) != 0) continue;
             const float u = sm.U[z];
             const float tz = per_phase ? sm.st->Tp[phase_of(sm.poff, nph, z)] : thr;
             if (u * rel + Emax < tz || !better(lv, li, u, (unsigned)z)) continue;
@@ -429,7 +441,7 @@ __device__ void block_topk(SelSmem& sm, int Z, int K, float thr, float rel, floa
             if (zi == 0xffffffffu) break;
             if (lane == 0) {
                 sm.cand[n] = (int)zi;
-                sm.ev[zi] = 2;
+                set_state(sm, (int)zi, 2);
             }
             ++n;
             lv = v;
@@ -470,7 +482,8 @@ struct SelectArgs {
     FftRadix rad;                     // inverse-transform factorisation
     acom_result out;
     int64_t off;
-    int* n_eval;                      // optional: total axes evaluated
+    int* n_eval;                      // [0] total axes evaluated, [1] patterns taken
+    int taken;                        // n_eval[1] when this launch starts
     const float* xscale;              // [nb] 2^e of FP16 pattern spectra, or nullptr
     float inv_pscale;                 // 2^-k of the plan operand's scale
     float xs_mul;                     // the pattern operand holds xscale * xs_mul times X^
@@ -478,8 +491,14 @@ struct SelectArgs {
     int rescore_top;                  // > 0: evaluate only the top axes by bound (no certificate)
     const uint32_t* smask;            // [Zp][Spad / 32] non-zero plan shells
     OrientIn* oin;                    // [nb] the winners, for k_orient_compose
+    float2* onbr;                     // [nb][kNbrCap] their neighbours (score, axis)
     float eta_rs = 0.f;               // eta sqrt(Spad), from the host (FP64 there)
 };
+
+__host__ __device__ inline size_t sel_items(int F) {
+    const int Fq = shell_row_stride(F) >> 2;
+    return (size_t)(kSelThreads > kBatch * Fq ? kSelThreads : kBatch * Fq);
+}
 
 // Spectra c_dir + i c_mir of the batch's candidate axes, scaled by 1/N, into
 // the rows y[c] (both halves of the conjugate-symmetric spectrum), stored as
@@ -494,6 +513,7 @@ __device__ void batch_spectra(const SelectArgs& a, int64_t b, int nc, int s_lo, 
     h = h < 1 ? 1 : (h > 8 ? 8 : h);
     if (h > len) h = len > 1 ? len : 1;
     const int total = items * h;
+    const int pl = (int)sel_items(F);
     // each candidate's shells: rows of both the pattern and the axis not zero
     // (a product with a zero row is exactly 0 and is skipped); warp c lists
     // candidate c in increasing shell order
@@ -553,23 +573,22 @@ __device__ void batch_spectra(const SelectArgs& a, int64_t b, int nc, int s_lo, 
             fma4(C, p1, x2);
             fma4(D, p2, x1);
         }
-        float4* q = sm.part + 4 * idx;
-        q[0] = A;
-        q[1] = B;
-        q[2] = C;
-        q[3] = D;
+        sm.part[idx] = A;
+        sm.part[pl + idx] = B;
+        sm.part[2 * pl + idx] = C;
+        sm.part[3 * pl + idx] = D;
     }
     __syncthreads();
     const float invN = 1.0f / (float)N;
     for (int e = threadIdx.x; e < nc * F; e += kSelThreads) {
-        const int c = e / F, f = e - c * F, l = f & 3;
+        const int c = e / F, f = e - c * F;
         float A = 0.f, B = 0.f, C = 0.f, D = 0.f;
         for (int hh = 0; hh < h; ++hh) {
-            const float* q = reinterpret_cast<const float*>(sm.part + 4 * (hh * items + c * Fq + (f >> 2)));
-            A += q[l];
-            B += q[4 + l];
-            C += q[8 + l];
-            D += q[12 + l];
+            const float* q = reinterpret_cast<const float*>(sm.part + hh * items + c * Fq) + f;
+            A += q[0];
+            B += q[4 * pl];
+            C += q[8 * pl];
+            D += q[12 * pl];
         }
         const float dre = (A + B) * invN, dim = (C - D) * invN;
         const float mre = (A - B) * invN, mim = -(C + D) * invN;
@@ -581,20 +600,32 @@ __device__ void batch_spectra(const SelectArgs& a, int64_t b, int nc, int s_lo, 
     __syncthreads();
 }
 
-// One warp per candidate: C_dir[k] + i C_mir[k] = sum_f y_f exp(2 pi i f k / N),
-// taken as the conjugate of the forward transform of conj(y) (the rows hold
-// conj(y)); the argmax over
-// (k, mirror) with the correlation at k - 1, k, k + 1 goes to res[c].
+// C_dir[k] + i C_mir[k] = sum_f y_f exp(2 pi i f k / N) of each candidate, taken as
+// the conjugate of the forward transform of conj(y) (the rows hold conj(y)); the
+// argmax over (k, mirror) with the correlation at k - 1, k, k + 1 goes to res[c].
+// The prime-factor transform's three stages run over all candidates' small DFTs
+// with every thread (a warp a candidate left five of eight warps idle at the usual
+// three candidates); other lengths and the argmax take one warp per candidate.
 template <bool PFA>
 __device__ void batch_transforms(const SelectArgs& a, int nc, SelSmem& sm) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, N = a.N;
+    if constexpr (PFA) {
+        for (int t = threadIdx.x; t < nc * 45; t += kSelThreads)
+            pfa360_stage8(sm.y + (t / 45) * 360, nullptr, t % 45);
+        __syncthreads();
+        for (int t = threadIdx.x; t < nc * 40; t += kSelThreads)
+            pfa360_stage9(sm.y + (t / 40) * 360, t % 40);
+        __syncthreads();
+        for (int t = threadIdx.x; t < nc * 72; t += kSelThreads)
+            pfa360_stage5(sm.y + (t / 72) * 360, t % 72);
+        __syncthreads();
+    }
     for (int c = warp; c < nc; c += kSelWarps) {
         float2* row = sm.y + c * N;
         float2* alt = sm.yt + c * N;
         const float2* out;
         const uint16_t* pout = sm.pout;     // PFA: bin k at out[pout[k]]
         if constexpr (PFA) {
-            warp_pfa360(row, nullptr, lane);
             out = row;
         } else if (a.rad.n > 0) {
             out = warp_fft_fixed(row, alt, N, a.rad, sm.tw, lane);
@@ -627,18 +658,26 @@ __device__ void batch_transforms(const SelectArgs& a, int nc, SelSmem& sm) {
                 bi = (unsigned)(N + k);
             }
         }
-        warp_argmax(bv, bi);
-        if (lane == 0) {
-            const int m = (int)(bi / (unsigned)N), k = (int)bi - m * N;
-            const int km = (k + N - 1) % N, kp = (k + 1) % N;
-            const float2 ym = out[PFA ? (int)pout[km] : km], y0 = out[PFA ? (int)pout[k] : k],
-                         yp = out[PFA ? (int)pout[kp] : kp];
+        // the largest value, then the lowest index that holds it (+ 0: a zero's sign
+        // must not order equal values)
+        const unsigned key = bi == 0xffffffffu ? 0u : float_order_key(bv + 0.f);
+        const unsigned top = __reduce_max_sync(0xffffffffu, key);
+        bi = __reduce_min_sync(0xffffffffu, key == top ? bi : 0xffffffffu);
+        if (lane < 3) {
+            // lane 0 the bin, lanes 1 and 2 those before and after it
+            float v = 0.f;
+            if (bi != 0xffffffffu) {
+                const int m = (int)(bi / (unsigned)N), k = (int)bi - m * N;
+                const int kk = lane == 0 ? k : (lane == 1 ? (k + N - 1) % N : (k + 1) % N);
+                const float2 y = out[PFA ? (int)pout[kk] : kk];
+                v = m ? -y.y : y.x;
+            }
             float* r = sm.res + 5 * c;
-            r[0] = bv;
-            r[1] = __uint_as_float(bi);
-            r[2] = m ? -ym.y : ym.x;
-            r[3] = m ? -y0.y : y0.x;
-            r[4] = m ? -yp.y : yp.x;
+            if (lane == 0) {
+                r[0] = bi == 0xffffffffu ? -CUDART_INF_F : v;
+                r[1] = __uint_as_float(bi);
+            }
+            r[lane == 0 ? 3 : (lane == 1 ? 2 : 4)] = v;
         }
         __syncwarp();
     }
@@ -661,8 +700,7 @@ __device__ void fold_batch(int nc, int N, bool update, int nph, SelSmem& sm) {
             gidx = (unsigned)z * 2u * (unsigned)N + bi;
             ph = phase_of(sm.poff, nph, z);
             sm.U[z] = bv;
-            sm.kb[z] = (uint16_t)bi;
-            sm.ev[z] = 1;
+            sm.ax[z] = (uint16_t)(bi | (1u << kStateBit));
         }
         for (int p = 0; p < nph; ++p) {
             float v = ph == p ? bv : -CUDART_INF_F;
@@ -718,7 +756,7 @@ __device__ int search_order(SelSmem& sm, int Z, float rel, float Emax, bool per_
     for (int z0 = threadIdx.x - lane; z0 < Z; z0 += kSelThreads) {
         const int z = z0 + lane;
         const float u = z < Z ? sm.U[z] : 0.f;
-        const bool in = z < Z && sm.ev[z] == 0 && u == u &&
+        const bool in = z < Z && state_of(sm, z) == 0 && u == u &&
                         !(u * rel + Emax < search_threshold(sm, per_phase, nph, z));
         const unsigned m = __ballot_sync(0xffffffffu, in);
         if (m == 0u) continue;
@@ -747,7 +785,7 @@ __device__ int search_order(SelSmem& sm, int Z, float rel, float Emax, bool per_
 }
 
 // The next up to K axes of `order` that can still reach their threshold, into cand
-// and st->nc; marks them ev = 2.  The first K of the list in order are the K
+// and st->nc; marks them in the batch.  The first K of the list in order are the K
 // largest bounds still pending.
 __device__ void next_in_order(SelSmem& sm, int n, int K, float rel, float Emax, bool per_phase,
                               int nph) {
@@ -762,7 +800,7 @@ __device__ void next_in_order(SelSmem& sm, int n, int K, float rel, float Emax, 
             const int r = nc + __popc(m & ((1u << lane) - 1u));
             if (in && r < K) {
                 sm.cand[r] = z;
-                sm.ev[z] = 2;
+                set_state(sm, z, 2);
             }
             // past the K-th taken entry, or the whole group
             const unsigned kth = __ballot_sync(0xffffffffu, in && r == K - 1);
@@ -783,12 +821,17 @@ __device__ inline void matmul3d(const double* a, const double* b, double* c) {
             c[3 * i + j] = a[3 * i] * b[j] + a[3 * i + 1] * b[3 + j] + a[3 * i + 2] * b[6 + j];
 }
 
-// Outputs of the winner (warp 0).  For the orientation, the score-weighted
-// sum of the neighbour axes within 0.9 of the best (the lanes take the
-// neighbours and a butterfly sums them, so every lane holds the same FP64
-// sum) and the correlation at bins k - 1, k, k + 1 go to oin[b]; the FP64
-// composition runs in k_orient_compose, one thread per pattern, so that it
-// does not hold up the block.
+// neighbour q of the winner
+__device__ __forceinline__ int neighbour(const SelectArgs& a, const SelSmem& sm, int q) {
+    const int i = q - sm.st->q0;
+    return i < kNbrCap ? sm.nbr[i] : a.nbr_idx[q];
+}
+
+// Outputs of the winner (warp 0).  For the orientation, the neighbour axes within
+// 0.9 of the best with their scores (of more than kNbrCap neighbours their
+// score-weighted FP64 sum, by a butterfly) and the correlation at bins k - 1, k,
+// k + 1 go to oin[b] and onbr[b]; the FP64 sum and composition run in
+// k_orient_compose, one thread per pattern, so that they do not hold up the block.
 __device__ __noinline__ void write_outputs(const SelectArgs& a, int64_t b, const SelSmem& sm,
                                            bool want_ref, int lane) {
     const SelState& st = *sm.st;
@@ -797,10 +840,20 @@ __device__ __noinline__ void write_outputs(const SelectArgs& a, int64_t b, const
     const int64_t o = a.off + b;
     const float score = T == -CUDART_INF_F ? 0.f : T;
     double a0 = 0, a1 = 0, a2 = 0;
-    if (want_ref && a.refine) {
-        for (int q = a.nbr_ptr[bz] + lane; q < a.nbr_ptr[bz + 1]; q += 32) {
-            const int z2 = a.nbr_idx[q];
-            if (!sm.ev[z2]) continue;             // its true score is below 0.9 of the best
+    int n = 0;
+    // (an axis not evaluated has a true score below 0.9 of the best)
+    if (st.qe - st.q0 <= kNbrCap) {
+        const int z2 = st.q0 + lane < st.qe ? sm.nbr[lane] : -1;
+        const bool in = z2 >= 0 && state_of(sm, z2) && sm.U[z2] >= 0.9f * T;
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        n = __popc(m);
+        if (in)
+            a.onbr[b * kNbrCap + __popc(m & ((1u << lane) - 1u))] =
+                make_float2(sm.U[z2], __int_as_float(z2));
+    } else {
+        for (int q = st.q0 + lane; q < st.qe; q += 32) {
+            const int z2 = neighbour(a, sm, q);
+            if (!state_of(sm, z2)) continue;
             const float sc = sm.U[z2];
             if (sc >= 0.9f * T) {
                 a0 += (double)sc * a.za[3 * z2];
@@ -813,6 +866,7 @@ __device__ __noinline__ void write_outputs(const SelectArgs& a, int64_t b, const
             a1 += __shfl_xor_sync(0xffffffffu, a1, w);
             a2 += __shfl_xor_sync(0xffffffffu, a2, w);
         }
+        n = -1;
     }
     if (lane != 0) return;
     a.out.za_idx[o] = bz;
@@ -826,7 +880,7 @@ __device__ __noinline__ void write_outputs(const SelectArgs& a, int64_t b, const
         // there is no runner-up
         const int rz = st.ru_z;
         const int z = rz >= 0 ? rz : bz;
-        const int kbz = rz >= 0 ? (int)sm.kb[rz] : bk + bm * N;
+        const int kbz = rz >= 0 ? (int)(sm.ax[rz] & ((1 << kStateBit) - 1)) : bk + bm * N;
         const int mm = kbz >= N ? 1 : 0, kk = kbz - mm * N;
         if (a.out.runner_za) a.out.runner_za[o] = rz;
         if (a.out.runner_score) a.out.runner_score[o] = rz >= 0 ? st.ru_v : 0.f;
@@ -864,13 +918,15 @@ __device__ __noinline__ void write_outputs(const SelectArgs& a, int64_t b, const
     r.c3[2] = st.best3[2];
     r.z = bz;
     r.km = bk + bm * N;
+    r.n = n;
 }
 
 // Orientation of each winner, one thread per pattern: parabolic phi3 offset
 // from the correlation at k - 1, k, k + 1; the zone axis refined toward the
 // normalised score-weighted neighbour sum; m = T frame Rz(phi3) [Ry(pi)]
 // composed in FP64.
-__global__ void k_orient_compose(const OrientIn* __restrict__ oin, int nb, int N, int refine,
+__global__ void k_orient_compose(const OrientIn* __restrict__ oin,
+                                 const float2* __restrict__ onbr, int nb, int N, int refine,
                                  const double* __restrict__ za, const double* __restrict__ frames,
                                  acom_result out, int64_t off) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
@@ -886,7 +942,14 @@ __global__ void k_orient_compose(const OrientIn* __restrict__ oin, int nb, int N
             dk = (cm - cp) / (2.0 * den);
             dk = dk > 0.5 ? 0.5 : (dk < -0.5 ? -0.5 : dk);
         }
-        const double a0 = r.w[0], a1 = r.w[1], a2 = r.w[2];
+        double a0 = r.w[0], a1 = r.w[1], a2 = r.w[2];
+        for (int i = 0; i < r.n; ++i) {
+            const float2 v = onbr[(int64_t)b * kNbrCap + i];
+            const int z2 = __float_as_int(v.y);
+            a0 += (double)v.x * za[3 * z2];
+            a1 += (double)v.x * za[3 * z2 + 1];
+            a2 += (double)v.x * za[3 * z2 + 2];
+        }
         const double nrm = sqrt(a0 * a0 + a1 * a1 + a2 * a2);
         wref[0] = nrm > 0 ? a0 / nrm : za[3 * bz];
         wref[1] = nrm > 0 ? a1 / nrm : za[3 * bz + 1];
@@ -928,18 +991,13 @@ __global__ void k_orient_compose(const OrientIn* __restrict__ oin, int nb, int N
     for (int i = 0; i < 9; ++i) out.orient[9 * o + i] = (float)m2[i];
 }
 
-void launch_orient_compose(const acom_plan_s* p, const OrientIn* oin, int nb, int refine,
+void launch_orient_compose(const acom_plan_s* p, const OrientIn* oin, const float2* onbr, int nb, int refine,
                            acom_result out, int64_t off, cudaStream_t st) {
     if (nb <= 0) return;
     prof_begin(kKRefine, st);
-    k_orient_compose<<<(nb + 127) / 128, 128, 0, st>>>(oin, nb, p->N, refine, p->za, p->frames,
+    k_orient_compose<<<(nb + 127) / 128, 128, 0, st>>>(oin, onbr, nb, p->N, refine, p->za, p->frames,
                                                        out, off);
     prof_end(kKRefine, st);
-}
-
-__host__ __device__ inline size_t sel_items(int F) {
-    const int Fq = shell_row_stride(F) >> 2;
-    return (size_t)(kSelThreads > kBatch * Fq ? kSelThreads : kBatch * Fq);
 }
 
 // PFA: N = 360 with the prime-factor inverse transform, compiled alone (the
@@ -958,7 +1016,7 @@ __global__ void __launch_bounds__(kSelThreads, 3) k_select_exact(SelectArgs a) {
         off += (bytes + 15) & ~(size_t)15;
         return p;
     };
-    sm.tw = reinterpret_cast<float2*>(take(sizeof(float2) * N));
+    sm.tw = PFA ? nullptr : reinterpret_cast<float2*>(take(sizeof(float2) * N));
     sm.y = reinterpret_cast<float2*>(take(sizeof(float2) * kBatch * N));
     {
         const size_t pb = sizeof(float4) * 4 * sel_items(F), yb = sizeof(float2) * kBatch * N;
@@ -982,8 +1040,8 @@ __global__ void __launch_bounds__(kSelThreads, 3) k_select_exact(SelectArgs a) {
         sm.pout = reinterpret_cast<uint16_t*>(take(sizeof(uint16_t) * 360));
     }
     sm.st = reinterpret_cast<SelState*>(take(sizeof(SelState)));
-    sm.ev = take(Z);
-    sm.kb = reinterpret_cast<uint16_t*>(take(sizeof(uint16_t) * Z));
+    sm.ax = reinterpret_cast<uint16_t*>(take(sizeof(uint16_t) * Z));
+    sm.nbr = reinterpret_cast<int*>(take(sizeof(int) * kNbrCap));
     sm.order = reinterpret_cast<uint16_t*>(take(sizeof(uint16_t) * kOrderCap));
     const int nph = a.n_phases;
     for (int i = threadIdx.x; i <= nph; i += kSelThreads) sm.poff[i] = a.phase_off[i];
@@ -1005,7 +1063,10 @@ __global__ void __launch_bounds__(kSelThreads, 3) k_select_exact(SelectArgs a) {
     const bool want_ref = (a.out.phi3 != nullptr) || (a.out.orient != nullptr);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
-    for (int64_t b = blockIdx.x; b < a.nb; b += gridDim.x) {
+    // A pattern's evaluations vary several-fold, so a CTA takes the next pattern not yet
+    // taken (a fixed share left 13 % of the SM time idle on 8,190 patterns); thread 0
+    // takes it while this one is set up.
+    for (int64_t b = blockIdx.x; b < a.nb; b = sm.st->next) {
         // the bounds, and the three largest of each lane's (ties: lowest axis) for
         // the first batch
         float tv[3] = {-1.f, -1.f, -1.f};
@@ -1013,7 +1074,7 @@ __global__ void __launch_bounds__(kSelThreads, 3) k_select_exact(SelectArgs a) {
         for (int z = threadIdx.x; z < Z; z += kSelThreads) {
             const float u = later_groups(a.ts, a.extra, (int)b, z, a.U[b * Z + z]);
             sm.U[z] = u;
-            sm.ev[z] = 0;
+            sm.ax[z] = 0;
             if (u > tv[2]) {
                 const bool b1 = u > tv[1], b0 = u > tv[0];
                 tv[2] = b1 ? tv[1] : u;
@@ -1092,7 +1153,7 @@ __global__ void __launch_bounds__(kSelThreads, 3) k_select_exact(SelectArgs a) {
                     if (r == 2) sm.st->next_u = bv;
                     else if (bz != 0xffffffffu && rescore_top == 0) {
                         sm.cand[n++] = (int)bz;
-                        sm.ev[bz] = 2;
+                        set_state(sm, (int)bz, 2);
                     }
                 }
                 if (zi == bz) {
@@ -1109,9 +1170,11 @@ __global__ void __launch_bounds__(kSelThreads, 3) k_select_exact(SelectArgs a) {
                 ta += sm.red[kSelWarps + w];
             }
             SelState& st = *sm.st;
+            st.next = gridDim.x + (int64_t)(atomicAdd(a.n_eval + 1, 1) - a.taken);
             const float abs_term =
                 a.xscale ? 4.0f * a.eta_rs * ta : 0.f;
             st.Emax = (a.kappa * t + abs_term) / (float)N * 1.01f;
+            st.q0 = st.q = st.qe = 0;
             st.T = -CUDART_INF_F;
             st.Tidx = 0xffffffffu;
             st.bz = st.bk = st.bm = 0;
@@ -1119,6 +1182,15 @@ __global__ void __launch_bounds__(kSelThreads, 3) k_select_exact(SelectArgs a) {
             for (int p = 0; p < kMaxPhases; ++p) st.Tp[p] = -CUDART_INF_F;
         }
         __syncthreads();
+        // the next pattern's bounds and norms on their way to L2 meanwhile
+        if (sm.st->next < a.nb) {
+            const char* un = reinterpret_cast<const char*>(a.U + sm.st->next * Z);
+            for (int i = threadIdx.x * 128; i < 4 * Z; i += kSelThreads * 128)
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(un + i));
+            const char* xn = reinterpret_cast<const char*>(a.xfn + sm.st->next * F);
+            if ((int)threadIdx.x * 128 < 4 * F)
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(xn + threadIdx.x * 128));
+        }
         const float Emax = sm.st->Emax;
         const int2 sr = a.srange[b];
         int evals = 0;
@@ -1129,7 +1201,7 @@ __global__ void __launch_bounds__(kSelThreads, 3) k_select_exact(SelectArgs a) {
         //  1 the winner's grid neighbours that may reach 0.9 of the best (their
         //    exact scores weight the orientation refinement);
         //  2 the runner-up: the best axis outside the winner and its grid
-        //    neighbours (bit 4 of ev marks them meanwhile), certified like the
+        //    neighbours (state 4 marks them meanwhile), certified like the
         //    winner.
         const bool single = !per_phase && rescore_top == 0;
         const bool want_ru = FULL && (a.out.runner_za || a.out.runner_score || a.out.runner_orient);
@@ -1158,19 +1230,30 @@ __global__ void __launch_bounds__(kSelThreads, 3) k_select_exact(SelectArgs a) {
                 }
                 update = true;
             } else if (stage == 1) {
-                // thread 0 gathers the next batch of neighbours; all threads run it
-                const float T = sm.st->T;
-                if (threadIdx.x == 0) {
-                    const int qe = a.nbr_ptr[sm.st->bz + 1];
-                    int q = sm.st->q, n = 0;
-                    for (; q < qe && n < kBatch; ++q) {
-                        const int z2 = a.nbr_idx[q];
-                        if (sm.ev[z2] || sm.U[z2] * rel + Emax < 0.9f * T) continue;
-                        sm.cand[n++] = z2;
-                        sm.ev[z2] = 2;
+                // warp 0 gathers the next batch of neighbours; all threads run it
+                if (warp == 0) {
+                    SelState& st = *sm.st;
+                    const float T = st.T;
+                    int q = st.q, n = 0;
+                    while (q < st.qe && n < kBatch) {
+                        const int z2 = q + lane < st.qe ? neighbour(a, sm, q + lane) : -1;
+                        const bool in = z2 >= 0 && state_of(sm, z2) == 0 &&
+                                        !(sm.U[z2] * rel + Emax < 0.9f * T);
+                        const unsigned m = __ballot_sync(0xffffffffu, in);
+                        const int r = n + __popc(m & ((1u << lane) - 1u));
+                        if (in && r < kBatch) {
+                            sm.cand[r] = z2;
+                            set_state(sm, z2, 2);
+                        }
+                        const unsigned kth = __ballot_sync(0xffffffffu, in && r == kBatch - 1);
+                        n = min(kBatch, n + __popc(m));
+                        q += kth ? __ffs(kth) : 32;
                     }
-                    sm.st->q = q;
-                    sm.st->nref = n;
+                    __syncwarp();
+                    if (lane == 0) {
+                        st.q = q;
+                        st.nref = n;
+                    }
                 }
                 __syncthreads();
                 nc = sm.st->nref;
@@ -1179,7 +1262,7 @@ __global__ void __launch_bounds__(kSelThreads, 3) k_select_exact(SelectArgs a) {
                 float v = -CUDART_INF_F;
                 unsigned zi = 0xffffffffu;
                 for (int z = threadIdx.x; z < Z; z += kSelThreads)
-                    if (sm.ev[z] == 1 && better(sm.U[z], (unsigned)z, v, zi)) {
+                    if (state_of(sm, z) == 1 && better(sm.U[z], (unsigned)z, v, zi)) {
                         v = sm.U[z];
                         zi = (unsigned)z;
                     }
@@ -1229,22 +1312,30 @@ __global__ void __launch_bounds__(kSelThreads, 3) k_select_exact(SelectArgs a) {
             const int bz = sm.st->bz;
             if (stage == 2) {
                 for (int q = a.nbr_ptr[bz] + threadIdx.x; q < a.nbr_ptr[bz + 1]; q += kSelThreads)
-                    sm.ev[a.nbr_idx[q]] &= 3;
-                if (threadIdx.x == 0) sm.ev[bz] &= 3;
+                    set_state(sm, a.nbr_idx[q], state_of(sm, a.nbr_idx[q]) & 3);
+                if (threadIdx.x == 0) set_state(sm, bz, state_of(sm, bz) & 3);
                 __syncthreads();
                 stage = 3;
                 continue;
             }
             if (stage == 0 && want_ref && a.refine && sm.st->T > 0.f) {
                 __syncthreads();                 // every thread has read nc
-                if (threadIdx.x == 0) sm.st->q = a.nbr_ptr[bz];
+                if (warp == 0) {
+                    const int q0 = a.nbr_ptr[bz], qe = a.nbr_ptr[bz + 1];
+                    if (q0 + lane < qe) sm.nbr[lane] = a.nbr_idx[q0 + lane];
+                    if (lane == 0) {
+                        sm.st->q0 = sm.st->q = q0;
+                        sm.st->qe = qe;
+                    }
+                    __syncwarp();
+                }
                 stage = 1;
                 continue;
             }
             if (want_ru) {
                 for (int q = a.nbr_ptr[bz] + threadIdx.x; q < a.nbr_ptr[bz + 1]; q += kSelThreads)
-                    sm.ev[a.nbr_idx[q]] |= 4;
-                if (threadIdx.x == 0) sm.ev[bz] |= 4;
+                    set_state(sm, a.nbr_idx[q], state_of(sm, a.nbr_idx[q]) | 4);
+                if (threadIdx.x == 0) set_state(sm, bz, state_of(sm, bz) | 4);
                 __syncthreads();
                 stage = 2;
                 continue;
@@ -1253,9 +1344,9 @@ __global__ void __launch_bounds__(kSelThreads, 3) k_select_exact(SelectArgs a) {
         }
         if (a.out.za_scores)
             for (int z = threadIdx.x; z < Z; z += kSelThreads)
-                a.out.za_scores[(a.off + b) * Z + z] = sm.ev[z] ? sm.U[z] : sm.U[z] * rel + Emax;
+                a.out.za_scores[(a.off + b) * Z + z] = state_of(sm, z) ? sm.U[z] : sm.U[z] * rel + Emax;
         if (warp == 0) {
-            if (lane == 0 && a.n_eval) atomicAdd(a.n_eval, evals);
+            if (lane == 0) atomicAdd(a.n_eval, evals);
             write_outputs(a, b, sm, want_ref, lane);
         }
         __syncthreads();
@@ -1294,14 +1385,14 @@ void launch_phase_outputs(const acom_plan_s* p, const float* za_scores, int nb, 
 size_t select_smem_bytes(int Z, int N, int F, int Spad) {
     auto r16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
     const size_t pb = sizeof(float4) * 4 * sel_items(F), yb = sizeof(float2) * kBatch * (size_t)N;
-    return r16(sizeof(float2) * N) + r16(sizeof(float2) * kBatch * (size_t)N) + r16(pb > yb ? pb : yb) +
+    return (N == 360 ? 0 : r16(sizeof(float2) * N)) + r16(sizeof(float2) * kBatch * (size_t)N) + r16(pb > yb ? pb : yb) +
            r16(sizeof(float) * Z) + 2 * r16(sizeof(float) * kSelWarps * kBatch) +
            r16(sizeof(int) * kBatch) + r16(sizeof(float) * 5 * kBatch) +
            r16(sizeof(float) * 2 * kSelWarps) + r16(sizeof(int) * (kMaxPhases + 1)) +
            r16(sizeof(uint32_t) * (Spad >> 5)) + r16(sizeof(uint16_t) * kBatch * Spad) +
            r16(sizeof(int) * kBatch) +
            (N == 360 ? 2 * r16(sizeof(uint16_t) * 360) : 0) +
-           r16(sizeof(SelState)) + r16(Z) + r16(sizeof(uint16_t) * Z) +
+           r16(sizeof(SelState)) + r16(sizeof(uint16_t) * Z) + r16(sizeof(int) * kNbrCap) +
            r16(sizeof(uint16_t) * kOrderCap);
 }
 
@@ -1309,14 +1400,15 @@ void launch_select_exact(const acom_plan_s* p, const float* Xsr, const float* Xs
                          const float* extra, const TileSplit& ts, const float* xfn, const int2* srange, const uint32_t* rmask,
                          const float* pfmax, const float* xnorm2, int nb,
                          float kappa, int refine, acom_result out, int64_t off, int* n_eval,
-                         cudaStream_t st, const float* xscale, int rescore_top, OrientIn* oin) {
+                         cudaStream_t st, const float* xscale, int rescore_top, OrientIn* oin,
+                         float2* onbr, int* taken) {
     SelectArgs a{p->Psr, p->Psi, Xsr, Xsi, U, extra, ts, xfn, srange, rmask, pfmax, xnorm2, p->za, p->frames,
                  p->nbr_ptr,
                  p->nbr_idx, p->phase_off, p->n_phases, p->Z, p->F, p->N, p->S, p->Spad, nb, refine, kappa,
-                 fft_radices(p->N), out, off, n_eval, xscale, 1.0f / p->pscale,
+                 fft_radices(p->N), out, off, n_eval, *taken, xscale, 1.0f / p->pscale,
                  p->precision == ACOM_PREC_FP8 ? kFp8Shift : 1.0f,
                  (float)(p->precision == ACOM_PREC_FP8 ? kFp8Eta : kFp16Eta), rescore_top,
-                 p->smask, oin};
+                 p->smask, oin, onbr};
     a.eta_rs = (float)((double)a.eta * std::sqrt((double)p->Spad));
     const size_t smem = select_smem_bytes(p->Z, p->N, p->F, p->Spad);
     const bool pfa = p->N == 360;
@@ -1334,6 +1426,7 @@ void launch_select_exact(const acom_plan_s* p, const float* Xsr, const float* Xs
     int64_t grid = (int64_t)nsm * (per_sm > 0 ? per_sm : 1);
     if (grid > nb) grid = nb;
     if (grid <= 0) return;
+    *taken += nb;                    // every CTA takes one number for each pattern it had
     prof_begin(kKSelect, st);
     void* args[] = {(void*)&a};
     cudaLaunchKernel(kern, dim3((unsigned)grid), dim3(kSelThreads), args, smem, st);

@@ -93,3 +93,28 @@ def test_search_with_more_pending_axes_than_the_sorted_list():
     assert evaluated > 512          # or the sorted list was never exceeded
     # the same axis scored in batches of another size: another split of the shell sums
     np.testing.assert_allclose(got[3], got[0], rtol=2e-6)
+
+
+def test_refined_axis_with_more_neighbours_than_are_handed_on():
+    """A grid whose step is so coarse against its region that an axis has more than 32
+    neighbours takes the summed hand-off: the orientation is the oracle's refinement."""
+    from oracle import acom_oracle as O
+    from gpu_common import au_refl
+    from paper_2111_00171_gb300 import acom
+    # a narrow triangle about [001] whose stated area gives it many axes within 1.5 steps
+    tri = [[0, 0, 1], [0, 0.1, 1], [0.1, 0.1, 1]]
+    area = 4.0 * (14 * math.radians(2.0)) ** 2 / 8.0           # n = 14 rows at 2 degrees
+    scan = synth.random_patterns(8, n_patterns=12)
+    plan = acom.Plan(acom.au_crystal(), tri, area, 2.0, 40, 0.0375, 72, lam=LAM)
+    za = O.zone_axis_grid(*tri, 2.0, area)
+    assert (za @ za[60] >= math.cos(math.radians(3.0))).sum() > 32
+    oplan = O.orientation_plan(au_refl(), za, O.PlanParams(40, 0.0375, 72, 0.08, lam=LAM))
+    r = plan.match(*to_dev(scan))
+    m = r["orient"].cpu().numpy()
+    for b in range(scan.n_patterns):
+        mt = O.match_pattern(oplan, *scan.pattern(b))
+        if (int(r["za_idx"][b]), int(r["phi3_bin"][b]), int(r["mirror"][b])) != (mt.za, mt.k, mt.mirror):
+            continue                                            # a tie resolved the other way
+        # FP32 scores weight the mean: 1e-5 relative, over a neighbourhood of 3 degrees
+        np.testing.assert_allclose(m[b], O.refine(mt, za, 2.0).m, atol=1e-4)
+    plan.close()
