@@ -281,14 +281,20 @@ void launch_plan_fnorm_max(const acom_plan_s* p, float* out, cudaStream_t st) {
 // Selection and exact evaluation.  Persistent CTAs take the patterns in turn.
 // The candidate axes of a pattern are evaluated in batches of up to kBatch:
 //  * spectra: thread (shell part, candidate, frequency quad) runs down its
-//    share of the pattern's non-zero shells with 16-byte loads of the
-//    shell-major rows (four frequencies at once; the pattern's rows are shared
-//    by the candidates through L1) and accumulates the four real products;
-//    the shell parts are summed in shared memory;
-//  * transform: one warp per candidate takes the inverse transform along phi3
-//    of c_dir + i c_mir (both correlations are real, so one complex transform
-//    carries both) and the argmax over (phi3, mirror);
-//  * selection: a block-wide top-K of the pending bounds, two barriers.
+//    share of the shells that both the pattern and the axis reach, 16 bytes of
+//    each row at a time (four frequencies), the plan's rows on their way three
+//    shells ahead in shared memory, the pattern's in registers, and accumulates
+//    the four real products; the shell parts are summed in shared memory;
+//  * transform: the inverse transform along phi3 of c_dir + i c_mir (both
+//    correlations are real, so one complex transform carries both), for 360 bins
+//    by the whole block, else one warp per candidate, and the argmax over (phi3,
+//    mirror) by one warp per candidate;
+//  * selection: the first batch (two largest bounds) is picked as the bounds
+//    load, the later ones from a list sorted once (search_order).
+// Bound by the latency and the L1 throughput of the row loads: ncu on 8,190
+// patterns x 903 axes shows L1 61 %, L2 37 %, DRAM 14 % and issue 33 % busy, and
+// warps waiting on loads and, behind them, on the block's barriers.  Each axis
+// evaluated moves its rows (140 KB on the 1-degree plan) from L2.
 // ---------------------------------------------------------------------------
 constexpr int kSelThreads = 256;
 constexpr int kSelWarps = kSelThreads / 32;
@@ -296,6 +302,11 @@ constexpr int kBatch = 8;
 constexpr int kStateBit = 11;           // 2 N <= 1440 < 2^11
 constexpr int kNbrCap = 32;             // neighbours kept in shared memory and handed on
 static_assert(2 * kMaxPhi <= 1 << kStateBit, "bin and mirror below the state bits");
+// Shells of plan and pattern rows in flight per thread.  Three of each measured best:
+// 16,000 patterns x 3,486 axes 2.95 -> 2.44 ms, 2,000 x 3 matches 9.8 -> 8.5 ms, one
+// pattern 70 -> 61 us, 65,536 x 903 axes 7.68 -> 7.77; two 8.2 ms on the last, four 8.2
+// (more shared memory, less L1), plan rows cached in L1 (.ca) 11.6.
+constexpr int kRing = 3;
 constexpr int kOrderCap = 512;          // pending axes sorted once per pattern
 
 struct SelState {
@@ -320,6 +331,7 @@ struct SelState {
 struct SelSmem {
     float2* tw;      // [N] (cos, sin)(2 pi i / N)
     float2* y;       // [kBatch][N] spectra of the batch, transformed in place
+    float4* ring;    // [kRing][2][kSelThreads] plan rows on their way (shares space with y)
     float2* yt;      // [kBatch][N] transform ping-pong (shares space with part)
     float4* part;    // [4][sel_items(F)] partial A, B, C, D of a shell part
     float* U;        // [Z] bound, replaced by the exact score once evaluated
@@ -454,6 +466,20 @@ __device__ void block_topk(SelSmem& sm, int Z, int K, float thr, float rel, floa
     __syncthreads();
 }
 
+// 16 bytes of global memory on their way to shared memory, seen after a wait of the
+// same thread
+__device__ __forceinline__ void copy16_async(float4* dst, const float4* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int Pending>
+__device__ __forceinline__ void copies_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(Pending) : "memory");
+}
+
 __device__ __forceinline__ void fma4(float4& acc, const float4 p, const float4 x) {
     acc.x = fmaf(p.x, x.x, acc.x);
     acc.y = fmaf(p.y, x.y, acc.y);
@@ -548,31 +574,46 @@ __device__ void batch_spectra(const SelectArgs& a, int64_t b, int nc, int s_lo, 
         const float4* xr = xr0 + fq;
         const float4* xi = xi0 + fq;
         float4 A = make_float4(0.f, 0.f, 0.f, 0.f), B = A, C = A, D = A;
-        int i = sa;
-        for (; i + 1 < se; i += 2) {
-            const int o0 = L[i] * Fq, o1 = L[i + 1] * Fq;
-            const float4 x1a = __ldg(xr + o0), x2a = __ldg(xi + o0);
-            const float4 x1b = __ldg(xr + o1), x2b = __ldg(xi + o1);
-            const float4 p1a = __ldg(pr + o0), p2a = __ldg(pi + o0);
-            const float4 p1b = __ldg(pr + o1), p2b = __ldg(pi + o1);
-            fma4(A, p1a, x1a);
-            fma4(B, p2a, x2a);
-            fma4(C, p1a, x2a);
-            fma4(D, p2a, x1a);
-            fma4(A, p1b, x1b);
-            fma4(B, p2b, x2b);
-            fma4(C, p1b, x2b);
-            fma4(D, p2b, x1b);
+        // the plan rows of the next kRing shells are on their way to this thread's own
+        // slots (no barrier, no registers), the pattern rows of as many in registers
+        float4* ring = sm.ring + threadIdx.x;
+        auto fetch = [&](int i, int d) {
+            if (i < se) {
+                const int o = L[i] * Fq;
+                copy16_async(ring + 2 * d * kSelThreads, pr + o);
+                copy16_async(ring + (2 * d + 1) * kSelThreads, pi + o);
+            }
+            copies_commit();
+        };
+        float4 xn1[kRing], xn2[kRing];
+        auto load_x = [&](int i, int d) {
+            if (i < se) {
+                const int o = L[i] * Fq;
+                xn1[d] = __ldg(xr + o);
+                xn2[d] = __ldg(xi + o);
+            }
+        };
+#pragma unroll
+        for (int d = 0; d < kRing; ++d) fetch(sa + d, d);
+#pragma unroll
+        for (int d = 0; d < kRing; ++d) load_x(sa + d, d);
+        for (int i0 = sa; i0 < se; i0 += kRing) {
+#pragma unroll
+            for (int d = 0; d < kRing; ++d) {
+                const int i = i0 + d;
+                if (i >= se) break;
+                copies_wait<kRing - 1>();
+                const float4 p1 = ring[2 * d * kSelThreads], p2 = ring[(2 * d + 1) * kSelThreads];
+                const float4 x1 = xn1[d], x2 = xn2[d];
+                fma4(A, p1, x1);
+                fma4(B, p2, x2);
+                fma4(C, p1, x2);
+                fma4(D, p2, x1);
+                fetch(i + kRing, d);
+                load_x(i + kRing, d);
+            }
         }
-        if (i < se) {
-            const int o0 = L[i] * Fq;
-            const float4 x1 = __ldg(xr + o0), x2 = __ldg(xi + o0);
-            const float4 p1 = __ldg(pr + o0), p2 = __ldg(pi + o0);
-            fma4(A, p1, x1);
-            fma4(B, p2, x2);
-            fma4(C, p1, x2);
-            fma4(D, p2, x1);
-        }
+        copies_wait<0>();
         sm.part[idx] = A;
         sm.part[pl + idx] = B;
         sm.part[2 * pl + idx] = C;
@@ -1000,6 +1041,12 @@ void launch_orient_compose(const acom_plan_s* p, const OrientIn* oin, const floa
     prof_end(kKRefine, st);
 }
 
+// the batch's spectra, and before them the plan rows on their way
+__host__ __device__ inline size_t sel_row_bytes(int N) {
+    const size_t y = sizeof(float2) * kBatch * (size_t)N, r = sizeof(float4) * 2 * kRing * kSelThreads;
+    return y > r ? y : r;
+}
+
 // PFA: N = 360 with the prime-factor inverse transform, compiled alone (the
 // radix transforms' code stays out of this kernel).  FULL: per-phase
 // certificates, top-K rescoring or the runner-up may be asked for; without
@@ -1017,7 +1064,8 @@ __global__ void __launch_bounds__(kSelThreads, 3) k_select_exact(SelectArgs a) {
         return p;
     };
     sm.tw = PFA ? nullptr : reinterpret_cast<float2*>(take(sizeof(float2) * N));
-    sm.y = reinterpret_cast<float2*>(take(sizeof(float2) * kBatch * N));
+    sm.y = reinterpret_cast<float2*>(take(sel_row_bytes(N)));
+    sm.ring = reinterpret_cast<float4*>(sm.y);
     {
         const size_t pb = sizeof(float4) * 4 * sel_items(F), yb = sizeof(float2) * kBatch * N;
         unsigned char* shared_area = take(pb > yb ? pb : yb);
@@ -1385,7 +1433,7 @@ void launch_phase_outputs(const acom_plan_s* p, const float* za_scores, int nb, 
 size_t select_smem_bytes(int Z, int N, int F, int Spad) {
     auto r16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
     const size_t pb = sizeof(float4) * 4 * sel_items(F), yb = sizeof(float2) * kBatch * (size_t)N;
-    return (N == 360 ? 0 : r16(sizeof(float2) * N)) + r16(sizeof(float2) * kBatch * (size_t)N) + r16(pb > yb ? pb : yb) +
+    return (N == 360 ? 0 : r16(sizeof(float2) * N)) + r16(sel_row_bytes(N)) + r16(pb > yb ? pb : yb) +
            r16(sizeof(float) * Z) + 2 * r16(sizeof(float) * kSelWarps * kBatch) +
            r16(sizeof(int) * kBatch) + r16(sizeof(float) * 5 * kBatch) +
            r16(sizeof(float) * 2 * kSelWarps) + r16(sizeof(int) * (kMaxPhases + 1)) +
