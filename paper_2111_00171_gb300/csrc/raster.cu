@@ -249,6 +249,7 @@ k_raster_dft(RasterGeom geo, Loader ld, int64_t n_items, RasterOut out, int* err
             ss[rank] = sp[i];
         }
         for (int f = threadIdx.x; f < F; f += blockDim.x) fn2[f] = 0.f;
+        if (threadIdx.x >= 16 && threadIdx.x < 32) s_int[threadIdx.x] = 0;   // shells the tents reach
         if (threadIdx.x == 0) {
             s_int[40] = Spad;                // first shell with a non-zero row
             s_int[41] = 0;                   // one past the last
@@ -344,6 +345,7 @@ k_raster_dft(RasterGeom geo, Loader ld, int64_t n_items, RasterOut out, int* err
                 if (lane == 0 && nonzero) {
                     atomicMin(&s_int[40], s);
                     atomicMax(&s_int[41], s + 1);
+                    atomicOr(reinterpret_cast<unsigned*>(s_int + 16 + (s >> 5)), 1u << (s & 31));
                 }
             }
 #pragma unroll
@@ -411,6 +413,8 @@ k_raster_dft(RasterGeom geo, Loader ld, int64_t n_items, RasterOut out, int* err
                 out.srange[item] = lo < hi ? make_int2(lo, hi) : make_int2(0, 0);
             }
         }
+        if (out.rmask && threadIdx.x < (Spad >> 5))
+            out.rmask[item * (int64_t)(Spad >> 5) + threadIdx.x] = (uint32_t)s_int[16 + threadIdx.x];
         if (out.sumsq) {
             // Parseval: sum_j X^2 = (1/N) sum_f w_f sum_s |X^_f|^2
             float e = 0.f;

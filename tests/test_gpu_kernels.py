@@ -118,3 +118,21 @@ def test_refined_axis_with_more_neighbours_than_are_handed_on():
         # FP32 scores weight the mean: 1e-5 relative, over a neighbourhood of 3 degrees
         np.testing.assert_allclose(m[b], O.refine(mt, za, 2.0).m, atol=1e-4)
     plan.close()
+
+
+@pytest.mark.parametrize("precision", [0, 2], ids=["fp32", "fp16"])
+def test_bins_with_a_prime_factor_above_five(precision):
+    """84 = 4 * 3 * 7 bins take the direct transform: the certified match finds the
+    oracle's score (the exact evaluation reads the shells that the raster records)."""
+    from oracle import acom_oracle as O
+    from gpu_common import au_refl
+    v0, v1, v2, area = O.cubic_triangle()
+    za = O.zone_axis_grid(v0, v1, v2, 4.0, area)
+    oplan = O.orientation_plan(au_refl(), za, O.PlanParams(33, 0.045, 84, 0.08, lam=LAM))
+    plan = au_plan(4.0, 33, 0.045, 84, precision=precision)
+    scan = synth.random_patterns(84, n_patterns=40)
+    r = plan.match(*to_dev(scan))
+    for b in range(scan.n_patterns):
+        assert math.isclose(float(r["score"][b]), O.match_pattern(oplan, *scan.pattern(b)).score,
+                            rel_tol=1e-4), b
+    plan.close()
