@@ -50,6 +50,7 @@ struct RasterOut {
     float* im = nullptr;
     float* sre = nullptr;      // [item][Spad][Fs] (shell-major rows of frequencies, Fs = shell_row_stride(F))
     float* sim = nullptr;
+    float2* xs = nullptr;      // [item][S][F] interleaved (no 16-bit copy then)
     float* sumsq = nullptr;    // [item] sum of squares of the polar image
     float* fnorm = nullptr;    // [item][F] ||X^_f|| over shells
     int2* srange = nullptr;    // [item] first and one-past-last shell with a non-zero row
@@ -307,10 +308,13 @@ void launch_raster_plan(const RasterGeom& geo, const PlanSource& src, int Z,
                         const RasterOut& out, int* err, cudaStream_t st);
 void launch_raster_patterns(const RasterGeom& geo, const PatternSource& src,
                             const RasterOut& out, int* err, cudaStream_t st);
-void launch_scale_rows(float* re, float* im, const float* sumsq, int items, int row_elems,
-                       cudaStream_t st);
-void launch_spectra_export(const float* re, const float* im, int items, int F, int Spad, int S,
+void launch_spectra_export(const float* sre, const float* sim, int items, int F, int Spad, int S,
                            float* dst, cudaStream_t st);
+// shell-major rows to the frequency-major operand of the FP32 contraction (shells
+// from the plan's k0 on; rows outside rmask as zeros)
+void launch_rows_to_fmajor(const acom_plan_s* p, const float* sre, const float* sim,
+                           const uint32_t* rmask, int items, float* re, float* im,
+                           cudaStream_t st);
 size_t raster_smem_bytes(int N, int F);
 // match_fp32.cu
 void launch_contract_fp32(const acom_plan_s* p, const float* Xr, const float* Xi, int nb,
@@ -325,7 +329,6 @@ void launch_contract_bound_fp32(const acom_plan_s* p, const float* Xr, const flo
 // adds the later groups' bounds of the split tiles to U [nb][Z]
 void launch_sum_groups(const TileSplit& ts, float* U, const float* extra, int nb, int Z,
                        cudaStream_t st);
-void launch_plan_fnorm_max(const acom_plan_s* p, float* out, cudaStream_t st);
 // p->smask from the plan's shell-major spectra (p->smask allocated, Zp x Spad/32)
 void launch_plan_shell_mask(const acom_plan_s* p, cudaStream_t st);
 // match_tc.cu
@@ -344,6 +347,11 @@ void launch_contract_bound_tc(const acom_plan_s* p, const void* map_x, int pt_st
 // BF16 of P^ (kind 0), FP16 (1) or E4M3 (2) of scale * P^
 void launch_plan_to_operand(const float* Pr, const float* Pi, int Zp, int F, int Spad, void* dst,
                             cudaStream_t st, int kind, float scale);
+// From the raster's unnormalised shell-major rows p->Psr, p->Psi and their sums of
+// squares: the normalised rows in place, the frequency-major Pr, Pi, the tensor-core
+// operand Pb (scale times the spectra), the shell mask and max_z ||P^_zf||, rows of the
+// padding axes as zeros
+void launch_plan_layouts(const acom_plan_s* p, const float* sumsq, cudaStream_t st);
 void launch_orient_compose(const acom_plan_s* p, const OrientIn* oin, const float2* onbr, int nb,
                            int refine,
                            acom_result out, int64_t off, cudaStream_t st);

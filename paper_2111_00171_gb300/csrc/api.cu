@@ -424,10 +424,15 @@ acom_status acom_plan_create(const acom_crystal* crystal, const acom_za_grid* gr
     p->host_words[0] = p->host_words[1] = 0;
     ACOM_CK(cudaMemcpyAsync(p->phase_off, p->phase_off_host.data(), sizeof(int) * 2,
                             cudaMemcpyHostToDevice, st));
-    ACOM_CK(cudaMemsetAsync(p->Pr, 0, sizeof(float) * pelems, st));
-    ACOM_CK(cudaMemsetAsync(p->Pi, 0, sizeof(float) * pelems, st));
-    ACOM_CK(cudaMemsetAsync(p->Psr, 0, sizeof(float) * selems, st));
-    ACOM_CK(cudaMemsetAsync(p->Psi, 0, sizeof(float) * selems, st));
+    ACOM_CK(dalloc(&p->smask, (size_t)p->Zp * (p->Spad / 32), &p->bytes, st));
+    if (tc_precision(p->precision)) {
+        const int kind = tc_kind(p->precision);
+        p->pscale = kind == 0 ? 1.0f
+                              : fp16_plan_scale(p->N) * (kind == 2 ? kFp8Shift : 1.0f);
+        const size_t n = (size_t)p->F * p->Zp * p->Spad * tc_elem_bytes(p->precision);
+        ACOM_CK(pool_alloc(&p->Pb, 2 * n, st));
+        p->bytes += 2 * n;
+    }
     ACOM_CK(cudaMemsetAsync(p->err, 0, sizeof(int), st));
     ACOM_CK(cudaMemcpyAsync(p->za, za.data(), sizeof(double) * za.size(), cudaMemcpyHostToDevice, st));
     ACOM_CK(cudaMemcpyAsync(p->frames, frames.data(), sizeof(double) * frames.size(),
@@ -441,19 +446,8 @@ acom_status acom_plan_create(const acom_crystal* crystal, const acom_za_grid* gr
         destroy_plan(p);
         return s;
     }
-    launch_plan_fnorm_max(p, p->pfmax, st);
-    ACOM_CK(dalloc(&p->smask, (size_t)p->Zp * (p->Spad / 32), &p->bytes, st));
-    launch_plan_shell_mask(p, st);
-    ACOM_CK(cudaGetLastError());
     if (tc_precision(p->precision)) {
         const int kind = tc_kind(p->precision);
-        p->pscale = kind == 0 ? 1.0f
-                              : fp16_plan_scale(p->N) * (kind == 2 ? kFp8Shift : 1.0f);
-        const size_t n = (size_t)p->F * p->Zp * p->Spad * tc_elem_bytes(p->precision);
-        ACOM_CK(pool_alloc(&p->Pb, 2 * n, st));
-        p->bytes += 2 * n;
-        launch_plan_to_operand(p->Pr, p->Pi, p->Zp, p->F, p->Spad, p->Pb, st, kind, p->pscale);
-        ACOM_CK(cudaGetLastError());
         s = make_bf16_map(p->map_p, p->Pb, (uint64_t)p->F * p->Zp * 2, (uint64_t)p->Spad, kind,
                           256);
         if (s == ACOM_OK)
@@ -669,7 +663,7 @@ acom_status acom_plan_get_zone_axes(acom_plan p, double* dst) {
 
 acom_status acom_plan_get_spectra(acom_plan p, float* dst, void* cuda_stream) {
     if (!p || !dst) return set_error(ACOM_ERR_INVALID_ARG, "null argument");
-    launch_spectra_export(p->Pr, p->Pi, p->Z, p->F, p->Spad, p->S, dst, (cudaStream_t)cuda_stream);
+    launch_spectra_export(p->Psr, p->Psi, p->Z, p->F, p->Spad, p->S, dst, (cudaStream_t)cuda_stream);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? ACOM_OK : cuda_error(e, "get_spectra");
 }
@@ -709,27 +703,16 @@ acom_status acom_polar_spectra(acom_plan p, const acom_peaks_csr* peaks, float* 
     const int64_t B = peaks->n_patterns;
     if (B == 0) return ACOM_OK;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    const int chunk = (int)std::min<int64_t>(B, 1024);
-    s = ensure_workspace(p, chunk, false, true, st);
-    if (s != ACOM_OK) return s;
     cudaMemsetAsync(p->err, 0, sizeof(int), st);
     launch_check_row0(peaks->row_ptr, p->err, st);
     RasterGeom geo{p->S, p->Spad, p->N, p->F, (float)p->dq, (float)p->delta, (float)p->gamma_pow, 0};
-    for (int64_t c0 = 0; c0 < B; c0 += chunk) {
-        const int nb = (int)std::min<int64_t>(chunk, B - c0);
-        PatternSource src{nullptr, 0, peaks->row_ptr + c0, peaks->qx, peaks->qy, peaks->I, nb,
-                          (float)p->gamma_pow, (float)p->omega};
-        RasterOut ro;
-        ro.re = p->ws.Xr;
-        ro.im = p->ws.Xi;
-        ro.sumsq = p->ws.xnorm2;
-        launch_raster_patterns(geo, src, ro, p->err, st);
-        launch_spectra_export(p->ws.Xr, p->ws.Xi, nb, p->F, p->Spad, p->S,
-                              dst + 2 * c0 * (int64_t)p->S * p->F, st);
-        if (xnorm) {
-            cudaMemcpyAsync(xnorm + c0, p->ws.xnorm2, sizeof(float) * nb, cudaMemcpyDeviceToDevice, st);
-        }
-    }
+    // straight into the caller's arrays
+    PatternSource src{nullptr, 0, peaks->row_ptr, peaks->qx, peaks->qy, peaks->I, B,
+                      (float)p->gamma_pow, (float)p->omega};
+    RasterOut ro;
+    ro.xs = reinterpret_cast<float2*>(dst);
+    ro.sumsq = xnorm;
+    launch_raster_patterns(geo, src, ro, p->err, st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "polar_spectra launch");
     s = read_error_word(p, st);
@@ -837,8 +820,8 @@ static acom_status match_enqueue(acom_plan p, const acom_peaks_csr* peaks,
                           peaks->qy, peaks->I, nb, (float)p->gamma_pow, (float)p->omega,
                           xscale ? 1 : 0, xscale, p->k0};
         RasterOut ro;
-        ro.re = fp32_contraction ? w.Xr : nullptr;
-        ro.im = fp32_contraction ? w.Xi : nullptr;
+        ro.re = exhaustive ? w.Xr : nullptr;
+        ro.im = exhaustive ? w.Xi : nullptr;
         ro.sre = w.Xsr;
         ro.sim = w.Xsi;
         ro.sumsq = w.xnorm2;
@@ -865,6 +848,7 @@ static acom_status match_enqueue(acom_plan p, const acom_peaks_csr* peaks,
                 launch_contract_bound_tc(p, w.map_x, w.PTs, nb, ts, w.U, w.extra, st, xscale,
                                          cta_pairs);
             } else {
+                launch_rows_to_fmajor(p, w.Xsr, w.Xsi, w.rmask, nb, w.Xr, w.Xi, st);
                 launch_contract_bound_fp32(p, w.Xr, w.Xi, nb, ts, w.U, w.extra, st);
             }
             launch_select_exact(p, w.Xsr, w.Xsi, w.U, w.extra, ts, w.xfn, w.srange, w.rmask, p->pfmax,
@@ -955,8 +939,11 @@ acom_status acom_bounds(acom_plan p, const acom_peaks_csr* peaks, float* dst, vo
                           peaks->qy, peaks->I, nb, (float)p->gamma_pow, (float)p->omega,
                           xscale ? 1 : 0, xscale, p->k0};
         RasterOut ro;
-        ro.re = tc ? nullptr : p->ws.Xr;
-        ro.im = tc ? nullptr : p->ws.Xi;
+        if (!tc) {
+            ro.sre = p->ws.Xsr;
+            ro.sim = p->ws.Xsi;
+            ro.rmask = p->ws.rmask;
+        }
         ro.sumsq = p->ws.xnorm2;
         launch_raster_patterns(geo, src, ro, p->err, st);
         float* U = dst + c0 * (int64_t)p->Z;
@@ -965,6 +952,7 @@ acom_status acom_bounds(acom_plan p, const acom_peaks_csr* peaks, float* dst, vo
             convert_fp8(p, p->ws, st);
             launch_contract_bound_tc(p, p->ws.map_x, p->ws.PTs, nb, ts, U, p->ws.extra, st, xscale);
         } else {
+            launch_rows_to_fmajor(p, p->ws.Xsr, p->ws.Xsi, p->ws.rmask, nb, p->ws.Xr, p->ws.Xi, st);
             launch_contract_bound_fp32(p, p->ws.Xr, p->ws.Xi, nb, ts, U, p->ws.extra, st);
         }
         launch_sum_groups(ts, U, p->ws.extra, nb, p->Z, st);

@@ -224,25 +224,6 @@ void launch_sum_groups(const TileSplit& ts, float* U, const float* extra, int nb
     prof_end(kKMisc, st);
 }
 
-// ---------------------------------------------------------------------------
-// max over zone axes of ||P^_zf||_2 (over shells), per frequency, times
-// 1.0001 for the rounding of the norm itself: one warp per (axis, frequency)
-// row, lanes over the shells; the maximum of non-negative floats by an
-// integer atomicMax on their bit patterns (out cleared to +0 first)
-__global__ void k_plan_fnorm_max(const float* __restrict__ Pr, const float* __restrict__ Pi,
-                                 int Z, int F, int Spad, float* __restrict__ out) {
-    const int lane = threadIdx.x & 31;
-    const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (row >= (int64_t)Z * F) return;
-    const int f = (int)(row % F);
-    const float* pr = Pr + row * Spad;
-    const float* pi = Pi + row * Spad;
-    float a = 0.f;
-    for (int s = lane; s < Spad; s += 32) a = fmaf(pr[s], pr[s], fmaf(pi[s], pi[s], a));
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    if (lane == 0) atomicMax(reinterpret_cast<int*>(out) + f, __float_as_int(sqrtf(a) * 1.0001f));
-}
-
 // bit s of word [z][s / 32]: shell row s of axis z (re or im) has a non-zero
 // entry; one warp per row
 __global__ void k_plan_shell_mask(const float* __restrict__ Pr, const float* __restrict__ Pi,
@@ -265,15 +246,6 @@ void launch_plan_shell_mask(const acom_plan_s* p, cudaStream_t st) {
     prof_begin(kKMisc, st);
     k_plan_shell_mask<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(
         p->Psr, p->Psi, rows, p->Spad, shell_row_stride(p->F), p->smask);
-    prof_end(kKMisc, st);
-}
-
-void launch_plan_fnorm_max(const acom_plan_s* p, float* out, cudaStream_t st) {
-    const int64_t rows = (int64_t)p->Z * p->F;
-    cudaMemsetAsync(out, 0, sizeof(float) * (size_t)p->F, st);
-    prof_begin(kKMisc, st);
-    k_plan_fnorm_max<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(p->Pr, p->Pi, p->Z, p->F, p->Spad,
-                                                                   out);
     prof_end(kKMisc, st);
 }
 

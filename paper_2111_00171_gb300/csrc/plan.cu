@@ -7,7 +7,7 @@
 //                   (V_g of Eq. 4 is zero there).
 //   raster (raster.cu, PlanLoader)  P0 per zone axis and its Fourier
 //                   transform along phi3, plus ||P0||^2.
-//   k_scale_rows    P = A P0, A = 1/||P0||_2.
+//   k_plan_layouts (match_tc.cu)  P = A P0, A = 1/||P0||_2, in every layout.
 //
 // The zone-axis grid, the rotations R = Rz(phi1) Rx(theta2) (first two factors
 // of Eq. 10) and the grid-neighbour lists are small host computations in FP64.
@@ -221,15 +221,12 @@ acom_status build_plan_device(acom_plan_s* p, const acom_crystal* cr, cudaStream
                        (float)p->gamma_pow, 1};
         PlanSource src{p->refl_g, p->refl_amp, p->frames, p->G, p->lambda};
         RasterOut ro;
-        ro.re = p->Pr;
-        ro.im = p->Pi;
         ro.sre = p->Psr;
         ro.sim = p->Psi;
         ro.sumsq = d_sumsq;
         launch_raster_plan(geo, src, p->Z, ro, p->err, st);
         ACOM_TRY(cudaGetLastError());
-        launch_scale_rows(p->Pr, p->Pi, d_sumsq, p->Z, p->F * p->Spad, st);
-        launch_scale_rows(p->Psr, p->Psi, d_sumsq, p->Z, shell_row_stride(p->F) * p->Spad, st);
+        launch_plan_layouts(p, d_sumsq, st);
         ACOM_TRY(cudaGetLastError());
         int herr = 0;
         ACOM_TRY(cudaMemcpyAsync(&herr, p->err, sizeof(int), cudaMemcpyDeviceToHost, st));

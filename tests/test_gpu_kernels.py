@@ -136,3 +136,24 @@ def test_bins_with_a_prime_factor_above_five(precision):
         assert math.isclose(float(r["score"][b]), O.match_pattern(oplan, *scan.pattern(b)).score,
                             rel_tol=1e-4), b
     plan.close()
+
+
+@pytest.mark.parametrize("geometry", [(6.0, 200, 0.0075, 72), (3.0, 150, 0.01, 360),
+                                      (4.0, 33, 0.045, 84), (3.0, 117, 0.0125, 300)], ids=str)
+@pytest.mark.parametrize("precision", [0, 1, 2, 3], ids=["fp32", "bf16", "fp16", "fp8"])
+def test_plan_layouts(geometry, precision):
+    """The plan's spectra are normalised slices (Parseval over shells and bins), and the
+    polar spectra's norms agree with their sums, at frequency and shell counts that are
+    no multiples of the tiles."""
+    import torch
+    plan = au_plan(*geometry, precision=precision)
+    F, N = plan.info["n_freq"], plan.info["n_phi"]
+    w = torch.full((F,), 2.0 / N, dtype=torch.float64, device="cuda")
+    w[0] = w[-1] = 1.0 / N
+    norm = lambda x: (x.double().square().sum((1, 3)) * w).sum(1)
+    # FP32 sums of F terms and the rounding of the scale
+    assert ((norm(plan.spectra()) - 1).abs() < 2 * F * 2.0 ** -24).all()
+    peaks = to_dev(synth.random_patterns(6, n_patterns=37))
+    X, xn = plan.polar_spectra(*peaks)
+    assert ((norm(X).sqrt() - xn).abs() < 2 * F * 2.0 ** -24 * xn).all()
+    plan.close()
