@@ -36,7 +36,10 @@ typedef enum {
 
 /* Arithmetic used by the shell contraction and the inverse transform. */
 typedef enum {
-    ACOM_PREC_FP32 = 0,   /* FP32 CUDA-core path (reference GPU path)               */
+    ACOM_PREC_FP32 = 0,   /* FP32 operands (reference GPU path): the contraction on CUDA
+                             cores, or with each value as a pair of FP16 values on
+                             the tensor cores where that is no less accurate (at
+                             most 128 shells past the plan's first, n_phi >= 180) */
     ACOM_PREC_BF16 = 1,   /* BF16 operands on tcgen05 tensor cores, FP32 accumulate,
                              top candidates re-scored in FP32                       */
     ACOM_PREC_FP16 = 2,   /* FP16 operands on tcgen05 tensor cores, FP32 accumulate;
@@ -495,10 +498,9 @@ acom_status acom_kinematical_score_strain(acom_plan plan, const acom_peaks_csr* 
  * the spectral bound U = (1/N) sum_f w_f max(|c_f^dir|, |c_f^mir|) of the
  * direct and mirror correlation spectra, which is >= max over phi3 of both C
  * and C_mirror (section "Correlation Pattern Matching"; w_0 = w_{N/2} = 1,
- * else 2).  Computed at the plan's precision (FP32 CUDA
- * cores, or BF16 / FP16 tensor cores with FP32 accumulation) without any
- * rounding margin.  ``dst``: DEVICE [n_patterns][Z] FP32.  Stream-ordered; synchronises
- * once to read the error word.
+ * else 2).  Computed at the plan's precision (FP32, or BF16 / FP16 tensor cores
+ * with FP32 accumulation) without any rounding margin.  ``dst``: DEVICE
+ * [n_patterns][Z] FP32.  Stream-ordered; synchronises once to read the error word.
  */
 acom_status acom_bounds(acom_plan plan, const acom_peaks_csr* peaks, float* dst,
                         void* cuda_stream);

@@ -79,7 +79,7 @@ struct PatternSource {         // one chunk of CSR patterns
     int64_t n_items;
     float gamma_pow, omega;
     int xb_fp16 = 0;           // xb holds FP16 of 2^e_b X^ instead of BF16 of X^
-    float* xscale = nullptr;   // [n_items] 2^e_b of each pattern (with xb_fp16)
+    float* xscale = nullptr;   // [n_items] 2^e_b of each pattern (with xb_fp16, or without xb)
     int xb_k0 = 0;             // the contraction reads xb from this shell on: 16-shell
                                // tiles wholly below it are not written
 };
@@ -141,6 +141,7 @@ struct Workspace {
     float* za_scores = nullptr;    // [chunk][Z]
     float* xscale = nullptr;       // [chunk] 2^e of each pattern's FP16 spectrum
     void* XB8 = nullptr;           // E4M3 copy of XB (FP8 plans)
+    void* XS = nullptr;            // [F][PTs][128][2 ks] FP16 hi and lo (plans with Ps; map_x)
     OrientIn* oin = nullptr;       // [chunk] winners for the orientation kernel
     float2* onbr = nullptr;        // [chunk][32] their neighbours' (score, axis)
     size_t bytes = 0;
@@ -197,6 +198,11 @@ struct acom_plan_s {
     // (rounded down to a multiple of 16) where some axis' plan row is not
     // zero; the products below it are zero for every axis and pattern
     int k0 = 0;
+    // FP32 plans of at most 128 shells past k0: FP16 hi and lo of 2^k P^ on those
+    // shells, [F][Zp / 128][256][2 ks], for the split tensor-core contraction
+    void* Ps = nullptr;
+    int ks = 0;
+    alignas(64) unsigned char map_ps[128];
     float4* refl_tab = nullptr;       // [G] FP32 (g, |g|^gamma |F_g|^omega) for refinement
     unsigned long long* refine_pairs = nullptr;  // (reflection, peak) pairs of the last refine
     int64_t last_refine_pairs = 0;
@@ -339,6 +345,15 @@ void launch_half_to_e4m3(const void* src, void* dst, int64_t n, float mul, cudaS
 void set_wait_cycles(long long cycles);
 // xscale: per-pattern 2^e of FP16 pattern spectra (nullptr: BF16, no scale)
 // cta_pairs: 0 one CTA per MMA (cta_group::1), 1 CTA pairs (cta_group::2)
+// FP32 operands as FP16 pairs on the tensor cores (plans with Ps)
+int split_shells(const acom_plan_s* p);
+void launch_plan_split(const acom_plan_s* p, cudaStream_t st);
+void launch_rows_to_split(const acom_plan_s* p, const float* sre, const float* sim,
+                          const uint32_t* rmask, const float* xscale, int items, int PTs, void* dst,
+                          cudaStream_t st);
+void launch_contract_bound_split(const acom_plan_s* p, const void* map_x, int pt_stride, int nb,
+                                 const TileSplit& ts, float* U, float* extra, cudaStream_t st,
+                                 const float* xscale);
 TileSplit tc_split(const acom_plan_s* p, int nb, int tile_order, bool split);
 void launch_contract_bound_tc(const acom_plan_s* p, const void* map_x, int pt_stride, int nb,
                               const TileSplit& ts, float* U, float* extra, cudaStream_t st,

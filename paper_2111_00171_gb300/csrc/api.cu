@@ -158,6 +158,7 @@ static void free_workspace(Workspace& ws, cudaStream_t st) {
     pool_free(ws.XB, st);
     pool_free(ws.xscale, st);
     pool_free(ws.XB8, st);
+    pool_free(ws.XS, st);
     pool_free(ws.oin, st);
     pool_free(ws.onbr, st);
     ws = Workspace{};
@@ -220,6 +221,18 @@ static acom_status ensure_ws(acom_plan_s* p, Workspace& ws, int chunk, bool need
             return ms;
         }
     }
+    if (p->Ps) {
+        ws.PTs = (chunk + 63) / 64;
+        const size_t rows = (size_t)p->F * ws.PTs * 128;
+        if ((e = pool_alloc(&ws.XS, rows * p->ks * 4, st)) != cudaSuccess) goto fail;
+        acc += rows * p->ks * 4;
+        if ((e = dalloc(&ws.xscale, (size_t)chunk, &acc, st)) != cudaSuccess) goto fail;
+        acom_status ms = make_bf16_map(ws.map_x, ws.XS, rows, 2 * (uint64_t)p->ks, 1);
+        if (ms != ACOM_OK) {
+            free_workspace(ws, st);
+            return ms;
+        }
+    }
     ws.chunk = chunk;
     ws.bytes = acc;
     return ACOM_OK;
@@ -252,6 +265,7 @@ static void destroy_plan(acom_plan_s* p) {
     pool_free(p->err, st);
     pool_free(p->pfmax, st);
     pool_free(p->Pb, st);
+    pool_free(p->Ps, st);
     pool_free(p->phase_off, st);
     pool_free(p->refl_tab, st);
     pool_free(p->refine_pairs, st);
@@ -285,6 +299,21 @@ static cudaError_t plan_k0(acom_plan_s* p, cudaStream_t st) {
         }
     p->k0 = lo < p->Spad ? lo / 16 * 16 : 0;
     return cudaSuccess;
+}
+
+// FP32 plans: the split operand, once k0 is known.
+static acom_status make_split_operand(acom_plan_s* p, cudaStream_t st) {
+    p->ks = split_shells(p);
+    if (p->ks == 0) return ACOM_OK;
+    const size_t rows = (size_t)p->F * p->Zp * 2;
+    cudaError_t e = pool_alloc(&p->Ps, rows * p->ks * 4, st);
+    if (e != cudaSuccess) return cuda_error(e, "plan operand");
+    p->bytes += rows * p->ks * 4;
+    launch_plan_split(p, st);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_error(e, "plan operand");
+    return make_bf16_map(p->map_ps, p->Ps, rows, 2 * (uint64_t)p->ks, 1, 256);
 }
 
 // The first row pointer of a CSR batch must be 0 (the other row checks run in
@@ -460,6 +489,11 @@ acom_status acom_plan_create(const acom_crystal* crystal, const acom_za_grid* gr
     }
     ACOM_CK(cudaStreamSynchronize(st));
     ACOM_CK(plan_k0(p, st));
+    s = make_split_operand(p, st);
+    if (s != ACOM_OK) {
+        destroy_plan(p);
+        return s;
+    }
     prof_resolve();
     *out = p;
     return ACOM_OK;
@@ -618,6 +652,13 @@ acom_status acom_plan_concat(const acom_plan* plans, int32_t n_plans, void* cuda
     }
     ACOM_CK(cudaStreamSynchronize(st));
     ACOM_CK(plan_k0(p, st));
+    {
+        const acom_status s = make_split_operand(p, st);
+        if (s != ACOM_OK) {
+            destroy_plan(p);
+            return s;
+        }
+    }
     *out = p;
     return ACOM_OK;
 cuda_fail:
@@ -797,7 +838,8 @@ static acom_status match_enqueue(acom_plan p, const acom_peaks_csr* peaks,
     int chunk = opts && opts->chunk > 0 ? opts->chunk : (exhaustive ? 1024 : 8192);
     if (chunk > 65536) return set_error(ACOM_ERR_INVALID_ARG, "chunk must be <= 65536");
     chunk = (int)std::min<int64_t>(chunk, B);
-    const bool fp32_contraction = exhaustive || p->precision == ACOM_PREC_FP32;
+    // frequency-major FP32 spectra: for the CUDA-core contractions
+    const bool fp32_contraction = exhaustive || (p->precision == ACOM_PREC_FP32 && !p->Ps);
     if (capture && !(p->ws.chunk >= chunk && (!exhaustive || p->ws.Chat) &&
                      (!fp32_contraction || p->ws.Xr)))
         return set_error(ACOM_ERR_INVALID_ARG,
@@ -815,10 +857,11 @@ static acom_status match_enqueue(acom_plan p, const acom_peaks_csr* peaks,
     for (int64_t c0 = 0; c0 < B; c0 += chunk) {
         const int nb = (int)std::min<int64_t>(chunk, B - c0);
         const bool tc = !exhaustive && tc_precision(p->precision);
+        const bool pairs16 = !exhaustive && p->Ps;            // FP32 operands as FP16 pairs
         float* xscale = tc && p->precision != ACOM_PREC_BF16 ? w.xscale : nullptr;
         PatternSource src{tc ? w.XB : nullptr, w.PTs, peaks->row_ptr + c0, peaks->qx,
                           peaks->qy, peaks->I, nb, (float)p->gamma_pow, (float)p->omega,
-                          xscale ? 1 : 0, xscale, p->k0};
+                          xscale ? 1 : 0, pairs16 ? w.xscale : xscale, p->k0};
         RasterOut ro;
         ro.re = exhaustive ? w.Xr : nullptr;
         ro.im = exhaustive ? w.Xi : nullptr;
@@ -842,11 +885,15 @@ static acom_status match_enqueue(acom_plan p, const acom_peaks_csr* peaks,
             if (out->phase || out->phase_score)
                 launch_phase_outputs(p, w.za_scores, nb, *out, c0, st);
         } else {
-            const TileSplit ts = tc ? tc_split(p, nb, tile_order, true) : fp32_split(p, nb, true);
+            const TileSplit ts = tc || pairs16 ? tc_split(p, nb, tile_order, true)
+                                               : fp32_split(p, nb, true);
             if (tc) {
                 convert_fp8(p, w, st);
                 launch_contract_bound_tc(p, w.map_x, w.PTs, nb, ts, w.U, w.extra, st, xscale,
                                          cta_pairs);
+            } else if (pairs16) {
+                launch_rows_to_split(p, w.Xsr, w.Xsi, w.rmask, w.xscale, nb, w.PTs, w.XS, st);
+                launch_contract_bound_split(p, w.map_x, w.PTs, nb, ts, w.U, w.extra, st, w.xscale);
             } else {
                 launch_rows_to_fmajor(p, w.Xsr, w.Xsi, w.rmask, nb, w.Xr, w.Xi, st);
                 launch_contract_bound_fp32(p, w.Xr, w.Xi, nb, ts, w.U, w.extra, st);
@@ -927,7 +974,8 @@ acom_status acom_bounds(acom_plan p, const acom_peaks_csr* peaks, float* dst, vo
     const int chunk = (int)std::min<int64_t>(B, 8192);
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const bool tc = tc_precision(p->precision);
-    s = ensure_workspace(p, chunk, false, !tc, st);
+    const bool pairs16 = p->Ps != nullptr;                // FP32 operands as FP16 pairs
+    s = ensure_workspace(p, chunk, false, !tc && !pairs16, st);
     if (s != ACOM_OK) return s;
     cudaMemsetAsync(p->err, 0, sizeof(int), st);
     launch_check_row0(peaks->row_ptr, p->err, st);
@@ -937,7 +985,7 @@ acom_status acom_bounds(acom_plan p, const acom_peaks_csr* peaks, float* dst, vo
         float* xscale = tc && p->precision != ACOM_PREC_BF16 ? p->ws.xscale : nullptr;
         PatternSource src{tc ? p->ws.XB : nullptr, p->ws.PTs, peaks->row_ptr + c0, peaks->qx,
                           peaks->qy, peaks->I, nb, (float)p->gamma_pow, (float)p->omega,
-                          xscale ? 1 : 0, xscale, p->k0};
+                          xscale ? 1 : 0, pairs16 ? p->ws.xscale : xscale, p->k0};
         RasterOut ro;
         if (!tc) {
             ro.sre = p->ws.Xsr;
@@ -947,10 +995,15 @@ acom_status acom_bounds(acom_plan p, const acom_peaks_csr* peaks, float* dst, vo
         ro.sumsq = p->ws.xnorm2;
         launch_raster_patterns(geo, src, ro, p->err, st);
         float* U = dst + c0 * (int64_t)p->Z;
-        const TileSplit ts = tc ? tc_split(p, nb, 0, true) : fp32_split(p, nb, true);
+        const TileSplit ts = tc || pairs16 ? tc_split(p, nb, 0, true) : fp32_split(p, nb, true);
         if (tc) {
             convert_fp8(p, p->ws, st);
             launch_contract_bound_tc(p, p->ws.map_x, p->ws.PTs, nb, ts, U, p->ws.extra, st, xscale);
+        } else if (pairs16) {
+            launch_rows_to_split(p, p->ws.Xsr, p->ws.Xsi, p->ws.rmask, p->ws.xscale, nb, p->ws.PTs,
+                                 p->ws.XS, st);
+            launch_contract_bound_split(p, p->ws.map_x, p->ws.PTs, nb, ts, U, p->ws.extra, st,
+                                        p->ws.xscale);
         } else {
             launch_rows_to_fmajor(p, p->ws.Xsr, p->ws.Xsi, p->ws.rmask, nb, p->ws.Xr, p->ws.Xi, st);
             launch_contract_bound_fp32(p, p->ws.Xr, p->ws.Xi, nb, ts, U, p->ws.extra, st);

@@ -48,6 +48,7 @@
 #include <cudaTypedefs.h>
 #include <math_constants.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "acom_internal.cuh"
@@ -683,6 +684,317 @@ constexpr size_t tc_smem_bytes() {
     return 1024 + (size_t)kPSlots * kPBytes + (size_t)kXSlots * kXBytes + 8 * kBars + 16;
 }
 
+// ---- FP32 operands as FP16 pairs.  x = hi + lo (hi = FP16(x), lo = FP16(x - hi)
+// hold 22 bits and more of x), and a product of two is hi hi + hi lo + lo hi, so
+// three MMAs stand in for FP32 multiply-adds that the CUDA cores run at 1/30 of
+// the rate: 8,190 patterns x 903 axes 26.5 -> 3.7 ms (their match 29.4 -> 6.4 ms).  The tensor core
+// truncates its FP32 accumulation, about 2^-25 a step downwards on a coherent
+// sum (measured), so a K tile of 64 shells is an accumulation of its own: first
+// the cross terms, 2^-11 of the rest, then four hi hi steps; the epilogue adds
+// the two tiles' accumulators of a frequency rounding to nearest, and the sum
+// over frequencies runs in groups of a quarter.  The bound's error against FP64 is then
+// no larger than the FP32 kernel's: relative 2-norm over all pairs of 333 patterns,
+// three kinds of peak lists, 2.2e-7 to 3.7e-7 against 4.1e-7 to 4.2e-7 on 150 shells and
+// 360 bins, 2.0e-7 to 2.5e-7 against 2.9e-7 to 3.6e-7 on 75 to 117 shells and 180 to
+// 300 bins (split_shells says where not).
+// Roles and tiles as in k_contract_bound_tc.  A pattern slot holds a pattern
+// tile's hi and lo of one K tile, a plan slot the axis tile's; both K tiles of a
+// frequency stay for the second pattern tile.
+#define ACOM_TMEM_LD16x256_X2(taddr, r)                                                      \
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"   \
+                 : "=r"((r)[0]), "=r"((r)[1]), "=r"((r)[2]), "=r"((r)[3]), "=r"((r)[4]),     \
+                   "=r"((r)[5]), "=r"((r)[6]), "=r"((r)[7])                                  \
+                 : "r"(taddr))
+
+__device__ __forceinline__ void add_pair2(uint32_t& a0, uint32_t& a1, uint32_t b0, uint32_t b1) {
+    asm("{\n"
+        ".reg .b64 A, B;\n"
+        "mov.b64 A, {%0, %1};\n"
+        "mov.b64 B, {%2, %3};\n"
+        "add.rn.f32x2 A, A, B;\n"
+        "mov.b64 {%0, %1}, A;\n"
+        "}\n"
+        : "+r"(a0), "+r"(a1)
+        : "r"(b0), "r"(b1));
+}
+
+// a.Spad: columns of the hi half (the lo half follows); a.KT: K tiles, 1 or 2
+__global__ void __launch_bounds__(kThreads, 1)
+k_contract_bound_split(const __grid_constant__ CUtensorMap map_p,
+                       const __grid_constant__ CUtensorMap map_x, TcArgs a, int flush) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* ring_p = reinterpret_cast<unsigned char*>(
+        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    unsigned char* ring_x = ring_p + kPSlots * kPBytes;
+    uint64_t* xfull = reinterpret_cast<uint64_t*>(ring_x + kXSlots * kXBytes);   // [kXSlots]
+    uint64_t* xempty = xfull + kXSlots;
+    uint64_t* pfull = xempty + kXSlots;             // [kPSlots]
+    uint64_t* pempty = pfull + kPSlots;
+    uint64_t* done = pempty + kPSlots;              // [2] accumulation finished, per TMEM buffer
+    uint64_t* tempty = done + 2;                    // [2] accumulator read (epilogue warps, warp 2)
+    uint64_t* drain = tempty + 2;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kXSlots; ++i) mbar_init(smem_u32(xfull + i), 1);
+        for (int i = 0; i < kXSlots; ++i) mbar_init(smem_u32(xempty + i), 1);
+        for (int i = 0; i < kPSlots; ++i) mbar_init(smem_u32(pfull + i), 1);
+        for (int i = 0; i < kPSlots; ++i) mbar_init(smem_u32(pempty + i), 1);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(smem_u32(done + i), 1);
+            mbar_init(smem_u32(tempty + i), kEpiWarps + 1);
+        }
+        mbar_init(smem_u32(drain), 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_p)));
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_x)));
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                         smem_u32(tmem_slot)),
+                     "r"(kTmemCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = *tmem_slot;
+    const int n_units = a.ts.units();
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+        return mbar_wait(smem_u32(bar), parity, abort_flag, a.err, a.wait_cycles);
+    };
+
+    if (warp == 0 || warp == kProdP) {
+        // ------------------------------------------------ TMA producers
+        if (elect_one()) {
+            const bool xprod = warp == 0;
+            const int slots = xprod ? kXSlots : kPSlots;
+            uint64_t* full = xprod ? xfull : pfull;
+            uint64_t* empty = xprod ? xempty : pempty;
+            int slot = 0;
+            uint32_t phase = 0;          // parity of the slots' current use
+            uint32_t used = 0, last = 0; // per slot: used at all, parity of its last use
+            bool ok = true;
+            for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
+                const Unit w = unit_of(a, u);
+                const int nsub = min(2, a.PT - 2 * w.pu);
+                for (int f = w.f0; f < w.f1 && ok; ++f)
+                    for (int sub = 0; sub < (xprod ? nsub : 1) && ok; ++sub)
+                        for (int k = 0; k < a.KT; ++k) {
+                            if (!(ok = wait(empty + slot, phase ^ 1u))) break;
+                            const uint32_t fb = smem_u32(full + slot);
+                            mbar_expect_tx(fb, (xprod ? 2 : 4) * kTileBytes);
+#pragma unroll
+                            for (int h = 0; h < 2; ++h)              // hi, lo
+                                if (xprod)
+                                    tma_load_2d(smem_u32(ring_x + slot * kXBytes + h * kTileBytes),
+                                                &map_x, h * a.Spad + k * kKT,
+                                                (f * a.PTs + 2 * w.pu + sub) * 128, fb);
+                                else
+                                    tma_load_2d(smem_u32(ring_p + slot * kPBytes + h * 2 * kTileBytes),
+                                                &map_p, h * a.Spad + k * kKT,
+                                                f * a.Zrows + w.zt * 256, fb);
+                            used |= 1u << slot;
+                            last = (last & ~(1u << slot)) | (phase << slot);
+                            if (++slot == slots) {
+                                slot = 0;
+                                phase ^= 1u;
+                            }
+                        }
+            }
+            // every copy lands before the CTA's shared memory goes away
+            for (int i = 0; i < slots; ++i)
+                if (used & (1u << i)) {
+                    const long long w0 = clock64();
+                    while (!mbar_try(smem_u32(full + i), (last >> i) & 1u) &&
+                           clock64() - w0 < kWaitCycles) {
+                    }
+                }
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // ------------------------------------------------ MMA issuer
+        if (elect_one()) {
+            int xs = 0, pi = 0;                      // pattern slot, plan uses so far
+            uint32_t xph = 0, tph = 0, buf = 0;      // tph: bit b, parity of buffer b's next use
+            bool ok = true;
+            for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
+                const Unit w = unit_of(a, u);
+                const int nsub = min(2, a.PT - 2 * w.pu);
+                for (int f = w.f0; f < w.f1 && ok; ++f, pi += a.KT)
+                    for (int sub = 0; sub < nsub && ok; ++sub)
+                        for (int k = 0; k < a.KT; ++k) {
+                            const int pu = pi + k, ps = pu % kPSlots;
+                            if (!(ok = wait(tempty + buf, ((tph >> buf) & 1u) ^ 1u))) break;
+                            tph ^= 1u << buf;
+                            if ((sub == 0 && !wait(pfull + ps, (pu / kPSlots) & 1u)) ||
+                                !wait(xfull + xs, xph)) {
+                                ok = false;
+                                break;
+                            }
+                            fence_after();
+                            const int nk = min(kKT, a.Spad - k * kKT) >> 4;
+                            const uint64_t xd = sdesc(smem_u32(ring_x + xs * kXBytes));
+                            const uint64_t pd = sdesc(smem_u32(ring_p + ps * kPBytes));
+                            const uint32_t dacc = tmem + buf * 256;
+                            // hi lo, lo hi, then hi hi
+#pragma unroll
+                            for (int pass = 0; pass < 3; ++pass) {
+                                const uint64_t xa = xd + (pass == 1 ? kTileBytes >> 4 : 0);
+                                const uint64_t pa = pd + (pass == 0 ? 2 * kTileBytes >> 4 : 0);
+#pragma unroll
+                                for (int j = 0; j < 4; ++j)
+                                    if (j < nk)
+                                        mma_f16kind(dacc, xa + 2 * j, pa + 2 * j, a.idesc,
+                                                    (pass | j) ? 1u : 0u);
+                            }
+                            mma_commit(smem_u32(done + buf));
+                            buf ^= 1u;
+                            if (++xs == kXSlots) {
+                                xs = 0;
+                                xph ^= 1u;
+                            }
+                        }
+            }
+            // all MMAs issued by this thread complete before TMEM is released
+            mma_commit(smem_u32(drain));
+            const long long w0 = clock64();
+            while (!mbar_try(smem_u32(drain), 0) && clock64() - w0 < kWaitCycles) {
+            }
+        }
+        __syncwarp();
+    } else if (warp == 2) {
+        // ------------------------------------------------ slot release
+        if (elect_one()) {
+            int xs = 0, pi = 0;
+            uint32_t dph = 0, buf = 0;
+            bool ok = true;
+            for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
+                const Unit w = unit_of(a, u);
+                const int nsub = min(2, a.PT - 2 * w.pu);
+                for (int f = w.f0; f < w.f1 && ok; ++f, pi += a.KT)
+                    for (int sub = 0; sub < nsub && ok; ++sub)
+                        for (int k = 0; k < a.KT; ++k) {
+                            if (!(ok = wait(done + buf, (dph >> buf) & 1u))) break;
+                            dph ^= 1u << buf;
+                            mbar_arrive(smem_u32(xempty + xs));
+                            if (sub + 1 == nsub) mbar_arrive(smem_u32(pempty + (pi + k) % kPSlots));
+                            mbar_arrive(smem_u32(tempty + buf));
+                            xs = xs + 1 == kXSlots ? 0 : xs + 1;
+                            buf ^= 1u;
+                        }
+            }
+        }
+        __syncwarp();
+    } else {
+        // ------------------------------------------------ epilogue
+        const int q = warp & 3;                  // TMEM lane quarter: patterns 16q .. 16q + 15
+        const int zq = (warp - kEpi0) >> 2;      // axis columns 32 zq .. 32 zq + 31
+        const float invN = 1.0f / (float)a.N;
+        const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16) + zq * 32;
+        const bool two = a.KT == 2;
+        float ud[2][16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) ud[0][j] = ud[1][j] = 0.f;
+        uint32_t dph = 0, buf = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
+            const Unit w = unit_of(a, u);
+            const int nsub = min(2, a.PT - 2 * w.pu);
+            int since = 0;                       // frequencies since the last flush
+            for (int f = w.f0; f < w.f1; ++f) {
+                const float wf = (f == 0 || 2 * f == a.N) ? 1.f : 2.f;
+#pragma unroll
+                for (int sub = 0; sub < 2; ++sub) {
+                    if (sub >= nsub) break;
+                    for (int k = 0; k < a.KT; ++k) {
+                        const uint32_t b = buf ^ (uint32_t)k;
+                        if (!wait(done + b, (dph >> b) & 1u)) {
+                            ok = false;
+                            break;
+                        }
+                        dph ^= 1u << b;
+                    }
+                    if (!ok) break;
+                    fence_after();
+                    const uint32_t tb = tq + buf * 256, t2 = tq + (buf ^ 1u) * 256;
+                    // 8 patterns (16 lanes) x 16 axes at a time
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const uint32_t o = ((uint32_t)(c >> 1) << 20) + 16u * (c & 1);
+                        uint32_t V[16], W[16];               // (Xr, Xi) . Pr, (Xr, Xi) . Pi
+                        ACOM_TMEM_LD16x256_X2(tb + o, V);
+                        ACOM_TMEM_LD16x256_X2(tb + o + 128, V + 8);
+                        if (two) {
+                            ACOM_TMEM_LD16x256_X2(t2 + o, W);
+                            ACOM_TMEM_LD16x256_X2(t2 + o + 128, W + 8);
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) W[j] = 0u;
+                        }
+                        ACOM_TMEM_WAIT32(V, W);
+                        if (c == 3) {
+                            fence_before();
+                            __syncwarp();
+                            if (lane == 0) {
+                                mbar_arrive(smem_u32(tempty + buf));
+                                if (two) mbar_arrive(smem_u32(tempty + (buf ^ 1u)));
+                            }
+                        }
+                        if (two)
+#pragma unroll
+                            for (int j = 0; j < 16; j += 2) add_pair2(V[j], V[j + 1], W[j], W[j + 1]);
+#pragma unroll
+                        for (int n = 0; n < 2; ++n) {
+                            float* d = ud[sub] + 8 * (c >> 1) + 4 * (c & 1) + 2 * n;
+                            accumulate_pair2(V[4 * n], V[4 * n + 1], V[4 * n + 2], V[4 * n + 3],
+                                             V[8 + 4 * n], V[8 + 4 * n + 1], V[8 + 4 * n + 2],
+                                             V[8 + 4 * n + 3], wf, d[0], d[1]);
+                        }
+                    }
+                    if (!two) buf ^= 1u;
+                }
+                if (!ok) break;
+                if (++since < flush && f + 1 < w.f1) continue;
+                // the group's sum onto the earlier ones (this thread's own values)
+                const bool first_group = f + 1 - since == w.f0;
+                since = 0;
+#pragma unroll
+                for (int sub = 0; sub < 2; ++sub)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int b = (2 * w.pu + sub) * kNP + 8 * (2 * q + h) + (lane >> 2);
+                        const float sc = b < a.nb ? invN * a.inv_pscale / a.xscale[b] : 0.f;
+#pragma unroll
+                        for (int n = 0; n < 4; ++n)
+#pragma unroll
+                            for (int e = 0; e < 2; ++e) {
+                                const int z = w.zt * kM + zq * 32 + 8 * n + 2 * (lane & 3) + e;
+                                if (b < a.nb && z < a.Z) {
+                                    float* at = bound_at(a, w, b, z);
+                                    const float v = ud[sub][h * 8 + 2 * n + e] * sc;
+                                    *at = first_group ? v : *at + v;
+                                }
+                                ud[sub][h * 8 + 2 * n + e] = 0.f;
+                            }
+                    }
+            }
+        }
+    }
+    fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                     "r"(kTmemCols)
+                     : "memory");
+    }
+}
+
 // ---- CTA pairs: a cluster of two CTAs computes each MMA together (cta_group::2,
 // M = 256): CTA rank r holds pattern tile 2 p + r of the unit's two pattern
 // tiles (its A rows) and half of the axis tile's B operand (rank 0 the real
@@ -1108,6 +1420,123 @@ void launch_contract_bound_tc(const acom_plan_s* p, const void* map_x, int pt_st
     kern<<<n_units < nsm ? n_units : nsm, tc::kThreads, smem, st>>>(
         *reinterpret_cast<const CUtensorMap*>(p->map_p), mx, a);
     prof_end(kKContractBf16, st);
+}
+
+// Shells of the split operands, 0 when the plan keeps the CUDA cores: the two lines
+// are where the error against FP64 stops being below the FP32 kernel's.  More than
+// two K tiles need more than four hi hi steps per accumulation (eight on all-positive
+// spectra: 4.8e-7 against 2.4e-7).  Below 180 bins the FP32 kernel's sum over the few
+// frequencies rounds as little as the truncation does (72 bins, 40 shells: 7.73e-7
+// against 7.72e-7, both from the spectra).
+int split_shells(const acom_plan_s* p) {
+    const int K = (p->S - p->k0 + 15) / 16 * 16;
+    const bool smaller_error = K > 0 && K <= 2 * tc::kKT && p->N >= 180;
+    return p->precision == ACOM_PREC_FP32 && smaller_error ? K : 0;
+}
+
+void launch_contract_bound_split(const acom_plan_s* p, const void* map_x, int pt_stride, int nb,
+                                 const TileSplit& ts, float* U, float* extra, cudaStream_t st,
+                                 const float* xscale) {
+    tc::TcArgs a{};
+    a.ts = ts;
+    a.F = p->F;
+    a.N = p->N;
+    a.Z = p->Z;
+    a.nb = nb;
+    a.ZT = ts.ZT;
+    a.PT = (nb + tc::kNP - 1) / tc::kNP;
+    a.PTs = pt_stride;
+    a.Spad = p->ks;
+    a.KT = (p->ks + tc::kKT - 1) / tc::kKT;
+    a.Zrows = 2 * p->Zp;
+    a.U = U;
+    a.extra = extra;
+    a.err = p->err;
+    a.idesc = tc::kIdescF16;
+    a.xscale = xscale;
+    a.inv_pscale = 1.0f / fp16_plan_scale(p->N);
+    a.wait_cycles = g_wait_cycles > 0 ? g_wait_cycles : tc::kWaitCycles;
+    const int n_units = ts.units();
+    if (n_units <= 0) return;
+    const size_t smem = tc::tc_smem_bytes();
+    set_max_dynamic_smem((const void*)tc::k_contract_bound_split, smem);
+    prof_begin(kKContract, st);
+    tc::k_contract_bound_split<<<std::min(n_units, sm_count()), tc::kThreads, smem, st>>>(
+        *reinterpret_cast<const CUtensorMap*>(p->map_ps),
+        *reinterpret_cast<const CUtensorMap*>(map_x), a, (p->F + 3) / 4);
+    prof_end(kKContract, st);
+}
+
+__device__ __forceinline__ void split_half(float x, __half& hi, __half& lo) {
+    hi = __float2half_rn(x);
+    lo = __float2half_rn(x - __half2float(hi));
+}
+
+// plan rows -> [F][Zp / 128][256][2 K], hi then lo of scale times the spectra on the
+// shells from k0 on; a warp per row
+__global__ void k_plan_split(const float* __restrict__ Pr, const float* __restrict__ Pi, int Zp, int F,
+                             int Spad, int k0, int K, float scale, __half* __restrict__ dst) {
+    const int lane = threadIdx.x & 31;
+    const int64_t orow = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int ZT = Zp / 128;
+    if (orow >= (int64_t)F * ZT * 256) return;
+    const int row = (int)(orow % 256), zt = (int)(orow / 256 % ZT), f = (int)(orow / 256 / ZT);
+    const float* src = (row < 128 ? Pr : Pi) + ((int64_t)(zt * 128 + (row & 127)) * F + f) * Spad + k0;
+    __half* d = dst + orow * 2 * K;
+    for (int s = lane; s < K; s += 32) split_half(scale * src[s], d[s], d[K + s]);
+}
+
+void launch_plan_split(const acom_plan_s* p, cudaStream_t st) {
+    const int64_t rows = (int64_t)p->F * p->Zp * 2;
+    prof_begin(kKMisc, st);
+    k_plan_split<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(
+        p->Pr, p->Pi, p->Zp, p->F, p->Spad, p->k0, p->ks, fp16_plan_scale(p->N),
+        reinterpret_cast<__half*>(p->Ps));
+    prof_end(kKMisc, st);
+}
+
+// the patterns' shell-major rows -> [F][PTs][128][2 K] (16-row groups: 8 patterns'
+// real rows, their imaginary rows), hi then lo of 2^e X^, through 32 x 32 tiles in
+// shared memory; rows outside the pattern's mask as zeros
+__global__ void __launch_bounds__(256)
+k_rows_to_split(const float* __restrict__ sre, const float* __restrict__ sim,
+                const uint32_t* __restrict__ rmask, const float* __restrict__ xscale, int F, int Spad,
+                int k0, int K, int PTs, __half* __restrict__ dst) {
+    __shared__ float tr[32][33], ti[32][33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t item = blockIdx.x;
+    const int f0 = blockIdx.y * 32, Fs = shell_row_stride(F), MW = Spad >> 5;
+    const float sc = xscale[item];
+    const int64_t row0 = (item >> 6) * 128 + ((item & 63) >> 3) * 16 + (item & 7);
+    for (int s0 = 0; s0 < K; s0 += 32) {
+        for (int r = warp; r < 32; r += 8) {
+            const int s = k0 + s0 + r;
+            const bool in = s0 + r < K && f0 + lane < Fs && (rmask[item * MW + (s >> 5)] >> (s & 31) & 1u);
+            const int64_t o = (item * Spad + s) * (int64_t)Fs + f0 + lane;
+            tr[r][lane] = in ? sre[o] : 0.f;
+            ti[r][lane] = in ? sim[o] : 0.f;
+        }
+        __syncthreads();
+        for (int r = warp; r < 32 && f0 + r < F; r += 8) {
+            if (s0 + lane < K) {
+                __half* d = dst + ((int64_t)(f0 + r) * PTs * 128 + row0) * 2 * K + s0 + lane;
+                split_half(sc * tr[lane][r], d[0], d[K]);
+                d += (int64_t)16 * K;                    // 8 rows on: the imaginary parts
+                split_half(sc * ti[lane][r], d[0], d[K]);
+            }
+        }
+        __syncthreads();
+    }
+}
+
+void launch_rows_to_split(const acom_plan_s* p, const float* sre, const float* sim,
+                          const uint32_t* rmask, const float* xscale, int items, int PTs, void* dst,
+                          cudaStream_t st) {
+    if (items <= 0) return;
+    prof_begin(kKMisc, st);
+    k_rows_to_split<<<dim3((unsigned)items, (unsigned)((p->F + 31) / 32)), 256, 0, st>>>(
+        sre, sim, rmask, xscale, p->F, p->Spad, p->k0, p->ks, PTs, reinterpret_cast<__half*>(dst));
+    prof_end(kKMisc, st);
 }
 
 // FP32 spectra [Zp][F][Spad] (real and imaginary arrays) -> the merged

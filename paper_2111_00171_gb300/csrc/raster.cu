@@ -256,7 +256,7 @@ k_raster_dft(RasterGeom geo, Loader ld, int64_t n_items, RasterOut out, int* err
             s_int[41] = 0;                   // one past the last
         }
         __syncthreads();
-        const bool half = ld.xb_out() && ld.xb_half();
+        const bool half = ld.xb_out() ? ld.xb_half() : ld.xscale_out() != nullptr;
         float xsc = 1.0f;
         if (half) {
             xsc = fp16_pattern_scale(sp, np, geo, dphi, s_int + 56);
@@ -571,9 +571,8 @@ k_raster_fft(RasterGeom geo, Loader ld, int64_t n_items, RasterOut out, FftRadix
         }
         if (threadIdx.x < 16) s_int[16 + threadIdx.x] = 0;    // shells the tents reach
         __syncthreads();
-        constexpr bool half = XB == 2;
         float xsc = 1.0f;
-        if (half) {
+        if (XB == 2 || (XB == 0 && ld.xscale_out())) {
             xsc = fp16_pattern_scale(sp, np, geo, dphi, s_int + 56);
             if (threadIdx.x == 0) ld.xscale_out()[item] = xsc;
         }

@@ -45,7 +45,9 @@ def bounds64(plan, peaks):
 
 
 # one pattern; a tile's edge and one past it; more tiles than the GPU holds CTAs of
-@pytest.mark.parametrize("geometry", [(3.0, 75, 0.02, 180), (6.0, 200, 0.0075, 72),
+# (on the tensor cores: one K tile, two, a second one not full; else on the CUDA cores)
+@pytest.mark.parametrize("geometry", [(3.0, 75, 0.02, 180), (3.0, 150, 0.01, 360),
+                                      (4.0, 117, 0.0125, 300), (6.0, 200, 0.0075, 72),
                                       (2.0, 33, 0.045, 84)], ids=str)
 @pytest.mark.parametrize("patterns", [1, 63, 65, 1300])
 def test_fp32_bounds_at_tile_edges(geometry, patterns):
@@ -156,4 +158,20 @@ def test_plan_layouts(geometry, precision):
     peaks = to_dev(synth.random_patterns(6, n_patterns=37))
     X, xn = plan.polar_spectra(*peaks)
     assert ((norm(X).sqrt() - xn).abs() < 2 * F * 2.0 ** -24 * xn).all()
+    plan.close()
+
+
+@pytest.mark.parametrize("geometry", [(3.0, 75, 0.02, 180), (3.0, 150, 0.01, 360),
+                                      (4.0, 117, 0.0125, 300)], ids=str)
+def test_fp16_pairs_are_no_less_accurate_than_fp32(geometry):
+    """The FP32 contraction on the tensor cores (FP16 pairs, bounds()) is no further from
+    FP64 than the one on the CUDA cores (bounds_static())."""
+    import torch
+    plan = au_plan(*geometry)
+    peaks = to_dev(synth.random_patterns(123, n_patterns=200))
+    want, _ = bounds64(plan, peaks)
+    pairs = plan.bounds(*peaks)
+    cores = plan.bounds_static(*peaks, out=torch.empty_like(pairs))
+    off = lambda u: float((u.double() - want).norm())
+    assert off(pairs) <= off(cores)
     plan.close()
