@@ -478,12 +478,36 @@ size_t raster_fft_smem_bytes(int N, int F, size_t peak_bytes) {
     const int W = kRasterThreads / 32;
     size_t b = 0;
     b += peak_bytes * kMaxPeaks;                         // peaks, sorted in place by radius
-    b += sizeof(float2) * N;                             // twiddles
+    b += sizeof(float2) * N;                             // twiddles (360 bins: room only)
     b += sizeof(float2) * 2 * W * N;                     // per-warp row and transform buffer
     b += sizeof(uint32_t) * 2 * F * kFftStageWords;      // BF16 staging of a shell tile
     b += sizeof(int) * 64;                               // scratch
     if (N == 360) b += sizeof(uint16_t) * 2 * 360;       // prime-factor input, output positions
     return b;
+}
+
+// Barrier of the warps' arrivals on a staged tile (below).  Every warp arrives on every
+// tile, so a wait ends; the count only keeps a broken invariant from hanging the GPU.
+__device__ __forceinline__ void tile_wait(uint64_t* bar, uint32_t parity) {
+    const uint32_t b = (uint32_t)__cvta_generic_to_shared(bar);
+    for (int i = 0; i < (1 << 22); ++i) {
+        uint32_t ok;
+        asm volatile(
+            "{\n"
+            ".reg .pred p;\n"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+            "selp.u32 %0, 1, 0, p;\n"
+            "}\n"
+            : "=r"(ok)
+            : "r"(b), "r"(parity)
+            : "memory");
+        if (ok) return;
+    }
+}
+__device__ __forceinline__ void tile_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(bar))
+                 : "memory");
 }
 
 // PFA: N = 360 and its prime-factor transform, compiled alone (the radix
@@ -515,11 +539,37 @@ k_raster_fft(RasterGeom geo, Loader ld, int64_t n_items, RasterOut out, FftRadix
     float* scratch = reinterpret_cast<float*>(zb);     // after the last transform of an item
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        double c, sn;
-        sincospi(2.0 * (double)i / (double)N, &sn, &c);
-        tw[i] = make_float2((float)c, (float)sn);
+    // The 16-bit copy of a 16-shell tile goes out through shared memory.  A pattern
+    // of few peaks leaves room behind its peak list for a second staging buffer:
+    // each warp then stages its pair of tile t, arrives, and only after its tents
+    // and transform of tile t + 1 waits for the others' arrivals and copies its
+    // share of tile t.  (The warps' work differs by the peaks of their pairs; with
+    // one buffer and two block barriers a tile a quarter of the kernel went into
+    // waiting.  65,536 patterns, 150 shells x 360 bins: 8.67 -> 7.86 ms.)  A warp that
+    // stages tile t has seen every arrival of tile t - 1, and each warp arrives there
+    // after its copy of tile t - 2, so the buffer is free.
+    uint32_t* stage2 = reinterpret_cast<uint32_t*>(smem + sizeof(PeakT) * kMaxPeaks +
+                                                   (pfa ? sizeof(float2) * 360 : 0)) -
+                       2 * F * kFftStageWords;
+    const int dbl_peaks =
+        XB == 0 ? -1
+                : (int)((reinterpret_cast<unsigned char*>(stage2) - smem) / (ptrdiff_t)sizeof(PeakT));
+    uint64_t* tile_bar = reinterpret_cast<uint64_t*>(s_int + 32);       // [2]
+    if (XB != 0 && threadIdx.x == 0) {
+        for (int i = 0; i < 2; ++i)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(
+                             (uint32_t)__cvta_generic_to_shared(tile_bar + i)),
+                         "r"(W)
+                         : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    uint32_t tile_ph = 0;                // bit i: parity of buffer i's next use
+    if (!pfa)
+        for (int i = threadIdx.x; i < N; i += blockDim.x) {
+            double c, sn;
+            sincospi(2.0 * (double)i / (double)N, &sn, &c);
+            tw[i] = make_float2((float)c, (float)sn);
+        }
     if (pfa)
         for (int i = threadIdx.x; i < 360; i += blockDim.x) {
             s_perm[i] = (uint16_t)pfa360_in(i);
@@ -580,6 +630,23 @@ k_raster_fft(RasterGeom geo, Loader ld, int64_t n_items, RasterOut out, FftRadix
 #pragma unroll
         for (int k = 0; k < kFL; ++k) fa[k] = 0.f;
         int w_lo = Spad, w_hi = 0;      // this warp's non-zero shells
+        // the tile's 16-bit copy in the tensor-core layout (64-pattern tiles whose
+        // 16-row groups hold 8 patterns' real rows, then their imaginary rows):
+        // 32 bytes (16 shells) per row
+        auto copy_tile = [&](const uint32_t* from, int t0) {
+            const int64_t tile = item / 64, r = item % 64;
+            const int64_t rbase = (r >> 3) * 16 + (r & 7);
+            for (int e = threadIdx.x; e < 2 * F * 2; e += blockDim.x) {
+                const int row = e >> 1, q = e & 1;
+                const int c = row >= F, f = row - c * F;
+                const uint32_t* src = from + row * kFftStageWords + 4 * q;
+                const uint4 v = make_uint4(src[0], src[1], src[2], src[3]);
+                const int64_t grow = ((int64_t)f * ld.xb_tiles() + tile) * 128 + rbase + c * 8;
+                *reinterpret_cast<uint4*>(xb + grow * Spad + t0 + 8 * q) = v;
+            }
+        };
+        const bool dbl = np <= dbl_peaks;       // room for a second staging buffer
+        int staged = 0, out_t0 = -1;            // tiles staged, the one still to copy
 
         for (int t0 = 0; t0 < Spad; t0 += kFftTile) {
             // the 16-bit copy of a tile the contraction never reads is skipped
@@ -745,6 +812,16 @@ k_raster_fft(RasterGeom geo, Loader ld, int64_t n_items, RasterOut out, FftRadix
                 }
                 const float2* Z =
                     !any ? nullptr : (pfa ? z : warp_fft_fixed(z, zz, N, rad, tw, lane));
+                uint32_t* stg_to = stage;
+                if (XB != 0 && stg && dbl) {
+                    if (out_t0 >= 0) {               // the tile before this one
+                        const int pb = (staged - 1) & 1;
+                        tile_wait(tile_bar + pb, (tile_ph >> pb) & 1u);
+                        tile_ph ^= 1u << pb;
+                        copy_tile(pb ? stage2 : stage, out_t0);
+                    }
+                    stg_to = staged & 1 ? stage2 : stage;
+                }
                 // real rows a (shell sA), b (shell sA + 1) from Z = FFT(a + i b):
                 //   A_f = (Z_f + conj Z_{N-f}) / 2,  B_f = -i (Z_f - conj Z_{N-f}) / 2
                 const int64_t srow = (item * (int64_t)Spad + sA) * Fs;
@@ -786,35 +863,35 @@ k_raster_fft(RasterGeom geo, Loader ld, int64_t n_items, RasterOut out, FftRadix
                         if (XB == 2 && stg) {
                             const __half2 vr = __floats2half2_rn(ar * xsc, br * xsc);
                             const __half2 vi = __floats2half2_rn(ai * xsc, bi * xsc);
-                            stage[f * kFftStageWords + pw] = *reinterpret_cast<const uint32_t*>(&vr);
-                            stage[(F + f) * kFftStageWords + pw] = *reinterpret_cast<const uint32_t*>(&vi);
+                            stg_to[f * kFftStageWords + pw] = *reinterpret_cast<const uint32_t*>(&vr);
+                            stg_to[(F + f) * kFftStageWords + pw] = *reinterpret_cast<const uint32_t*>(&vi);
                         } else if (XB == 1 && stg) {
                             const __nv_bfloat162 vr = __floats2bfloat162_rn(ar, br);
                             const __nv_bfloat162 vi = __floats2bfloat162_rn(ai, bi);
-                            stage[f * kFftStageWords + pw] = *reinterpret_cast<const uint32_t*>(&vr);
-                            stage[(F + f) * kFftStageWords + pw] = *reinterpret_cast<const uint32_t*>(&vi);
+                            stg_to[f * kFftStageWords + pw] = *reinterpret_cast<const uint32_t*>(&vr);
+                            stg_to[(F + f) * kFftStageWords + pw] = *reinterpret_cast<const uint32_t*>(&vi);
                         }
                     }
                 }
                 __syncwarp();
             }
-            if (stg) {
-                // the tile's BF16 copy in the tensor-core layout (64-pattern tiles whose
-                // 16-row groups hold 8 patterns' real rows, then their imaginary rows):
-                // 32 bytes (16 shells) per row
-                __syncthreads();
-                const int64_t tile = item / 64, r = item % 64;
-                const int64_t rbase = (r >> 3) * 16 + (r & 7);
-                for (int e = threadIdx.x; e < 2 * F * 2; e += blockDim.x) {
-                    const int row = e >> 1, q = e & 1;
-                    const int c = row >= F, f = row - c * F;
-                    const uint32_t* src = stage + row * kFftStageWords + 4 * q;
-                    const uint4 v = make_uint4(src[0], src[1], src[2], src[3]);
-                    const int64_t grow = ((int64_t)f * ld.xb_tiles() + tile) * 128 + rbase + c * 8;
-                    *reinterpret_cast<uint4*>(xb + grow * Spad + t0 + 8 * q) = v;
+            if (XB != 0 && stg) {
+                if (dbl) {                           // (the warp's lanes synced above)
+                    if (lane == 0) tile_arrive(tile_bar + (staged & 1));
+                    out_t0 = t0;
+                    ++staged;
+                } else {
+                    __syncthreads();
+                    copy_tile(stage, t0);
+                    __syncthreads();
                 }
-                __syncthreads();
             }
+        }
+        if (XB != 0 && out_t0 >= 0) {
+            const int pb = (staged - 1) & 1;
+            tile_wait(tile_bar + pb, (tile_ph >> pb) & 1u);
+            tile_ph ^= 1u << pb;
+            copy_tile(pb ? stage2 : stage, out_t0);
         }
         if (w_lo < w_hi) {
             atomicMin(&s_int[40], w_lo);

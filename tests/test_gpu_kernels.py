@@ -175,3 +175,33 @@ def test_fp16_pairs_are_no_less_accurate_than_fp32(geometry):
     off = lambda u: float((u.double() - want).norm())
     assert off(pairs) <= off(cores)
     plan.close()
+
+
+@pytest.mark.parametrize("geometry", [(6.0, 150, 0.01, 360), (6.0, 75, 0.02, 180)], ids=str)
+@pytest.mark.parametrize("precision", [1, 2], ids=["bf16", "fp16"])
+def test_sixteen_bit_copies_with_one_and_two_staging_buffers(geometry, precision):
+    """Patterns of few and of many peaks in turn in the same CTAs (a second staging
+    buffer fits behind 178 peaks at 360 bins, 478 at 180): each pattern's bounds are
+    those it has alone with others of its kind."""
+    import torch
+    rng = np.random.default_rng(5)
+    counts = np.array([20, 600, 178, 179, 478, 479, 0, 1000, 3] * 120)
+    rp = np.zeros(len(counts) + 1, np.int64)
+    np.cumsum(counts, out=rp[1:])
+    r, t = rng.uniform(0.1, 1.45, rp[-1]), rng.uniform(-np.pi, np.pi, rp[-1])
+    scan = synth.Scan(rp, (r * np.cos(t)).astype(np.float32), (r * np.sin(t)).astype(np.float32),
+                      rng.lognormal(0.0, 1.0, rp[-1]).astype(np.float32),
+                      np.tile(np.eye(3), (len(counts), 1, 1)), np.zeros(len(counts), np.int32),
+                      (synth.au_fcc(),), "few and many peaks")
+    plan = au_plan(*geometry, precision=precision)
+    peaks = to_dev(scan)
+    want, scale = bounds64(plan, peaks)
+    S, F = math.ceil(geometry[1] / 32) * 32, geometry[3] // 2 + 1
+    tol = (2.0 ** -6 + (3 * (S + 2) + 2 * F) * 2.0 ** -21) * scale
+    got = plan.bounds(*peaks)
+    assert ((got.double() - want).abs() <= tol[:, None]).all()
+    # the same values whichever buffers the pattern's neighbours used
+    few = np.nonzero(counts <= 178)[0]
+    alone = plan.bounds(*to_dev(scan.subset(few)))
+    assert torch.equal(got[torch.from_numpy(few).cuda()], alone)
+    plan.close()
