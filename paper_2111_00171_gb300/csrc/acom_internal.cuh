@@ -80,6 +80,8 @@ struct PatternSource {         // one chunk of CSR patterns
     float gamma_pow, omega;
     int xb_fp16 = 0;           // xb holds FP16 of 2^e_b X^ instead of BF16 of X^
     float* xscale = nullptr;   // [n_items] 2^e_b of each pattern (with xb_fp16, or without xb)
+    int* tickets = nullptr;    // patterns taken so far by all launches (or nullptr: fixed
+    int taken = 0;             // shares), and its value when this launch starts
     int xb_k0 = 0;             // the contraction reads xb from this shell on: 16-shell
                                // tiles wholly below it are not written
 };
@@ -134,7 +136,8 @@ struct Workspace {
     int PTs = 0;                   // pattern tiles of 64 in XB
     alignas(64) unsigned char map_x[128];   // TMA map of XB
     float* xfn = nullptr;          // [chunk][F] ||X^_bf|| over shells
-    int* n_eval = nullptr;         // [2] axes evaluated exactly in the last match, patterns taken
+    int* n_eval = nullptr;         // [3] axes evaluated exactly in the last match, patterns taken
+                                   // by select and by the raster
     int2* srange = nullptr;        // [chunk] non-zero shell range of each pattern
     uint32_t* rmask = nullptr;     // [chunk][Spad / 32] shells each pattern's tents reach
     unsigned long long* best = nullptr;  // [chunk] packed (score, index)

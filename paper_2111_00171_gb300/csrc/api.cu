@@ -193,7 +193,7 @@ static acom_status ensure_ws(acom_plan_s* p, Workspace& ws, int chunk, bool need
     if ((e = dalloc(&ws.U, (size_t)chunk * p->Z, &acc, st)) != cudaSuccess) goto fail;
     if ((e = dalloc(&ws.extra, split_extra_floats(), &acc, st)) != cudaSuccess) goto fail;
     if ((e = dalloc(&ws.xfn, (size_t)chunk * p->F, &acc, st)) != cudaSuccess) goto fail;
-    if ((e = dalloc(&ws.n_eval, (size_t)2, &acc, st)) != cudaSuccess) goto fail;
+    if ((e = dalloc(&ws.n_eval, (size_t)3, &acc, st)) != cudaSuccess) goto fail;
     if ((e = dalloc(&ws.srange, (size_t)chunk, &acc, st)) != cudaSuccess) goto fail;
     if ((e = dalloc(&ws.rmask, (size_t)chunk * (p->Spad / 32), &acc, st)) != cudaSuccess) goto fail;
     if ((e = dalloc(&ws.best, (size_t)chunk, &acc, st)) != cudaSuccess) goto fail;
@@ -848,7 +848,7 @@ static acom_status match_enqueue(acom_plan p, const acom_peaks_csr* peaks,
     s = ensure_workspace(p, chunk, exhaustive, fp32_contraction, st);
     if (s != ACOM_OK) return s;
     cudaMemsetAsync(p->err, 0, sizeof(int), st);
-    cudaMemsetAsync(p->ws.n_eval, 0, 2 * sizeof(int), st);
+    cudaMemsetAsync(p->ws.n_eval, 0, 3 * sizeof(int), st);
     int taken = 0;
     launch_check_row0(peaks->row_ptr, p->err, st);
     RasterGeom geo{p->S, p->Spad, p->N, p->F, (float)p->dq, (float)p->delta, (float)p->gamma_pow, 0};
@@ -861,7 +861,10 @@ static acom_status match_enqueue(acom_plan p, const acom_peaks_csr* peaks,
         float* xscale = tc && p->precision != ACOM_PREC_BF16 ? w.xscale : nullptr;
         PatternSource src{tc ? w.XB : nullptr, w.PTs, peaks->row_ptr + c0, peaks->qx,
                           peaks->qy, peaks->I, nb, (float)p->gamma_pow, (float)p->omega,
-                          xscale ? 1 : 0, pairs16 ? w.xscale : xscale, p->k0};
+                          xscale ? 1 : 0, pairs16 ? w.xscale : xscale};
+        src.xb_k0 = p->k0;
+        src.tickets = w.n_eval + 2;
+        src.taken = (int)c0;
         RasterOut ro;
         ro.re = exhaustive ? w.Xr : nullptr;
         ro.im = exhaustive ? w.Xi : nullptr;
@@ -985,7 +988,8 @@ acom_status acom_bounds(acom_plan p, const acom_peaks_csr* peaks, float* dst, vo
         float* xscale = tc && p->precision != ACOM_PREC_BF16 ? p->ws.xscale : nullptr;
         PatternSource src{tc ? p->ws.XB : nullptr, p->ws.PTs, peaks->row_ptr + c0, peaks->qx,
                           peaks->qy, peaks->I, nb, (float)p->gamma_pow, (float)p->omega,
-                          xscale ? 1 : 0, pairs16 ? p->ws.xscale : xscale, p->k0};
+                          xscale ? 1 : 0, pairs16 ? p->ws.xscale : xscale};
+        src.xb_k0 = p->k0;
         RasterOut ro;
         if (!tc) {
             ro.sre = p->ws.Xsr;

@@ -77,6 +77,11 @@ struct PatternLoader {
     __host__ __device__ bool xb_half() const { return src.xb_fp16 != 0; }
     __device__ float* xscale_out() const { return src.xscale; }
     __device__ int xb_k0() const { return src.xb_k0; }
+    // the CTA's item after this one (thread 0, once an item)
+    __device__ int64_t next(int64_t item) const {
+        return src.tickets ? gridDim.x + (int64_t)(atomicAdd(src.tickets, 1) - src.taken)
+                           : item + gridDim.x;
+    }
     __device__ int load(int64_t item, PeakXY* sp, int* s_warp, int* err) const {
         const int64_t b0 = src.row_ptr[item];
         const int64_t b1 = src.row_ptr[item + 1];
@@ -118,6 +123,7 @@ struct PlanLoader {
     __host__ __device__ bool xb_half() const { return false; }
     __device__ float* xscale_out() const { return nullptr; }
     __device__ int xb_k0() const { return 0; }
+    __device__ int64_t next(int64_t item) const { return item + gridDim.x; }
     __device__ int load(int64_t item, Peak* sp, int* s_warp, int* err) const {
         const double* R = src.frames + 9 * item;
         double R00 = R[0], R01 = R[1], R02 = R[2], R10 = R[3], R11 = R[4], R12 = R[5],
@@ -588,7 +594,9 @@ k_raster_fft(RasterGeom geo, Loader ld, int64_t n_items, RasterOut out, FftRadix
     float2* zz = zt + warp * N;
     __nv_bfloat16* xb = XB ? reinterpret_cast<__nv_bfloat16*>(ld.xb_out()) : nullptr;
 
-    for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
+    // patterns differ several-fold in their peaks: a CTA takes the next one not yet taken
+    int64_t* s_next = reinterpret_cast<int64_t*>(s_int + 36);
+    for (int64_t item = blockIdx.x; item < n_items; item = *s_next) {
         const int np = ld.load(item, sp, s_int, err);
         // rank sort by (radius, index), in place: every thread holds its peaks
         // and their ranks in registers across the barrier, then stores them
@@ -618,6 +626,7 @@ k_raster_fft(RasterGeom geo, Loader ld, int64_t n_items, RasterOut out, FftRadix
         if (threadIdx.x == 0) {
             s_int[40] = Spad;
             s_int[41] = 0;
+            *s_next = ld.next(item);
         }
         if (threadIdx.x < 16) s_int[16 + threadIdx.x] = 0;    // shells the tents reach
         __syncthreads();

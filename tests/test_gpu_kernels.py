@@ -182,7 +182,7 @@ def test_fp16_pairs_are_no_less_accurate_than_fp32(geometry):
 def test_sixteen_bit_copies_with_one_and_two_staging_buffers(geometry, precision):
     """Patterns of few and of many peaks in turn in the same CTAs (a second staging
     buffer fits behind 178 peaks at 360 bins, 478 at 180): each pattern's bounds are
-    those it has alone with others of its kind."""
+    those it has among patterns of its kind."""
     import torch
     rng = np.random.default_rng(5)
     counts = np.array([20, 600, 178, 179, 478, 479, 0, 1000, 3] * 120)
@@ -200,8 +200,9 @@ def test_sixteen_bit_copies_with_one_and_two_staging_buffers(geometry, precision
     tol = (2.0 ** -6 + (3 * (S + 2) + 2 * F) * 2.0 ** -21) * scale
     got = plan.bounds(*peaks)
     assert ((got.double() - want).abs() <= tol[:, None]).all()
-    # the same values whichever buffers the pattern's neighbours used
+    # the same terms whichever buffers the pattern's neighbours used; a batch of another
+    # size may sum the frequencies in other groups, F terms in FP32
     few = np.nonzero(counts <= 178)[0]
     alone = plan.bounds(*to_dev(scan.subset(few)))
-    assert torch.equal(got[torch.from_numpy(few).cuda()], alone)
+    assert ((got[torch.from_numpy(few).cuda()] - alone).abs() <= F * 2.0 ** -23 * alone).all()
     plan.close()
