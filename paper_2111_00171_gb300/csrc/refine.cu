@@ -41,6 +41,7 @@ constexpr int kRefWarps = 8;                    // patterns per block
 constexpr int kRefPeakSmem = 128;               // peaks per pattern kept in shared memory
 constexpr float kExcCut = 18.0f;                // skip when s^2 / (2 sigma_e^2) > kExcCut
 constexpr int kRefActCap = 512;                 // contributing reflections listed at a time
+constexpr int kRefRhos = 64;                    // spot widths kept per block
 
 struct RefArgs {
     const float4* refl;        // [G] (g_x, g_y, g_z, |g|^gamma |F_g|^omega)
@@ -226,14 +227,20 @@ __device__ void score_at(const RefArgs& a, const float R[9], const float e[6], f
     const float l2_half_inv_r2 = 0.5f * inv_r2 * 1.4426950408889634f;
     const bool exc = a.omega > 0.0f;
     const float inv_se2 = exc ? 1.0f / a.se2 : 0.0f;
+    const float k2 = a.inv_lam * a.inv_lam;
+    const float wide = exc ? 8.0f * 1.03f * kExcCut * a.se2 : 0.0f;
     Acc acc{};
     for (int c0 = 0; c0 < a.G; c0 += kRefActCap) {
-        // list the contributing reflections of [c0, c0 + kRefActCap)
+        // list the contributing reflections of [c0, c0 + kRefActCap): first those a
+        // bound without a root or a quotient cannot rule out (with t = |k + v|^2 - |k|^2,
+        // |s| = |t| / 2|k + v| and |k + v|^2 = |k|^2 + t: t^2 <= 8 cut sigma_e^2 |k + v|^2,
+        // 3 % and ten times the rounding of t wider than the cut), then of those the ones
+        // inside the cut; both in order
         int n = 0;
         const int c1 = c0 + kRefActCap < a.G ? c0 + kRefActCap : a.G;
         for (int g0 = c0; g0 < c1; g0 += 32) {
             const int gi = g0 + lane;
-            bool active = false;
+            bool near = false;
             if (gi < c1) {
                 const float4 g = __ldg(a.refl + gi);
                 float gx = g.x, gy = g.y, gz = g.z;
@@ -241,15 +248,39 @@ __device__ void score_at(const RefArgs& a, const float R[9], const float e[6], f
                 const float vx = R[0] * gx + R[1] * gy + R[2] * gz;
                 const float vy = R[3] * gx + R[4] * gy + R[5] * gz;
                 const float vz = R[6] * gx + R[7] * gy + R[8] * gz;
-                const float v2 = vx * vx + vy * vy + vz * vz;
-                const float kz = vz - a.inv_lam;
-                const float nkv = sqrtf(vx * vx + vy * vy + kz * kz);
-                const float s = -(v2 - 2.0f * vz * a.inv_lam) / (2.0f * nkv);
-                active = g.w > 0.0f && (!exc || 0.5f * s * s * inv_se2 <= kExcCut);
+                const float v2 = vx * vx + vy * vy + vz * vz, l = 2.0f * vz * a.inv_lam;
+                const float t = v2 - l, tau = 9.5367432e-7f * (v2 + fabsf(l));   // 2^-20
+                near = g.w > 0.0f && (!exc || !(t * t > fmaf(wide, k2 + t, 100.0f * tau * tau)));
             }
-            const unsigned mask = __ballot_sync(0xffffffffu, active);
-            if (active) act[n + __popc(mask & ((1u << lane) - 1u))] = gi;
+            const unsigned mask = __ballot_sync(0xffffffffu, near);
+            if (near) act[n + __popc(mask & ((1u << lane) - 1u))] = gi;
             n += __popc(mask);
+        }
+        __syncwarp();
+        if (exc) {
+            const int m = n;
+            n = 0;
+            for (int j0 = 0; j0 < m; j0 += 32) {
+                const int gi = j0 + lane < m ? act[j0 + lane] : -1;
+                bool active = false;
+                if (gi >= 0) {
+                    const float4 g = __ldg(a.refl + gi);
+                    float gx = g.x, gy = g.y, gz = g.z;
+                    if (STRAIN) strained(e, gx, gy, gz);
+                    const float vx = R[0] * gx + R[1] * gy + R[2] * gz;
+                    const float vy = R[3] * gx + R[4] * gy + R[5] * gz;
+                    const float vz = R[6] * gx + R[7] * gy + R[8] * gz;
+                    const float v2 = vx * vx + vy * vy + vz * vz;
+                    const float kz = vz - a.inv_lam;
+                    const float nkv = sqrtf(vx * vx + vy * vy + kz * kz);
+                    const float s = -(v2 - 2.0f * vz * a.inv_lam) / (2.0f * nkv);
+                    active = 0.5f * s * s * inv_se2 <= kExcCut;
+                }
+                const unsigned mask = __ballot_sync(0xffffffffu, active);
+                if (active) act[n + __popc(mask & ((1u << lane) - 1u))] = gi;
+                n += __popc(mask);
+                __syncwarp();
+            }
         }
         __syncwarp();
         if (a.pairs && lane == 0) atomicAdd(a.pairs, (unsigned long long)n * (unsigned long long)M);
@@ -382,20 +413,24 @@ __device__ __forceinline__ void load9(const float* Rf, float R[9]) {
     for (int i = 0; i < 9; ++i) R[i] = Rf[i];
 }
 
+// Spot width of step t.
+__device__ __forceinline__ float step_rho(const RefArgs& a, int t) {
+    return a.steps > 1 ? a.rho_start * powf(a.rho_end / a.rho_start, (float)t / (float)(a.steps - 1))
+                       : a.rho_end;
+}
+
 // One refinement run from Rd (FP64 in the warp's shared memory, with its FP32
 // copy Rf).  Every lane holds the same score, gradient and matrix, so every
 // lane takes the same step; lanes 0..8 compose one element of Exp(w) Rd each
 // in FP64 (FP64 instructions are scarce on this GPU: nine lanes issue three
 // multiply-adds where one lane issued a hundred).
 __device__ float refine_run(const RefArgs& a, double* Rd, float* Rf, int64_t p0, int M,
-                            const float* px, const float* py, const float* pa, int* act) {
+                            const float* px, const float* py, const float* pa, int* act,
+                            const float* rhos) {
     const int lane = threadIdx.x & 31;
     float R[9], S, g[3], H[6];
     for (int t = 0; t < a.steps; ++t) {
-        const float rho = a.steps > 1
-                              ? a.rho_start * powf(a.rho_end / a.rho_start,
-                                                   (float)t / (float)(a.steps - 1))
-                              : a.rho_end;
+        const float rho = t < kRefRhos ? rhos[t] : step_rho(a, t);
         load9(Rf, R);
         score_at<false>(a, R, nullptr, rho, p0, M, px, py, pa, act, S, g, H, nullptr);
         float w[3], E[9];
@@ -455,6 +490,9 @@ __global__ void __launch_bounds__(kRefWarps * 32, 3) k_refine(RefArgs a) {
     __shared__ int s_act[kRefWarps][kRefActCap];
     __shared__ double s_R[kRefWarps][2][9];
     __shared__ float s_Rf[kRefWarps][9];
+    __shared__ float s_rho[kRefRhos];
+    for (int t = threadIdx.x; t < a.steps && t < kRefRhos; t += blockDim.x) s_rho[t] = step_rho(a, t);
+    __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float* px = s_px[warp];
     float* py = s_py[warp];
@@ -485,7 +523,7 @@ __global__ void __launch_bounds__(kRefWarps * 32, 3) k_refine(RefArgs a) {
                 Rc[lane] = (double)r;
                 s_Rf[warp][lane] = r;
             }
-            const float S = refine_run(a, Rc, s_Rf[warp], p0, M, px, py, pa, act);
+            const float S = refine_run(a, Rc, s_Rf[warp], p0, M, px, py, pa, act, s_rho);
             __syncwarp();
             if (S > best || st == 0) {
                 best = S;
@@ -504,71 +542,86 @@ __global__ void __launch_bounds__(kRefWarps * 32, 3) k_refine(RefArgs a) {
     }
 }
 
-// Score, gradient dS/dr and Gauss-Newton matrix at R = Exp(r) m^T.
+// Left Jacobian of SO(3), J = I + (1 - cos t)/t^2 K + (t - sin t)/t^3 K^2; below 0.05
+// rad the factors by their series (remainder under 1e-12).
+__device__ void jacobian_so3(const double r[3], double J[9]) {
+    const double t2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
+    double A, B;
+    if (t2 < 0.0025) {
+        A = 0.5 - t2 * (1.0 / 24.0 - t2 * (1.0 / 720.0));
+        B = 1.0 / 6.0 - t2 * (1.0 / 120.0 - t2 * (1.0 / 5040.0));
+    } else {
+        const double t = sqrt(t2);
+        A = (1.0 - cos(t)) / t2;
+        B = (t - sin(t)) / (t2 * t);
+    }
+    const double K[9] = {0, -r[2], r[1], r[2], 0, -r[0], -r[1], r[0], 0};
+    for (int i = 0; i < 3; ++i)
+        for (int j = 0; j < 3; ++j) {
+            double k2 = 0;
+            for (int l = 0; l < 3; ++l) k2 += K[3 * i + l] * K[3 * l + j];
+            J[3 * i + j] = (i == j ? 1.0 : 0.0) + A * K[3 * i + j] + B * k2;
+        }
+}
+
+// Score, gradient dS/dr and Gauss-Newton matrix at R = Exp(r) m^T, a warp per
+// pattern.  The FP64 rotations and Jacobians of the block's patterns are taken by
+// one warp, a lane each: an FP64 instruction occupies the scarce FP64 pipe for a
+// whole warp whether one lane needs it or eight.  STRAIN: a strain or its gradient
+// is asked for (else twelve of the sums and their reductions fall away).  4,000
+// patterns: 78 -> 37 us.
+template <bool STRAIN>
 __global__ void __launch_bounds__(kRefWarps * 32) k_kin_score(RefArgs a) {
     __shared__ float s_px[kRefWarps][kRefPeakSmem], s_py[kRefWarps][kRefPeakSmem],
         s_pa[kRefWarps][kRefPeakSmem];
     __shared__ int s_act[kRefWarps][kRefActCap];
-    __shared__ double s_R[kRefWarps][9];
+    __shared__ float s_R[kRefWarps][9];
+    __shared__ double s_J[kRefWarps][9];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float* px = s_px[warp];
     float* py = s_py[warp];
     float* pa = s_pa[warp];
     int* act = s_act[warp];
-    double* Rd = s_R[warp];
-    for (int64_t b = (int64_t)blockIdx.x * kRefWarps + warp; b < a.nb;
-         b += (int64_t)gridDim.x * kRefWarps) {
-        int64_t p0;
-        __syncwarp();
-        const int M = load_peaks(a, b, p0, px, py, pa);
-        if (M < 0) continue;
-        double r[3] = {0, 0, 0};
-        if (lane == 0) {
-            double M0[9];
+    for (int64_t b0 = (int64_t)blockIdx.x * kRefWarps; b0 < a.nb;
+         b0 += (int64_t)gridDim.x * kRefWarps) {
+        const int64_t b = b0 + warp;
+        __syncthreads();
+        // the last warp's lanes take a pattern each, the other warps load peaks meanwhile
+        if (warp == kRefWarps - 1 && lane < kRefWarps && b0 + lane < a.nb) {
+            const int64_t bl = b0 + lane;
+            double r[3] = {0, 0, 0}, M0[9], E[9];
             for (int i = 0; i < 3; ++i)
-                for (int j = 0; j < 3; ++j) M0[3 * i + j] = (double)a.orient[9 * b + 3 * j + i];
+                for (int j = 0; j < 3; ++j) M0[3 * i + j] = (double)a.orient[9 * bl + 3 * j + i];
             if (a.r)
-                for (int i = 0; i < 3; ++i) r[i] = a.r[3 * b + i];
-            double E[9];
+                for (int i = 0; i < 3; ++i) r[i] = a.r[3 * bl + i];
             exp_so3(r, E);
             for (int i = 0; i < 3; ++i)
                 for (int j = 0; j < 3; ++j)
-                    Rd[3 * i + j] = E[3 * i] * M0[j] + E[3 * i + 1] * M0[3 + j] +
-                                    E[3 * i + 2] * M0[6 + j];
+                    s_R[lane][3 * i + j] = (float)(E[3 * i] * M0[j] + E[3 * i + 1] * M0[3 + j] +
+                                                   E[3 * i + 2] * M0[6 + j]);
+            if (a.grad) jacobian_so3(r, s_J[lane]);
         }
+        int64_t p0 = 0;
+        const int M = b < a.nb ? load_peaks(a, b, p0, px, py, pa) : -1;
+        __syncthreads();
+        if (M < 0) continue;
         float R[9], S, g[3], H[6], e[6], de[6];
-        __syncwarp();
-        for (int i = 0; i < 9; ++i) R[i] = (float)Rd[i];
-        for (int i = 0; i < 6; ++i) e[i] = a.strain ? a.strain[6 * b + i] : 0.0f;
-        score_at<true>(a, R, e, a.rho, p0, M, px, py, pa, act, S, g, H, de);
+        for (int i = 0; i < 9; ++i) R[i] = s_R[warp][i];
+        if (STRAIN)
+            for (int i = 0; i < 6; ++i) e[i] = a.strain ? a.strain[6 * b + i] : 0.0f;
+        score_at<STRAIN>(a, R, e, a.rho, p0, M, px, py, pa, act, S, g, H, de);
+        if (lane == 0 && a.score) a.score[b] = S;
+        if (a.grad && lane < 3) {
+            // dS/dr = J(r)^T dS/dw
+            const double* J = s_J[warp];
+            double acc = 0;
+            for (int i = 0; i < 3; ++i) acc += J[3 * i + lane] * (double)g[i];
+            a.grad[3 * b + lane] = (float)acc;
+        }
         if (lane == 0) {
-            if (a.score) a.score[b] = S;
-            if (a.grad) {
-                // dS/dr = J(r)^T dS/dw, J = I + (1 - cos t)/t^2 K + (t - sin t)/t^3 K^2
-                const double t = sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
-                double A, B;
-                if (t < 1e-6) {
-                    A = 0.5;
-                    B = 1.0 / 6.0;
-                } else {
-                    A = (1.0 - cos(t)) / (t * t);
-                    B = (t - sin(t)) / (t * t * t);
-                }
-                const double K[9] = {0, -r[2], r[1], r[2], 0, -r[0], -r[1], r[0], 0};
-                for (int j = 0; j < 3; ++j) {
-                    double acc = 0;
-                    for (int i = 0; i < 3; ++i) {
-                        double k2 = 0;
-                        for (int l = 0; l < 3; ++l) k2 += K[3 * i + l] * K[3 * l + j];
-                        const double Jij = (i == j ? 1.0 : 0.0) + A * K[3 * i + j] + B * k2;
-                        acc += Jij * (double)g[i];
-                    }
-                    a.grad[3 * b + j] = (float)acc;
-                }
-            }
             if (a.gn)
                 for (int i = 0; i < 6; ++i) a.gn[6 * b + i] = H[i];
-            if (a.strain_grad)
+            if (STRAIN && a.strain_grad)
                 for (int i = 0; i < 6; ++i) a.strain_grad[6 * b + i] = de[i];
         }
     }
@@ -668,7 +721,10 @@ void launch_kin_score(const acom_plan_s* p, const acom_peaks_csr* pk, const floa
     const int grid = ref_grid(pk->n_patterns);
     if (grid <= 0) return;
     prof_begin(kKRefineOrient, st);
-    k_kin_score<<<grid, kRefWarps * 32, 0, st>>>(a);
+    if (strain || strain_grad)
+        k_kin_score<true><<<grid, kRefWarps * 32, 0, st>>>(a);
+    else
+        k_kin_score<false><<<grid, kRefWarps * 32, 0, st>>>(a);
     prof_end(kKRefineOrient, st);
 }
 

@@ -206,3 +206,33 @@ def test_sixteen_bit_copies_with_one_and_two_staging_buffers(geometry, precision
     alone = plan.bounds(*to_dev(scan.subset(few)))
     assert ((got[torch.from_numpy(few).cuda()] - alone).abs() <= F * 2.0 ** -23 * alone).all()
     plan.close()
+
+
+@pytest.mark.parametrize("sigma", [1e-6, 0.02, 0.3])
+def test_kinematical_score_reflection_list(sigma):
+    """The reflections that contribute are found in two steps (a bound, then the cut):
+    scores and gradients at shape factors from far narrower than the rounding of an
+    excitation error to wider than all reflections, for a last block that is not full,
+    against FP64 autograd of the definition."""
+    import torch
+    from paper_2111_00171_gb300 import acom
+    from oracle import acom_oracle as O
+    from gpu_common import au_refl
+    tri, area = acom.cubic_triangle()
+    plan = acom.Plan(acom.au_crystal(), tri, area, 6.0, 40, 0.0375, 72, lam=LAM, sigma_exc=sigma)
+    scan = synth.random_patterns(21, n_patterns=13)
+    m = torch.from_numpy(scan.truth.astype(np.float32)).cuda()
+    s, g, _ = plan.kinematical_score(*to_dev(scan), m, rho=0.05)
+    refl = au_refl()
+    for b in range(scan.n_patterns):
+        want = O.kinematical_score(scan.truth[b].astype(np.float32).astype(np.float64).T,
+                                   *scan.pattern(b), refl, LAM, sigma, 0.05)
+        if sigma < 1e-3:
+            # at such a width FP32 excitation errors decide at random; finite and no larger
+            # than the peaks' weights allow
+            assert math.isfinite(float(s[b])) and torch.isfinite(g[b]).all()
+            continue
+        assert float(s[b]) == pytest.approx(want.S, rel=1e-4), b
+        np.testing.assert_allclose(g[b].cpu().numpy(), want.grad, rtol=0,
+                                   atol=1e-3 * np.abs(want.grad).max(), err_msg=str(b))
+    plan.close()
