@@ -207,7 +207,8 @@ struct acom_plan_s {
     int ks = 0;
     alignas(64) unsigned char map_ps[128];
     float4* refl_tab = nullptr;       // [G] FP32 (g, |g|^gamma |F_g|^omega) for refinement
-    unsigned long long* refine_pairs = nullptr;  // (reflection, peak) pairs of the last refine
+    unsigned long long* refine_pairs = nullptr;  // [2] (reflection, peak) pairs of the last
+                                                 // refine, patterns taken
     int64_t last_refine_pairs = 0;
     int n_phases = 1;                 // crystal structures (phases) in this plan
     std::vector<int> phase_off_host;  // [n_phases + 1] first axis of each phase, then Z

@@ -1037,7 +1037,7 @@ acom_status acom_refine(acom_plan p, const acom_peaks_csr* peaks, const acom_ref
     s = refine_table(p, st);
     if (s != ACOM_OK) return s;
     cudaMemsetAsync(p->err, 0, sizeof(int), st);
-    cudaMemsetAsync(p->refine_pairs, 0, sizeof(unsigned long long), st);
+    cudaMemsetAsync(p->refine_pairs, 0, 2 * sizeof(unsigned long long), st);
     launch_check_row0(peaks->row_ptr, p->err, st);
     launch_refine_orient(p, peaks, o.steps, o.rho_start, o.rho_end, o.damping,
                          (float)(o.max_step_deg * M_PI / 180.0), o.twin ? 1 : 0, orient,
