@@ -415,17 +415,6 @@ acom_status acom_plan_create(const acom_crystal* crystal, const acom_za_grid* gr
 
     std::vector<double> frames(9 * (size_t)Z);
     for (int z = 0; z < Z; ++z) za_frame(&za[3 * z], &frames[9 * z]);
-    // grid neighbours: axes within 1.5 steps
-    std::vector<int> nptr(Z + 1, 0), nidx;
-    const double lim = std::cos(1.5 * grid->step_deg * M_PI / 180.0);
-    for (int z = 0; z < Z; ++z) {
-        for (int z2 = 0; z2 < Z; ++z2) {
-            double c = za[3 * z] * za[3 * z2] + za[3 * z + 1] * za[3 * z2 + 1] +
-                       za[3 * z + 2] * za[3 * z2 + 2];
-            if (c >= lim) nidx.push_back(z2);
-        }
-        nptr[z + 1] = (int)nidx.size();
-    }
 
     cudaError_t e = cudaSuccess;
     acom_status s;
@@ -442,8 +431,7 @@ acom_status acom_plan_create(const acom_crystal* crystal, const acom_za_grid* gr
     ACOM_CK(dalloc(&p->Psi, selems, &p->bytes, st));
     ACOM_CK(dalloc(&p->za, za.size(), &p->bytes, st));
     ACOM_CK(dalloc(&p->frames, frames.size(), &p->bytes, st));
-    ACOM_CK(dalloc(&p->nbr_ptr, nptr.size(), &p->bytes, st));
-    ACOM_CK(dalloc(&p->nbr_idx, nidx.size(), &p->bytes, st));
+    ACOM_CK(dalloc(&p->nbr_ptr, (size_t)Z + 1, &p->bytes, st));
     ACOM_CK(dalloc(&p->err, 1, &p->bytes, st));
     ACOM_CK(dalloc(&p->pfmax, (size_t)p->F, &p->bytes, st));
     p->phase_off_host = {0, Z};
@@ -465,10 +453,6 @@ acom_status acom_plan_create(const acom_crystal* crystal, const acom_za_grid* gr
     ACOM_CK(cudaMemsetAsync(p->err, 0, sizeof(int), st));
     ACOM_CK(cudaMemcpyAsync(p->za, za.data(), sizeof(double) * za.size(), cudaMemcpyHostToDevice, st));
     ACOM_CK(cudaMemcpyAsync(p->frames, frames.data(), sizeof(double) * frames.size(),
-                            cudaMemcpyHostToDevice, st));
-    ACOM_CK(cudaMemcpyAsync(p->nbr_ptr, nptr.data(), sizeof(int) * nptr.size(),
-                            cudaMemcpyHostToDevice, st));
-    ACOM_CK(cudaMemcpyAsync(p->nbr_idx, nidx.data(), sizeof(int) * nidx.size(),
                             cudaMemcpyHostToDevice, st));
     s = build_plan_device(p, crystal, st);
     if (s != ACOM_OK) {

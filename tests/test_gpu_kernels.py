@@ -236,3 +236,28 @@ def test_kinematical_score_reflection_list(sigma):
         np.testing.assert_allclose(g[b].cpu().numpy(), want.grad, rtol=0,
                                    atol=1e-3 * np.abs(want.grad).max(), err_msg=str(b))
     plan.close()
+
+
+@pytest.mark.parametrize("step", [45.0, 9.0, 2.0])
+def test_grid_neighbours(step):
+    """Neighbour lists of grids with fewer axes than a warp's lanes, some more, and several
+    hundred: the refined orientation, a mean over the listed axes, is the oracle's."""
+    from oracle import acom_oracle as O
+    from gpu_common import au_refl
+    v0, v1, v2, area = O.cubic_triangle()
+    za = O.zone_axis_grid(v0, v1, v2, step, area)
+    oplan = O.orientation_plan(au_refl(), za, O.PlanParams(40, 0.0375, 72, 0.08, lam=LAM))
+    plan = au_plan(step, 40, 0.0375, 72)
+    scan = synth.random_patterns(9, n_patterns=12)
+    r = plan.match(*to_dev(scan))
+    m = r["orient"].cpu().numpy()
+    same = 0
+    for b in range(scan.n_patterns):
+        mt = O.match_pattern(oplan, *scan.pattern(b))
+        if (int(r["za_idx"][b]), int(r["phi3_bin"][b]), int(r["mirror"][b])) != (mt.za, mt.k, mt.mirror):
+            continue                                            # a tie resolved the other way
+        same += 1
+        # FP32 scores weight the mean: 1e-5 relative, over a neighbourhood below 1.2 radians
+        np.testing.assert_allclose(m[b], O.refine(mt, za, step).m, atol=1e-4)
+    assert same > 0
+    plan.close()
