@@ -2,9 +2,9 @@
 //
 //   k_reflections   every lattice point 0 < |g| < q_max (Eq. 2) and its
 //                   structure factor F_hkl = sum_n f_n(|g|) exp(-2 pi i hkl.p_n)
-//                   (Eq. 3), in FP64, compacted in lexicographic (h, k, l)
-//                   order; reflections with |F| < 1e-9 max|F| are dropped
-//                   (V_g of Eq. 4 is zero there).
+//                   (Eq. 3), in FP64.
+//   k_compact_reflections  those with |F| >= 1e-9 max|F| (V_g of Eq. 4 is zero
+//                   below) in lexicographic (h, k, l) order.
 //   raster (raster.cu, PlanLoader)  P0 per zone axis and its Fourier
 //                   transform along phi3, plus ||P0||^2.
 //   k_plan_layouts (match_tc.cu)  P = A P0, A = 1/||P0||_2, in every layout.
@@ -30,108 +30,83 @@ struct ReflParams {
     int n_atoms;
 };
 
-constexpr int kReflThreads = 1024;
+constexpr int kReflThreads = 128, kCompactThreads = 1024;
 
-// Single CTA: the candidate box is at most a few hundred thousand points.
+// A thread per point of the index box: its g, |F| (-1 outside the sphere) and |F|^omega,
+// and the largest |F| in *fmax (non-negative doubles order like their bits).  Bound by
+// the FP64 rate, some 10^3 operations a point at 2 a clock and SM: in the single CTA that
+// also compacted, the 2,197 points of Au to 1.5 / A took 168 us; over the SMs, with the
+// compaction below, 30 us.
 __global__ void __launch_bounds__(kReflThreads)
 k_reflections(ReflParams prm, const double* __restrict__ atoms,  // [n][5]: px py pz A B
-              double* tmp_g, double* tmp_F, double* out_g, double* out_amp, int* out_count) {
-    __shared__ int s_warp[33];
-    __shared__ double s_max[32];
+              double* __restrict__ tmp_g, double* __restrict__ tmp_F,
+              double* __restrict__ tmp_amp, unsigned long long* fmax) {
     const int64_t n1w = 2 * prm.n1 + 1, n2w = 2 * prm.n2 + 1;
     const int64_t total = (int64_t)(2 * prm.n0 + 1) * n1w * n2w;
+    const int64_t idx = (int64_t)blockIdx.x * kReflThreads + threadIdx.x;
+    double absF = -1.0;
+    if (idx < total) {
+        int h = (int)(idx / (n1w * n2w)) - prm.n0;
+        int k = (int)((idx / n2w) % n1w) - prm.n1;
+        int l = (int)(idx % n2w) - prm.n2;
+        double gx = h * prm.rb[0] + k * prm.rb[3] + l * prm.rb[6];
+        double gy = h * prm.rb[1] + k * prm.rb[4] + l * prm.rb[7];
+        double gz = h * prm.rb[2] + k * prm.rb[5] + l * prm.rb[8];
+        double q = sqrt(gx * gx + gy * gy + gz * gz);
+        if ((q > 0.0) && (q < prm.q_max)) {
+            double re = 0.0, im = 0.0;
+            for (int n = 0; n < prm.n_atoms; ++n) {
+                const double* a = atoms + 5 * n;
+                double fn = a[3] * exp(-a[4] * q * q);
+                double ph = h * a[0] + k * a[1] + l * a[2];
+                double sn, cs;
+                sincospi(2.0 * ph, &sn, &cs);     // exp(-2 pi i ph)
+                re += fn * cs;
+                im -= fn * sn;
+            }
+            absF = sqrt(re * re + im * im);
+            tmp_g[3 * idx] = gx;
+            tmp_g[3 * idx + 1] = gy;
+            tmp_g[3 * idx + 2] = gz;
+            tmp_amp[idx] = pow(absF, prm.omega);
+        }
+        tmp_F[idx] = absF;
+    }
+    double m = absF > 0.0 ? absF : 0.0;
+    for (int o = 16; o > 0; o >>= 1) m = ::fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0 && m > 0.0) atomicMax(fmax, (unsigned long long)__double_as_longlong(m));
+}
+
+// Single CTA, one pass over the index box (at most 4M points), order kept.
+__global__ void __launch_bounds__(kCompactThreads)
+k_compact_reflections(int total, const double* __restrict__ tmp_g,
+                      const double* __restrict__ tmp_F, const double* __restrict__ tmp_amp,
+                      const unsigned long long* fmax, double* __restrict__ out_g,
+                      double* __restrict__ out_amp, int* out_count) {
+    __shared__ int s_warp[2][33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int count = 0;
-    double fmx = 0.0;
-    for (int64_t base = 0; base < total; base += blockDim.x) {
-        int64_t idx = base + threadIdx.x;
-        bool keep = false;
-        double gx = 0, gy = 0, gz = 0, absF = 0;
-        if (idx < total) {
-            int h = (int)(idx / (n1w * n2w)) - prm.n0;
-            int k = (int)((idx / n2w) % n1w) - prm.n1;
-            int l = (int)(idx % n2w) - prm.n2;
-            gx = h * prm.rb[0] + k * prm.rb[3] + l * prm.rb[6];
-            gy = h * prm.rb[1] + k * prm.rb[4] + l * prm.rb[7];
-            gz = h * prm.rb[2] + k * prm.rb[5] + l * prm.rb[8];
-            double q = sqrt(gx * gx + gy * gy + gz * gz);
-            keep = (q > 0.0) && (q < prm.q_max);
-            if (keep) {
-                double re = 0.0, im = 0.0;
-                for (int n = 0; n < prm.n_atoms; ++n) {
-                    const double* a = atoms + 5 * n;
-                    double fn = a[3] * exp(-a[4] * q * q);
-                    double ph = h * a[0] + k * a[1] + l * a[2];
-                    double sn, cs;
-                    sincospi(2.0 * ph, &sn, &cs);     // exp(-2 pi i ph)
-                    re += fn * cs;
-                    im -= fn * sn;
-                }
-                absF = sqrt(re * re + im * im);
-                fmx = fmx > absF ? fmx : absF;
-            }
-        }
-        unsigned m = __ballot_sync(0xffffffffu, keep);
-        if (lane == 0) s_warp[warp] = __popc(m);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int acc = 0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-                int c = s_warp[w];
-                s_warp[w] = acc;
-                acc += c;
-            }
-            s_warp[32] = acc;
-        }
-        __syncthreads();
-        if (keep) {
-            int pos = count + s_warp[warp] + __popc(m & ((1u << lane) - 1u));
-            tmp_g[3 * pos] = gx;
-            tmp_g[3 * pos + 1] = gy;
-            tmp_g[3 * pos + 2] = gz;
-            tmp_F[pos] = absF;
-        }
-        count += s_warp[32];
-        __syncthreads();
-    }
-    // block max of |F|
-    for (int o = 16; o > 0; o >>= 1) fmx = fmax(fmx, __shfl_xor_sync(0xffffffffu, fmx, o));
-    if (lane == 0) s_max[warp] = fmx;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double mm = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) mm = mm > s_max[w] ? mm : s_max[w];
-        s_max[0] = mm;
-    }
-    __syncthreads();
-    const double thr = 1e-9 * s_max[0];
-    // second pass: drop extinct reflections, keep order
+    const double thr = 1e-9 * __longlong_as_double((long long)*fmax);
     int out = 0;
-    for (int base = 0; base < count; base += blockDim.x) {
-        int i = base + threadIdx.x;
-        bool keep = (i < count) && (tmp_F[i] >= thr);
-        unsigned m = __ballot_sync(0xffffffffu, keep);
-        if (lane == 0) s_warp[warp] = __popc(m);
+    for (int base = 0, t = 0; base < total; base += kCompactThreads, t ^= 1) {
+        const int i = base + threadIdx.x;
+        const double f = i < total ? tmp_F[i] : -1.0;
+        const bool keep = f >= 0.0 && f >= thr;
+        const unsigned m = __ballot_sync(0xffffffffu, keep);
+        if (lane == 0) s_warp[t][warp] = __popc(m);
         __syncthreads();
-        if (threadIdx.x == 0) {
-            int acc = 0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-                int c = s_warp[w];
-                s_warp[w] = acc;
-                acc += c;
-            }
-            s_warp[32] = acc;
+        int before = 0, all = 0;
+        for (int w = 0; w < kCompactThreads / 32; ++w) {
+            before += w < warp ? s_warp[t][w] : 0;
+            all += s_warp[t][w];
         }
-        __syncthreads();
         if (keep) {
-            int pos = out + s_warp[warp] + __popc(m & ((1u << lane) - 1u));
+            const int pos = out + before + __popc(m & ((1u << lane) - 1u));
             out_g[3 * pos] = tmp_g[3 * i];
             out_g[3 * pos + 1] = tmp_g[3 * i + 1];
             out_g[3 * pos + 2] = tmp_g[3 * i + 2];
-            out_amp[pos] = pow(tmp_F[i], prm.omega);
+            out_amp[pos] = tmp_amp[i];
         }
-        out += s_warp[32];
-        __syncthreads();
+        out += all;
     }
     if (threadIdx.x == 0) *out_count = out;
 }
@@ -227,9 +202,9 @@ acom_status build_plan_device(acom_plan_s* p, const acom_crystal* cr, cudaStream
         atoms[5 * n + 3] = cr->ff_A[n];
         atoms[5 * n + 4] = cr->ff_B[n];
     }
-    double *d_atoms = nullptr, *d_tmp_g = nullptr, *d_tmp_F = nullptr, *d_g = nullptr,
-           *d_amp = nullptr;
-    int* d_cnt = nullptr;
+    double *d_atoms = nullptr, *d_tmp_g = nullptr, *d_tmp_F = nullptr, *d_tmp_amp = nullptr,
+           *d_g = nullptr, *d_amp = nullptr;
+    unsigned long long* d_cnt = nullptr;           // largest |F|, then the count
     cudaError_t e;
 #define ACOM_TRY(x)                                        \
     do {                                                   \
@@ -240,9 +215,11 @@ acom_status build_plan_device(acom_plan_s* p, const acom_crystal* cr, cudaStream
         ACOM_TRY(pool_alloc(reinterpret_cast<void**>(&d_atoms), sizeof(double) * atoms.size(), st));
         ACOM_TRY(pool_alloc(reinterpret_cast<void**>(&d_tmp_g), sizeof(double) * 3 * cand, st));
         ACOM_TRY(pool_alloc(reinterpret_cast<void**>(&d_tmp_F), sizeof(double) * cand, st));
+        ACOM_TRY(pool_alloc(reinterpret_cast<void**>(&d_tmp_amp), sizeof(double) * cand, st));
         ACOM_TRY(pool_alloc(reinterpret_cast<void**>(&d_g), sizeof(double) * 3 * cand, st));
         ACOM_TRY(pool_alloc(reinterpret_cast<void**>(&d_amp), sizeof(double) * cand, st));
-        ACOM_TRY(pool_alloc(reinterpret_cast<void**>(&d_cnt), sizeof(int), st));
+        ACOM_TRY(pool_alloc(reinterpret_cast<void**>(&d_cnt), 2 * sizeof(*d_cnt), st));
+        ACOM_TRY(cudaMemsetAsync(d_cnt, 0, 2 * sizeof(*d_cnt), st));
         ACOM_TRY(cudaMemcpyAsync(d_atoms, atoms.data(), sizeof(double) * atoms.size(),
                                  cudaMemcpyHostToDevice, st));
         const double lim = std::cos(1.5 * p->step_deg * M_PI / 180.0);
@@ -253,11 +230,13 @@ acom_status build_plan_device(acom_plan_s* p, const acom_crystal* cr, cudaStream
         k_sum_counts<<<1, 1024, 0, st>>>(p->nbr_ptr, p->Z);
         prof_end(kKMisc, st);
         prof_begin(kKReflections, st);
-        k_reflections<<<1, kReflThreads, 0, st>>>(prm, d_atoms, d_tmp_g, d_tmp_F, d_g, d_amp,
-                                                  d_cnt);
+        k_reflections<<<(unsigned)((cand + kReflThreads - 1) / kReflThreads), kReflThreads, 0, st>>>(
+            prm, d_atoms, d_tmp_g, d_tmp_F, d_tmp_amp, d_cnt);
+        k_compact_reflections<<<1, kCompactThreads, 0, st>>>((int)cand, d_tmp_g, d_tmp_F, d_tmp_amp,
+                                                             d_cnt, d_g, d_amp, (int*)(d_cnt + 1));
         prof_end(kKReflections, st);
         ACOM_TRY(cudaGetLastError());
-        ACOM_TRY(cudaMemcpyAsync(p->host_words, d_cnt, sizeof(int), cudaMemcpyDeviceToHost, st));
+        ACOM_TRY(cudaMemcpyAsync(p->host_words, d_cnt + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
         ACOM_TRY(cudaMemcpyAsync(p->host_words + 1, p->nbr_ptr + p->Z, sizeof(int),
                                  cudaMemcpyDeviceToHost, st));
         ACOM_TRY(cudaStreamSynchronize(st));
@@ -278,8 +257,9 @@ acom_status build_plan_device(acom_plan_s* p, const acom_crystal* cr, cudaStream
         pool_free(d_atoms, st);
         pool_free(d_tmp_g, st);
         pool_free(d_tmp_F, st);
+        pool_free(d_tmp_amp, st);
         pool_free(d_cnt, st);
-        d_atoms = d_tmp_g = d_tmp_F = nullptr;
+        d_atoms = d_tmp_g = d_tmp_F = d_tmp_amp = nullptr;
         d_cnt = nullptr;
 
         // P0 -> FFT along phi3 -> scale by A
@@ -311,6 +291,7 @@ fail:
     pool_free(d_atoms, st);
     pool_free(d_tmp_g, st);
     pool_free(d_tmp_F, st);
+    pool_free(d_tmp_amp, st);
     pool_free(d_g, st);
     pool_free(d_amp, st);
     pool_free(d_cnt, st);

@@ -261,3 +261,25 @@ def test_grid_neighbours(step):
         np.testing.assert_allclose(m[b], O.refine(mt, za, step).m, atol=1e-4)
     assert same > 0
     plan.close()
+
+
+@pytest.mark.parametrize("q_max", [0.5, 1.5, 3.1])
+def test_reflections_of_small_and_large_boxes(q_max):
+    """Index boxes of a part of a block, of several blocks, and of several rounds of the
+    compaction: as many reflections as the oracle's, and their order and amplitudes through
+    the plan's spectra (rows are normalised sums in that order)."""
+    from oracle import acom_oracle as O
+    from paper_2111_00171_gb300 import acom
+    tri, area = acom.cubic_triangle()
+    au = acom.au_crystal()
+    refl = O.reflections(au.lattice, au.frac_pos, au.ff_A, au.ff_B, q_max)
+    plan = acom.Plan(au, tri, area, 12.0, 40, 0.08, 72, lam=LAM, q_max=q_max)
+    assert plan.info["n_reflections"] == len(refl.F)
+    za = O.zone_axis_grid(*O.cubic_triangle()[:3], 12.0, O.cubic_triangle()[3])
+    oplan = O.orientation_plan(refl, za, O.PlanParams(40, 0.08, 72, 0.08, lam=LAM))
+    scan = synth.random_patterns(10, n_patterns=8)
+    r = plan.match(*to_dev(scan))
+    for b in range(scan.n_patterns):
+        assert math.isclose(float(r["score"][b]), O.match_pattern(oplan, *scan.pattern(b)).score,
+                            rel_tol=1e-4), b
+    plan.close()
