@@ -24,6 +24,7 @@ constexpr int kErrRowPtr = 1;       // row_ptr[0] != 0 or decreasing
 constexpr int kErrNonFinite = 2;    // qx, qy or I not finite
 constexpr int kErrTooManyPeaks = 4; // more than kMaxPeaks peaks in a pattern
 constexpr int kErrTimeout = 8;      // a bounded device wait gave up
+constexpr int kWords = 4, kHostWords = 6;
 
 // Parameters of the sparse polar raster shared by plan and pattern sources.
 // Row stride (in floats) of the shell-major spectra [item][Spad][Fs]: F
@@ -82,6 +83,7 @@ struct PatternSource {         // one chunk of CSR patterns
     float* xscale = nullptr;   // [n_items] 2^e_b of each pattern (with xb_fp16, or without xb)
     int* tickets = nullptr;    // patterns taken so far by all launches (or nullptr: fixed
     int taken = 0;             // shares), and its value when this launch starts
+    int row0 = 0;              // row_ptr is the batch's: its first entry must be 0
     int xb_k0 = 0;             // the contraction reads xb from this shell on: 16-shell
                                // tiles wholly below it are not written
 };
@@ -136,8 +138,6 @@ struct Workspace {
     int PTs = 0;                   // pattern tiles of 64 in XB
     alignas(64) unsigned char map_x[128];   // TMA map of XB
     float* xfn = nullptr;          // [chunk][F] ||X^_bf|| over shells
-    int* n_eval = nullptr;         // [3] axes evaluated exactly in the last match, patterns taken
-                                   // by select and by the raster
     int2* srange = nullptr;        // [chunk] non-zero shell range of each pattern
     uint32_t* rmask = nullptr;     // [chunk][Spad / 32] shells each pattern's tents reach
     unsigned long long* best = nullptr;  // [chunk] packed (score, index)
@@ -187,7 +187,9 @@ struct acom_plan_s {
     int* nbr_idx = nullptr;
     double* refl_g = nullptr;         // [G][3]
     double* refl_amp = nullptr;       // [G]
-    int* err = nullptr;               // device error word
+    // device words [kWords]: error word; axes evaluated exactly in the last match; patterns
+    // taken in it by select, by the raster.  One clear and one copy a match.
+    int* err = nullptr;
     float* pfmax = nullptr;           // [F] max over axes of ||P^_zf|| over shells
     float pscale = 1.0f;              // 2^k of the FP16 plan spectra (1 otherwise)
     uint32_t* smask = nullptr;        // [Zp][Spad / 32] bit s: shell row s of the axis not zero
@@ -207,15 +209,14 @@ struct acom_plan_s {
     int ks = 0;
     alignas(64) unsigned char map_ps[128];
     float4* refl_tab = nullptr;       // [G] FP32 (g, |g|^gamma |F_g|^omega) for refinement
-    unsigned long long* refine_pairs = nullptr;  // [2] (reflection, peak) pairs of the last
-                                                 // refine, patterns taken
     int64_t last_refine_pairs = 0;
     int n_phases = 1;                 // crystal structures (phases) in this plan
     std::vector<int> phase_off_host;  // [n_phases + 1] first axis of each phase, then Z
     int* phase_off = nullptr;         // the same on the device
     int64_t last_evaluated = 0;       // axes evaluated exactly in the last match
-    int* host_words = nullptr;        // pinned [2]: error word and evaluations of the last
-                                      // match (read by acom_sync / acom_match)
+    // pinned [6]: error word and evaluations of the last match (read by acom_sync and
+    // acom_match), the error word of another call, -, its 64-bit pair count
+    int* host_words = nullptr;
     int64_t async_exhaustive_evals = -1;  // exhaustive: evaluations of the last match
     size_t bytes = 0;
     acom::Workspace ws;
@@ -307,8 +308,6 @@ acom_status set_error(acom_status s, const std::string& msg);
 acom_status cuda_error(cudaError_t e, const char* what);
 void clear_error();                 // acom_last_error() returns "" afterwards
 void count_allocation();            // one device or pinned allocation requested
-// device check that row_ptr[0] == 0 (sets kErrRowPtr in err); allocates nothing
-void launch_check_row0(const int64_t* row_ptr, int* err, cudaStream_t st);
 
 // ---- launchers (defined in the .cu files) ----
 // plan.cu
@@ -387,6 +386,7 @@ acom_status refine_table(acom_plan_s* p, cudaStream_t st);
 void launch_refine_orient(const acom_plan_s* p, const acom_peaks_csr* pk, int steps,
                           float rho_start, float rho_end, float damping, float max_step, int twin,
                           float* orient, const float* orient_alt, float* score, uint8_t* start_out,
+                          unsigned long long* counters,
                           cudaStream_t st);
 void launch_kin_score(const acom_plan_s* p, const acom_peaks_csr* pk, const float* orient,
                       const float* r, const float* strain, float rho, float* score, float* grad,

@@ -150,7 +150,6 @@ static void free_workspace(Workspace& ws, cudaStream_t st) {
     pool_free(ws.U, st);
     pool_free(ws.extra, st);
     pool_free(ws.xfn, st);
-    pool_free(ws.n_eval, st);
     pool_free(ws.srange, st);
     pool_free(ws.rmask, st);
     pool_free(ws.best, st);
@@ -193,7 +192,6 @@ static acom_status ensure_ws(acom_plan_s* p, Workspace& ws, int chunk, bool need
     if ((e = dalloc(&ws.U, (size_t)chunk * p->Z, &acc, st)) != cudaSuccess) goto fail;
     if ((e = dalloc(&ws.extra, split_extra_floats(), &acc, st)) != cudaSuccess) goto fail;
     if ((e = dalloc(&ws.xfn, (size_t)chunk * p->F, &acc, st)) != cudaSuccess) goto fail;
-    if ((e = dalloc(&ws.n_eval, (size_t)3, &acc, st)) != cudaSuccess) goto fail;
     if ((e = dalloc(&ws.srange, (size_t)chunk, &acc, st)) != cudaSuccess) goto fail;
     if ((e = dalloc(&ws.rmask, (size_t)chunk * (p->Spad / 32), &acc, st)) != cudaSuccess) goto fail;
     if ((e = dalloc(&ws.best, (size_t)chunk, &acc, st)) != cudaSuccess) goto fail;
@@ -268,7 +266,6 @@ static void destroy_plan(acom_plan_s* p) {
     pool_free(p->Ps, st);
     pool_free(p->phase_off, st);
     pool_free(p->refl_tab, st);
-    pool_free(p->refine_pairs, st);
     pool_free(p->smask, st);
     if (p->host_words) cudaFreeHost(p->host_words);
     delete p;
@@ -314,18 +311,6 @@ static acom_status make_split_operand(acom_plan_s* p, cudaStream_t st) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_error(e, "plan operand");
     return make_bf16_map(p->map_ps, p->Ps, rows, 2 * (uint64_t)p->ks, 1, 256);
-}
-
-// The first row pointer of a CSR batch must be 0 (the other row checks run in
-// the raster, per pattern); one thread, no allocation.
-__global__ void k_check_row0(const int64_t* row_ptr, int* err) {
-    if (row_ptr[0] != 0) atomicOr(err, kErrRowPtr);
-}
-
-void launch_check_row0(const int64_t* row_ptr, int* err, cudaStream_t st) {
-    prof_begin(kKMisc, st);
-    k_check_row0<<<1, 1, 0, st>>>(row_ptr, err);
-    prof_end(kKMisc, st);
 }
 
 }  // namespace acom
@@ -432,13 +417,13 @@ acom_status acom_plan_create(const acom_crystal* crystal, const acom_za_grid* gr
     ACOM_CK(dalloc(&p->za, za.size(), &p->bytes, st));
     ACOM_CK(dalloc(&p->frames, frames.size(), &p->bytes, st));
     ACOM_CK(dalloc(&p->nbr_ptr, (size_t)Z + 1, &p->bytes, st));
-    ACOM_CK(dalloc(&p->err, 1, &p->bytes, st));
+    ACOM_CK(dalloc(&p->err, kWords, &p->bytes, st));
     ACOM_CK(dalloc(&p->pfmax, (size_t)p->F, &p->bytes, st));
     p->phase_off_host = {0, Z};
     ACOM_CK(dalloc(&p->phase_off, 2, &p->bytes, st));
     count_allocation();
-    ACOM_CK(cudaMallocHost(reinterpret_cast<void**>(&p->host_words), 2 * sizeof(int)));
-    p->host_words[0] = p->host_words[1] = 0;
+    ACOM_CK(cudaMallocHost(reinterpret_cast<void**>(&p->host_words), kHostWords * sizeof(int)));
+    std::fill_n(p->host_words, kHostWords, 0);
     ACOM_CK(cudaMemcpyAsync(p->phase_off, p->phase_off_host.data(), sizeof(int) * 2,
                             cudaMemcpyHostToDevice, st));
     ACOM_CK(dalloc(&p->smask, (size_t)p->Zp * (p->Spad / 32), &p->bytes, st));
@@ -450,7 +435,7 @@ acom_status acom_plan_create(const acom_crystal* crystal, const acom_za_grid* gr
         ACOM_CK(pool_alloc(&p->Pb, 2 * n, st));
         p->bytes += 2 * n;
     }
-    ACOM_CK(cudaMemsetAsync(p->err, 0, sizeof(int), st));
+    ACOM_CK(cudaMemsetAsync(p->err, 0, kWords * sizeof(int), st));
     ACOM_CK(cudaMemcpyAsync(p->za, za.data(), sizeof(double) * za.size(), cudaMemcpyHostToDevice, st));
     ACOM_CK(cudaMemcpyAsync(p->frames, frames.data(), sizeof(double) * frames.size(),
                             cudaMemcpyHostToDevice, st));
@@ -573,17 +558,17 @@ acom_status acom_plan_concat(const acom_plan* plans, int32_t n_plans, void* cuda
     ACOM_CK(dalloc(&p->frames, (size_t)9 * Z, &p->bytes, st));
     ACOM_CK(dalloc(&p->nbr_ptr, nptr.size(), &p->bytes, st));
     ACOM_CK(dalloc(&p->nbr_idx, nidx.size(), &p->bytes, st));
-    ACOM_CK(dalloc(&p->err, 1, &p->bytes, st));
+    ACOM_CK(dalloc(&p->err, kWords, &p->bytes, st));
     ACOM_CK(dalloc(&p->pfmax, (size_t)F, &p->bytes, st));
     ACOM_CK(dalloc(&p->phase_off, p->phase_off_host.size(), &p->bytes, st));
     count_allocation();
-    ACOM_CK(cudaMallocHost(reinterpret_cast<void**>(&p->host_words), 2 * sizeof(int)));
-    p->host_words[0] = p->host_words[1] = 0;
+    ACOM_CK(cudaMallocHost(reinterpret_cast<void**>(&p->host_words), kHostWords * sizeof(int)));
+    std::fill_n(p->host_words, kHostWords, 0);
     ACOM_CK(cudaMemsetAsync(p->Pr, 0, sizeof(float) * pelems, st));
     ACOM_CK(cudaMemsetAsync(p->Pi, 0, sizeof(float) * pelems, st));
     ACOM_CK(cudaMemsetAsync(p->Psr, 0, sizeof(float) * selems, st));
     ACOM_CK(cudaMemsetAsync(p->Psi, 0, sizeof(float) * selems, st));
-    ACOM_CK(cudaMemsetAsync(p->err, 0, sizeof(int), st));
+    ACOM_CK(cudaMemsetAsync(p->err, 0, kWords * sizeof(int), st));
     ACOM_CK(cudaMemcpyAsync(p->nbr_ptr, nptr.data(), sizeof(int) * nptr.size(),
                             cudaMemcpyHostToDevice, st));
     if (!nidx.empty())
@@ -702,10 +687,12 @@ static acom_status check_peaks(const acom_peaks_csr* pk) {
 }
 
 static acom_status read_error_word(acom_plan_s* p, cudaStream_t st) {
-    int herr = 0;
-    cudaError_t e = cudaMemcpyAsync(&herr, p->err, sizeof(int), cudaMemcpyDeviceToHost, st);
+    // pinned: a copy to pageable memory is staged and waits twice
+    cudaError_t e = cudaMemcpyAsync(p->host_words + 2, p->err, sizeof(int), cudaMemcpyDeviceToHost,
+                                    st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_error(e, "match");
+    const int herr = p->host_words[2];
     prof_resolve();
     if (herr & kErrTimeout) return set_error(ACOM_ERR_TIMEOUT, "device wait timed out");
     if (herr & (kErrRowPtr | kErrNonFinite | kErrTooManyPeaks)) {
@@ -729,11 +716,11 @@ acom_status acom_polar_spectra(acom_plan p, const acom_peaks_csr* peaks, float* 
     if (B == 0) return ACOM_OK;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     cudaMemsetAsync(p->err, 0, sizeof(int), st);
-    launch_check_row0(peaks->row_ptr, p->err, st);
     RasterGeom geo{p->S, p->Spad, p->N, p->F, (float)p->dq, (float)p->delta, (float)p->gamma_pow, 0};
     // straight into the caller's arrays
     PatternSource src{nullptr, 0, peaks->row_ptr, peaks->qx, peaks->qy, peaks->I, B,
                       (float)p->gamma_pow, (float)p->omega};
+    src.row0 = 1;
     RasterOut ro;
     ro.xs = reinterpret_cast<float2*>(dst);
     ro.sumsq = xnorm;
@@ -831,10 +818,8 @@ static acom_status match_enqueue(acom_plan p, const acom_peaks_csr* peaks,
                          "(run acom_match once with the same chunk and mode first)");
     s = ensure_workspace(p, chunk, exhaustive, fp32_contraction, st);
     if (s != ACOM_OK) return s;
-    cudaMemsetAsync(p->err, 0, sizeof(int), st);
-    cudaMemsetAsync(p->ws.n_eval, 0, 3 * sizeof(int), st);
+    cudaMemsetAsync(p->err, 0, kWords * sizeof(int), st);
     int taken = 0;
-    launch_check_row0(peaks->row_ptr, p->err, st);
     RasterGeom geo{p->S, p->Spad, p->N, p->F, (float)p->dq, (float)p->delta, (float)p->gamma_pow, 0};
     const int wchunk = p->ws.chunk;
     Workspace& w = p->ws;
@@ -847,7 +832,8 @@ static acom_status match_enqueue(acom_plan p, const acom_peaks_csr* peaks,
                           peaks->qy, peaks->I, nb, (float)p->gamma_pow, (float)p->omega,
                           xscale ? 1 : 0, pairs16 ? w.xscale : xscale};
         src.xb_k0 = p->k0;
-        src.tickets = w.n_eval + 2;
+        src.row0 = c0 == 0;
+        src.tickets = p->err + 3;
         src.taken = (int)c0;
         RasterOut ro;
         ro.re = exhaustive ? w.Xr : nullptr;
@@ -887,7 +873,7 @@ static acom_status match_enqueue(acom_plan p, const acom_peaks_csr* peaks,
             }
             launch_select_exact(p, w.Xsr, w.Xsi, w.U, w.extra, ts, w.xfn, w.srange, w.rmask, p->pfmax,
                                 w.xnorm2, nb, tc ? kappa_tc(p) : kappa_fp32(p), refine, *out,
-                                c0, w.n_eval, st, xscale, rescore_top, w.oin, w.onbr,
+                                c0, p->err + 1, st, xscale, rescore_top, w.oin, w.onbr,
                                 &taken);
             if (out->phi3 || out->orient)
                 launch_orient_compose(p, w.oin, w.onbr, nb, refine, *out, c0, st);
@@ -896,8 +882,7 @@ static acom_status match_enqueue(acom_plan p, const acom_peaks_csr* peaks,
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "match launch");
     // error word and evaluations into the plan's pinned words
-    cudaMemcpyAsync(p->host_words, p->err, sizeof(int), cudaMemcpyDeviceToHost, st);
-    cudaMemcpyAsync(p->host_words + 1, p->ws.n_eval, sizeof(int), cudaMemcpyDeviceToHost, st);
+    cudaMemcpyAsync(p->host_words, p->err, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
     p->async_exhaustive_evals = exhaustive ? (int64_t)B * p->Z : -1;
     return ACOM_OK;
 }
@@ -965,7 +950,6 @@ acom_status acom_bounds(acom_plan p, const acom_peaks_csr* peaks, float* dst, vo
     s = ensure_workspace(p, chunk, false, !tc && !pairs16, st);
     if (s != ACOM_OK) return s;
     cudaMemsetAsync(p->err, 0, sizeof(int), st);
-    launch_check_row0(peaks->row_ptr, p->err, st);
     RasterGeom geo{p->S, p->Spad, p->N, p->F, (float)p->dq, (float)p->delta, (float)p->gamma_pow, 0};
     for (int64_t c0 = 0; c0 < B; c0 += chunk) {
         const int nb = (int)std::min<int64_t>(chunk, B - c0);
@@ -974,6 +958,7 @@ acom_status acom_bounds(acom_plan p, const acom_peaks_csr* peaks, float* dst, vo
                           peaks->qy, peaks->I, nb, (float)p->gamma_pow, (float)p->omega,
                           xscale ? 1 : 0, pairs16 ? p->ws.xscale : xscale};
         src.xb_k0 = p->k0;
+        src.row0 = c0 == 0;
         RasterOut ro;
         if (!tc) {
             ro.sre = p->ws.Xsr;
@@ -1020,18 +1005,21 @@ acom_status acom_refine(acom_plan p, const acom_peaks_csr* peaks, const acom_ref
     cudaStream_t st = (cudaStream_t)cuda_stream;
     s = refine_table(p, st);
     if (s != ACOM_OK) return s;
+    // the call's own counters: (reflection, peak) pairs, patterns taken
+    unsigned long long* counters = nullptr;
+    cudaError_t e = pool_alloc(reinterpret_cast<void**>(&counters), 2 * sizeof(*counters), st);
+    if (e != cudaSuccess) return cuda_error(e, "refine counters");
     cudaMemsetAsync(p->err, 0, sizeof(int), st);
-    cudaMemsetAsync(p->refine_pairs, 0, 2 * sizeof(unsigned long long), st);
-    launch_check_row0(peaks->row_ptr, p->err, st);
+    cudaMemsetAsync(counters, 0, 2 * sizeof(*counters), st);
     launch_refine_orient(p, peaks, o.steps, o.rho_start, o.rho_end, o.damping,
                          (float)(o.max_step_deg * M_PI / 180.0), o.twin ? 1 : 0, orient,
-                         orient_alt, score, start, st);
-    cudaError_t e = cudaGetLastError();
+                         orient_alt, score, start, counters, st);
+    e = cudaGetLastError();
+    cudaMemcpyAsync(p->host_words + 4, counters, sizeof(*counters), cudaMemcpyDeviceToHost, st);
+    pool_free(counters, st);
     if (e != cudaSuccess) return cuda_error(e, "refine launch");
-    unsigned long long pairs = 0;
-    cudaMemcpyAsync(&pairs, p->refine_pairs, sizeof(pairs), cudaMemcpyDeviceToHost, st);
     s = read_error_word(p, st);
-    p->last_refine_pairs = (int64_t)pairs;
+    std::memcpy(&p->last_refine_pairs, p->host_words + 4, sizeof(p->last_refine_pairs));
     return s;
 }
 
@@ -1050,7 +1038,6 @@ acom_status acom_kinematical_score_strain(acom_plan p, const acom_peaks_csr* pea
     s = refine_table(p, st);
     if (s != ACOM_OK) return s;
     cudaMemsetAsync(p->err, 0, sizeof(int), st);
-    launch_check_row0(peaks->row_ptr, p->err, st);
     launch_kin_score(p, peaks, orient, r, strain, rho, score, grad, gn, strain_grad, st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "score launch");

@@ -101,13 +101,12 @@ extern "C" acom_status acom_bounds_static(acom_plan p, const acom_peaks_csr* pea
         prof_suppress(false);
         return cuda_error(e, "bounds_static: clearing the error word");
     }
-    // row_ptr[0] == 0 (the raster checks the rest of the row pointers)
-    launch_check_row0(peaks->row_ptr, p->err, st);
     RasterGeom geo{p->S, p->Spad, p->N, p->F, (float)p->dq, (float)p->delta, (float)p->gamma_pow, 0};
     for (int64_t c0 = 0; c0 < B; c0 += chunk) {
         const int nb = (int)std::min<int64_t>(chunk, B - c0);
         PatternSource src{XB, PTs, peaks->row_ptr + c0, peaks->qx, peaks->qy, peaks->I, nb,
                           (float)p->gamma_pow, (float)p->omega};
+        src.row0 = c0 == 0;
         RasterOut ro;
         ro.re = Xr;
         ro.im = Xi;

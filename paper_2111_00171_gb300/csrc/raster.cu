@@ -86,6 +86,7 @@ struct PatternLoader {
         const int64_t b0 = src.row_ptr[item];
         const int64_t b1 = src.row_ptr[item + 1];
         int64_t cnt = b1 - b0;
+        if (src.row0 && item == 0 && b0 != 0 && threadIdx.x == 0) atomicOr(err, kErrRowPtr);
         if (cnt < 0) {
             if (threadIdx.x == 0) atomicOr(err, kErrRowPtr);
             return 0;

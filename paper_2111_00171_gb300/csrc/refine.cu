@@ -472,6 +472,7 @@ __device__ int load_peaks(const RefArgs& a, int64_t b, int64_t& p0, float* px, f
     p0 = a.row_ptr[b];
     const int64_t p1 = a.row_ptr[b + 1];
     const int64_t n = p1 - p0;
+    if (b == 0 && p0 != 0 && lane == 0) atomicOr(a.err, kErrRowPtr);
     if (n < 0 || n > kMaxPeaks) {
         if (lane == 0) atomicOr(a.err, n < 0 ? kErrRowPtr : kErrTooManyPeaks);
         return -1;
@@ -663,8 +664,6 @@ acom_status refine_table(acom_plan_s* p, cudaStream_t st) {
     cudaError_t e = pool_alloc(reinterpret_cast<void**>(&p->refl_tab), sizeof(float4) * p->G, st);
     if (e != cudaSuccess) return cuda_error(e, "refinement table allocation");
     p->bytes += sizeof(float4) * p->G;
-    e = pool_alloc(reinterpret_cast<void**>(&p->refine_pairs), 2 * sizeof(unsigned long long), st);
-    if (e != cudaSuccess) return cuda_error(e, "refinement counter allocation");
     prof_begin(kKMisc, st);
     k_refl_table<<<(p->G + 255) / 256, 256, 0, st>>>(p->refl_g, p->refl_amp, p->G, p->gamma_pow,
                                                       p->refl_tab);
@@ -701,7 +700,7 @@ static int ref_grid(int64_t nb) {
 void launch_refine_orient(const acom_plan_s* p, const acom_peaks_csr* pk, int steps,
                           float rho_start, float rho_end, float damping, float max_step, int twin,
                           float* orient, const float* orient_alt, float* score, uint8_t* start_out,
-                          cudaStream_t st) {
+                          unsigned long long* counters, cudaStream_t st) {
     RefArgs a = ref_args(p, pk);
     a.steps = steps;
     a.rho_start = rho_start;
@@ -713,8 +712,8 @@ void launch_refine_orient(const acom_plan_s* p, const acom_peaks_csr* pk, int st
     a.orient_alt = orient_alt;
     a.score = score;
     a.start_out = start_out;
-    a.pairs = p->refine_pairs;
-    a.taken = p->refine_pairs + 1;
+    a.pairs = counters;
+    a.taken = counters + 1;
     const int grid = std::min(ref_grid(pk->n_patterns), 3 * sm_count());   // three CTAs an SM
     if (grid <= 0) return;
     prof_begin(kKRefineOrient, st);

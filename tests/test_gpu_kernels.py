@@ -283,3 +283,23 @@ def test_reflections_of_small_and_large_boxes(q_max):
         assert math.isclose(float(r["score"][b]), O.match_pattern(oplan, *scan.pattern(b)).score,
                             rel_tol=1e-4), b
     plan.close()
+
+
+@pytest.mark.parametrize("call", ["match", "bounds", "polar_spectra", "refine", "kinematical_score"])
+def test_rows_that_do_not_start_at_zero(call):
+    """A batch whose rows start at the second peak (all in range) is refused by whichever
+    kernel reads the first pattern, and the next good batch is accepted."""
+    import torch
+    from paper_2111_00171_gb300 import acom
+    plan = au_plan(6.0, 40, 0.0375, 72)
+    scan = synth.random_patterns(11, n_patterns=70)
+    rp, qx, qy, I = to_dev(scan)
+    bad = rp.clone()
+    bad[0] = 1
+    m = torch.from_numpy(scan.truth.astype(np.float32)).cuda()
+    run = getattr(plan, call)
+    more = {"refine": (m.clone(),), "kinematical_score": (m,)}.get(call, ())
+    with pytest.raises(acom.AcomError, match="row_ptr"):
+        run(bad, qx, qy, I, *more)
+    run(rp, qx, qy, I, *more)
+    plan.close()
