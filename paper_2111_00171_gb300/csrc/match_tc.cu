@@ -1564,7 +1564,9 @@ __device__ __forceinline__ __nv_fp8_e4m3 to_half_type<__nv_fp8_e4m3>(float x) {
 // 150 shells x 181 frequencies 0.2 GB in, 0.6 GB out.  It replaced a scaling pass over
 // both layouts, the raster's 8-byte frequency-major stores, three passes for the
 // norms, the mask and the operand, and 0.95 GB of clearing: after the reflections the
-// plan's build took 0.98 ms of the GPU and now 0.40.  T void: no operand.
+// plan's build took 0.98 ms of the GPU and now 0.35.  A warp loads its four rows of the
+// next tile together while this one is stored (one row at a time, each load waited
+// through the mask's vote: 276 us, now 200).  T void: no operand.
 template <class T>
 __global__ void __launch_bounds__(256)
 k_plan_layouts(const float* __restrict__ sumsq, int Z, int ZT, int F, int Spad,
@@ -1578,37 +1580,49 @@ k_plan_layouts(const float* __restrict__ sumsq, int Z, int ZT, int F, int Spad,
     const float ss = real_axis ? sumsq[z] : 0.f;
     const float a = ss > 0.f ? rsqrtf(ss) : 0.f;
     float nrm[4] = {0.f, 0.f, 0.f, 0.f};      // of frequencies f0 + warp + 8 j, lanes over shells
-    for (int s0 = 0; s0 < Spad; s0 += 32) {
-        for (int r = warp; r < 32; r += 8) {
-            const int64_t o = ((int64_t)z * Spad + s0 + r) * Fs + f0 + lane;
-            float u = 0.f, v = 0.f;
-            if (f0 + lane < Fs) {
-                if (real_axis) {
-                    u = sre[o] * a;
-                    v = sim[o] * a;
-                }
-                sre[o] = u;
-                sim[o] = v;
-            }
-            tr[r][lane] = u;
-            ti[r][lane] = v;
-            if (__any_sync(0xffffffffu, u != 0.f || v != 0.f) && lane == 0)
-                atomicOr(smask + (int64_t)z * (Spad >> 5) + (s0 >> 5), 1u << r);
+    const bool in_row = f0 + lane < Fs;
+    float u[4], v[4];                         // the next tile's rows warp + 8 j, loads in flight
+    auto load = [&](int s0) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int64_t o = ((int64_t)z * Spad + s0 + warp + 8 * j) * Fs + f0 + lane;
+            const bool get = real_axis && in_row;
+            u[j] = get ? sre[o] : 0.f;
+            v[j] = get ? sim[o] : 0.f;
         }
+    };
+    load(0);
+    for (int s0 = 0; s0 < Spad; s0 += 32) {
+        uint32_t rows = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int r = warp + 8 * j;
+            const float x = u[j] * a, y = v[j] * a;
+            tr[r][lane] = x;
+            ti[r][lane] = y;
+            if (in_row) {
+                const int64_t o = ((int64_t)z * Spad + s0 + r) * Fs + f0 + lane;
+                sre[o] = x;
+                sim[o] = y;
+            }
+            if (__any_sync(0xffffffffu, x != 0.f || y != 0.f)) rows |= 1u << r;
+        }
+        if (rows && lane == 0) atomicOr(smask + (int64_t)z * (Spad >> 5) + (s0 >> 5), rows);
+        if (s0 + 32 < Spad) load(s0 + 32);
         __syncthreads();
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int f = f0 + warp + 8 * j;
             if (f < F) {
-                const float u = tr[lane][warp + 8 * j], v = ti[lane][warp + 8 * j];
+                const float x = tr[lane][warp + 8 * j], y = ti[lane][warp + 8 * j];
                 const int64_t o = ((int64_t)z * F + f) * Spad + s0 + lane;
-                re[o] = u;
-                im[o] = v;
-                nrm[j] = fmaf(u, u, fmaf(v, v, nrm[j]));
+                re[o] = x;
+                im[o] = y;
+                nrm[j] = fmaf(x, x, fmaf(y, y, nrm[j]));
                 if constexpr (!std::is_void<T>::value) {
                     T* d = op + (((int64_t)f * ZT + (z >> 7)) * 256 + (z & 127)) * Spad + s0 + lane;
-                    d[0] = to_half_type<T>(scale * u);
-                    d[(int64_t)128 * Spad] = to_half_type<T>(scale * v);
+                    d[0] = to_half_type<T>(scale * x);
+                    d[(int64_t)128 * Spad] = to_half_type<T>(scale * y);
                 }
             }
         }
