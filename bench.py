@@ -717,7 +717,7 @@ def sweep_combos(args, acom, lib, scan, d_in, flush, stream, n_oracle=1000):
             def step():
                 p = plan()
                 p.match(*d_in, out=out, rescore_top=top)
-                info["ev"] = p.get_info()["last_evaluated"]
+                info["ev"], info["k0"] = p.get_info()["last_evaluated"], p.info["k0"]
                 p.close()
             step()
             torch.cuda.synchronize()
@@ -738,8 +738,8 @@ def sweep_combos(args, acom, lib, scan, d_in, flush, stream, n_oracle=1000):
             flops = 8.0 * Z * S * F * B
             tflops = flops / (cms / 1e3) / 1e12 if cms else 0.0
             # E4M3's dense rate is twice BF16's (4.5 vs 2.25 PFLOP/s nominal)
-            peak = fp32_peak if prec == "fp32" else peaks["bf16_tflops"] * \
-                (2.0 if prec == "fp8" else 1.0)
+            alu = prec == "fp32" and not fp32_on_tensor_cores(S, info["k0"], N)
+            peak = fp32_peak if alu else peaks["bf16_tflops"] * (2.0 if prec == "fp8" else 1.0)
             mis, mis_twin, tilt = misorientation(out["orient"].cpu().numpy(), scan.truth)
             res = {k: out[k].cpu().numpy() for k in ("za_idx", "phi3_bin", "mirror")}
             choices.append([(int(res["za_idx"][b]), int(res["phi3_bin"][b]),
@@ -749,7 +749,7 @@ def sweep_combos(args, acom, lib, scan, d_in, flush, stream, n_oracle=1000):
                                      else "certified pruning",
                              "patterns_per_s": B / (ms / 1e3), "ms_per_step": ms,
                              "contraction_tflops": tflops, "contraction_frac": tflops / peak,
-                             "contraction_bound": "alu" if prec == "fp32" else "tensor",
+                             "contraction_bound": "alu" if alu else "tensor",
                              "axes_evaluated_per_pattern": info["ev"] / B,
                              "mean_misorientation_deg": mis,
                              "mean_misorientation_friedel_deg": mis_twin})
@@ -867,6 +867,12 @@ def kernel_traffic(name, pats, precision):
     return t[0] * pats / t[1] if t[6] else None
 
 
+def fp32_on_tensor_cores(S, k0, N):
+    """Whether the pruned match of an FP32 plan contracts FP16 pairs on the tensor cores:
+    at most 128 shells from the first non-zero one, at least 180 bins."""
+    return -(-(S - k0) // 16) * 16 <= 128 and N >= 180
+
+
 def kernel_roofline(name, cnt, ms, peaks, src, B, K, nnz, precision, refine_pairs=0,
                     rows_nz=None, k0=0):
     """Achieved rate of one kernel class: algorithmic work per launch over its
@@ -886,6 +892,11 @@ def kernel_roofline(name, cnt, ms, peaks, src, B, K, nnz, precision, refine_pair
         if k0:
             note += (f"; the kernel skips shells 0..{k0 - 1}, where every plan row is zero "
                      f"(it executes {W['S'] - k0} of the {W['S']} shells counted)")
+    elif name == "contract_fp32" and rows_nz is not None and fp32_on_tensor_cores(S, k0, N):
+        work, unit, bound, peak = 8.0 * Z * S * F * pats, "TFLOP/s", "tensor", \
+            peaks["bf16_tflops"]
+        note = (f"8 Z S F flops per pattern, each FP32 product taken as three of FP16 halves; "
+                f"bf16 burst peak ({src})")
     elif name == "contract_fp32":
         work, unit, bound, peak = 8.0 * Z * S * F * pats, "TFLOP/s", "alu", fp32_peak
         note = "8 Z S F flops per pattern; FP32 FMA peak 152 SMs x 128 lanes x 2 x max clock"
