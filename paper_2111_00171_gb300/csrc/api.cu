@@ -304,6 +304,12 @@ static acom_status make_split_operand(acom_plan_s* p, cudaStream_t st) {
     if (p->ks == 0) return ACOM_OK;
     const size_t rows = (size_t)p->F * p->Zp * 2;
     cudaError_t e = pool_alloc(&p->Ps, rows * p->ks * 4, st);
+    if (e == cudaErrorMemoryAllocation) {      // no room for it: the FP32 pipe's contraction
+        cudaGetLastError();
+        p->Ps = nullptr;
+        p->ks = 0;
+        return ACOM_OK;
+    }
     if (e != cudaSuccess) return cuda_error(e, "plan operand");
     p->bytes += rows * p->ks * 4;
     launch_plan_split(p, st);
