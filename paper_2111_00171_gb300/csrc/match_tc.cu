@@ -505,8 +505,10 @@ k_contract_bound_tc(const __grid_constant__ CUtensorMap map_p,
                     for (int kt = 0; kt < a.KT && ok; ++kt) {
                         const bool last_k = kt + 1 == a.KT;
                         // K steps of 32 bytes inside the shells (16 16-bit or 32 8-bit
-                        // elements); a step moves the descriptors by 32 bytes (2 units)
-                        const int nk = (min(ktel * kSub, a.Spad - a.k0 - kt * ktel * kSub) * (F8 ? 1 : 2)) >> 5;
+                        // elements; E4M3 rounds up into the zero fill past the shells when k0
+                        // is an odd multiple of 16); a step moves the descriptors by 32 bytes
+                        // (2 units)
+                        const int nk = (min(ktel * kSub, a.Spad - a.k0 - kt * ktel * kSub) * (F8 ? 1 : 2) + 31) >> 5;
                         const uint64_t pd = sdesc(smem_u32(ring_p + ps * kPBytes));
                         for (int sub = 0; sub < nsub; ++sub) {
                             const uint32_t b = buf ^ (uint32_t)sub;
@@ -1175,7 +1177,7 @@ k_contract_bound_pair(const __grid_constant__ CUtensorMap map_p,
                         // fill); a step moves the descriptors' start address by
                         // 32 bytes (2 units of 16)
                         constexpr int ktel = F8 ? kKT8 : kKT;
-                        const int nk = (min(ktel, a.Spad - a.k0 - kt * ktel) * (F8 ? 1 : 2)) >> 5;
+                        const int nk = (min(ktel, a.Spad - a.k0 - kt * ktel) * (F8 ? 1 : 2) + 31) >> 5;
                         if (!mbar_wait(smem_u32(myfull + stage), spar, abort_flag, a.err,
                                        a.wait_cycles)) {
                             ok = false;

@@ -303,3 +303,34 @@ def test_rows_that_do_not_start_at_zero(call):
         run(bad, qx, qy, I, *more)
     run(rp, qx, qy, I, *more)
     plan.close()
+
+
+@pytest.mark.parametrize("geometry", [(6.0, 117, 0.0125, 300), (6.0, 85, 0.0175, 120)], ids=str)
+def test_e4m3_bounds_of_the_last_shells(geometry):
+    """Plans whose first shell is an odd multiple of 16, so that E4M3's K steps of 32 end
+    past the last shell: bounds of patterns with all peaks there against FP64.  Rounding a
+    product of two E4M3 values costs 2^-3 + 2^-8 of it at most, both parts of a complex
+    product sqrt 2 times that; 2^-6 more for values below the normal range."""
+    import torch
+    plan = au_plan(*geometry, precision=3)
+    N, F = geometry[3], geometry[3] // 2 + 1
+    assert plan.info["k0"] % 32 == 16
+    P = torch.view_as_complex(plan.spectra()).to(torch.complex128)
+    last = int((P.abs().amax((0, 2)) > 0).nonzero().max())     # the last shell that is not empty
+    rng = np.random.default_rng(5)
+    rp = np.concatenate([[0], np.cumsum(rng.integers(4, 12, 9))]).astype(np.int64)
+    r, t = last * geometry[2] + 0.05, rng.uniform(-np.pi, np.pi, rp[-1])
+    peaks = tuple(torch.from_numpy(x).cuda() for x in (
+        rp, (r * np.cos(t)).astype(np.float32), (r * np.sin(t)).astype(np.float32),
+        np.ones(rp[-1], np.float32)))
+    X = torch.view_as_complex(plan.polar_spectra(*peaks)[0]).to(torch.complex128)
+    w = torch.full((F,), 2.0 / N, dtype=torch.float64, device="cuda")
+    w[0] = w[-1] = 1.0 / N
+    want, _ = bounds64(plan, peaks)
+    tol = (math.sqrt(2.0) * (2.0 ** -3 + 2.0 ** -8) + 2.0 ** -6) * (
+        torch.einsum("zsf,bsf->bzf", P.abs(), X.abs()) * w).sum(2)
+    assert ((plan.bounds(*peaks).double() - want).abs() <= tol).all()
+    assert (want > 2.0 * tol).any()                            # a missing shell would show
+    one, pair = (plan.match(*peaks, cta_pairs=c) for c in (0, 1))
+    assert (one["za_idx"] == pair["za_idx"]).all() and (one["score"] == pair["score"]).all()
+    plan.close()
