@@ -196,12 +196,23 @@ void launch_contract_bound_fp32(const acom_plan_s* p, const float* Xr, const flo
     prof_end(kKContract, st);
 }
 
-// a split tile's later groups, in their order
+// a split tile's later groups onto its first, eight at a time: a small batch's tiles are
+// cut into up to a frequency each, and one chain of that many FP32 additions rounds more
+// than a whole tile's sum (split_shells)
 __device__ __forceinline__ float later_groups(const TileSplit& ts, const float* __restrict__ extra,
                                               int b, int z, float u) {
     const int t = ts.groups > 1 ? ts.split_tile(b, z) : -1;
-    if (t >= 0)
-        for (int g = 1; g < ts.groups; ++g) u += extra[ts.extra_at(g, t, b, z)];
+    if (t >= 0) {
+        float s = 0.f;
+        for (int g = 1; g < ts.groups; ++g) {
+            s += extra[ts.extra_at(g, t, b, z)];
+            if ((g & 7) == 0) {
+                u += s;
+                s = 0.f;
+            }
+        }
+        u += s;
+    }
     return u;
 }
 

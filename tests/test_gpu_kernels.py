@@ -177,6 +177,29 @@ def test_fp16_pairs_are_no_less_accurate_than_fp32(geometry):
     plan.close()
 
 
+# one tile, cut into a group per frequency or two; 168 tiles, the last 16 in groups of 21
+# frequencies and the others whole, each in four sums
+@pytest.mark.parametrize("geometry,patterns", [
+    ((4.0, 75, 0.02, 180), 8), ((4.0, 75, 0.02, 180), 120), ((4.0, 100, 0.015, 240), 120),
+    ((4.0, 117, 0.0125, 300), 120), ((1.0, 150, 0.01, 360), 2600)], ids=str)
+def test_fp16_pairs_in_few_and_in_many_tiles(geometry, patterns):
+    """However the batch cuts the frequencies into groups, the FP16 pairs' bounds are no
+    further from FP64 than those of the CUDA cores, which add all frequencies in turn."""
+    import torch
+    plan = au_plan(*geometry)
+    scan = synth.random_patterns(145, n_patterns=patterns)
+    peaks = to_dev(scan)
+    pairs = plan.bounds(*peaks)
+    cores = plan.bounds_static(*peaks, out=torch.empty_like(pairs))
+    # patterns of the first and of the last tiles
+    idx = np.r_[0:min(patterns, 128), max(128, patterns - 168):patterns]
+    want, _ = bounds64(plan, to_dev(scan.subset(idx)))
+    for part in (slice(0, 128), slice(128, None)):
+        off = lambda u: float((u[torch.from_numpy(idx).cuda()].double() - want)[part].norm())
+        assert off(pairs) <= off(cores)
+    plan.close()
+
+
 @pytest.mark.parametrize("geometry", [(6.0, 150, 0.01, 360), (6.0, 75, 0.02, 180)], ids=str)
 @pytest.mark.parametrize("precision", [1, 2], ids=["bf16", "fp16"])
 def test_sixteen_bit_copies_with_one_and_two_staging_buffers(geometry, precision):
