@@ -197,9 +197,10 @@ __device__ float fp16_pattern_scale(const PeakT* sp, int np, const RasterGeom& g
     __syncthreads();
     float tot = 0.f;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += __int_as_float(red[w]);
-    if (!(tot > 0.f) || !isfinite(tot)) return 1.0f;
-    int e = (int)floorf(log2f(kFp16Target / tot));
-    e = e < -100 ? -100 : (e > 100 ? 100 : e);
+    if (!(tot > 0.f)) return 1.0f;
+    // (a sum past FLT_MAX: 2^-114 brings any FP32 value below the target)
+    int e = isfinite(tot) ? (int)floorf(log2f(kFp16Target / tot)) : -114;
+    e = e < -114 ? -114 : (e > 100 ? 100 : e);
     float sc = ldexpf(1.0f, e);
     if (sc * tot > kFp16Target) sc *= 0.5f;      // guard the log2 rounding
     return sc;

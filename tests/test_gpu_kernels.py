@@ -200,6 +200,26 @@ def test_fp16_pairs_in_few_and_in_many_tiles(geometry, patterns):
     plan.close()
 
 
+@pytest.mark.parametrize("precision", [0, 2], ids=["fp32", "fp16"])
+def test_weights_near_the_top_of_fp32(precision):
+    """Peak weights up to 1e36 (omega 2, so a weight is its intensity times q): the FP16
+    scale covers FP32's range, and the winners and scores are those of the same pattern
+    with weights near 1, but for the scale."""
+    import torch
+    from paper_2111_00171_gb300 import acom
+    tri, area = acom.cubic_triangle()
+    plan = acom.Plan(acom.au_crystal(), tri, area, 3.0, 75, 0.02, 180, lam=LAM, omega=2.0,
+                     precision=precision)
+    rp, qx, qy, I = to_dev(synth.random_patterns(12, n_patterns=20))
+    I = I / I.max()
+    want = plan.match(rp, qx, qy, I)["score"].double()
+    up = 2.0 ** 119                                   # exact
+    got = plan.match(rp, qx, qy, I * up)["score"].double() / up
+    # the same axis scored in batches of another size: another split of the shell sums
+    assert ((got - want).abs() <= 2e-6 * want).all()
+    plan.close()
+
+
 @pytest.mark.parametrize("geometry", [(6.0, 150, 0.01, 360), (6.0, 75, 0.02, 180)], ids=str)
 @pytest.mark.parametrize("precision", [1, 2], ids=["bf16", "fp16"])
 def test_sixteen_bit_copies_with_one_and_two_staging_buffers(geometry, precision):
