@@ -45,13 +45,28 @@ struct RasterGeom {
     int shell_power;   // 1: multiply rows by q_s^gamma_pow (plan); 0: peaks carry q_m^gamma
 };
 
+__host__ __device__ inline bool aligned8(const void* p) {
+    return (reinterpret_cast<uintptr_t>(p) & 7) == 0;
+}
+
+// A pair of floats at p, in one store if the array that p lies in is 8-byte aligned.
+__device__ __forceinline__ void store2(float* p, float a, float b, bool aligned) {
+    if (aligned) {
+        *reinterpret_cast<float2*>(p) = make_float2(a, b);
+    } else {
+        p[0] = a;
+        p[1] = b;
+    }
+}
+
 // Outputs of the raster + transform kernel (every pointer optional but one).
 struct RasterOut {
     float* re = nullptr;       // [item][F][Spad] (frequency-major rows of shells)
     float* im = nullptr;
     float* sre = nullptr;      // [item][Spad][Fs] (shell-major rows of frequencies, Fs = shell_row_stride(F))
     float* sim = nullptr;
-    float2* xs = nullptr;      // [item][S][F] interleaved (no 16-bit copy then)
+    float* xs = nullptr;       // [item][S][F][2] interleaved (no 16-bit copy then), the
+                               // caller's array: any float address (store2)
     float* sumsq = nullptr;    // [item] sum of squares of the polar image
     float* fnorm = nullptr;    // [item][F] ||X^_f|| over shells
     int2* srange = nullptr;    // [item] first and one-past-last shell with a non-zero row

@@ -728,7 +728,7 @@ acom_status acom_polar_spectra(acom_plan p, const acom_peaks_csr* peaks, float* 
                       (float)p->gamma_pow, (float)p->omega};
     src.row0 = 1;
     RasterOut ro;
-    ro.xs = reinterpret_cast<float2*>(dst);
+    ro.xs = dst;
     ro.sumsq = xnorm;
     launch_raster_patterns(geo, src, ro, p->err, st);
     cudaError_t e = cudaGetLastError();

@@ -71,6 +71,7 @@ __device__ inline int block_compact(bool keep, int* s_warp, int* total) {
 struct PatternLoader {
     using PeakT = PeakXY;
     static constexpr int kMinBlocks = 3;   // FFT raster CTAs per SM (74.5 KB of shared memory)
+    static constexpr bool kXs8 = true;     // out.xs is 8-byte aligned
     PatternSource src;
     __host__ __device__ void* xb_out() const { return src.xb; }
     __device__ int xb_tiles() const { return src.PTs; }
@@ -114,9 +115,16 @@ struct PatternLoader {
     }
 };
 
+// The same for a caller's spectra at an address that is not 8-byte aligned (a kernel of its
+// own: the test of the address in the aligned one's stores cost 5 % of it).
+struct PatternLoaderXs4 : PatternLoader {
+    static constexpr bool kXs8 = false;
+};
+
 struct PlanLoader {
     using PeakT = Peak;
     static constexpr int kMinBlocks = 2;
+    static constexpr bool kXs8 = true;
     PlanSource src;
     float delta;
     __host__ __device__ void* xb_out() const { return nullptr; }
@@ -415,8 +423,8 @@ k_raster_dft(RasterGeom geo, Loader ld, int64_t n_items, RasterOut out, int* err
                 for (int e = threadIdx.x; e < F * W; e += blockDim.x) {
                     const int w = e / F, f = e - w * F;
                     if (s0 + w < S)
-                        out.xs[(item * (int64_t)S + s0 + w) * F + f] =
-                            make_float2(st_re[w * F + f], st_im[w * F + f]);
+                        store2(out.xs + 2 * ((item * (int64_t)S + s0 + w) * F + f),
+                               st_re[w * F + f], st_im[w * F + f], Loader::kXs8);
                 }
             }
             __syncthreads();
@@ -858,9 +866,9 @@ k_raster_fft(RasterGeom geo, Loader ld, int64_t n_items, RasterOut out, FftRadix
                         out.sim[srow + Fs + f] = bi;
                     }
                     if (XB == 0 && out.xs && f < F) {
-                        float2* xs = out.xs + (item * (int64_t)S + sA) * F + f;
-                        if (sA < S) xs[0] = make_float2(ar, ai);
-                        if (vB) xs[F] = make_float2(br, bi);
+                        float* xs = out.xs + 2 * ((item * (int64_t)S + sA) * F + f);
+                        if (sA < S) store2(xs, ar, ai, Loader::kXs8);
+                        if (vB) store2(xs + 2 * F, br, bi, Loader::kXs8);
                     }
                     if (f < F) {
                         fa[k] = fmaf(ar, ar, fmaf(ai, ai, fmaf(br, br, fmaf(bi, bi, fa[k]))));
@@ -953,9 +961,11 @@ static bool launch_raster_fft(const RasterGeom& geo, const Loader& ld, int64_t n
     const int xk = ld.xb_out() ? (ld.xb_half() ? 2 : 1) : 0;
     auto pick = [&](auto pfa_c) -> const void* {
         constexpr bool P = decltype(pfa_c)::value;
-        return xk == 2 ? (const void*)k_raster_fft<Loader, P, 2>
-                       : (xk == 1 ? (const void*)k_raster_fft<Loader, P, 1>
-                                  : (const void*)k_raster_fft<Loader, P, 0>);
+        if constexpr (Loader::kXs8) {
+            if (xk == 2) return (const void*)k_raster_fft<Loader, P, 2>;
+            if (xk == 1) return (const void*)k_raster_fft<Loader, P, 1>;
+        }
+        return (const void*)k_raster_fft<Loader, P, 0>;      // (spectra: no 16-bit copy)
     };
     const void* kern = pfa ? pick(std::true_type{}) : pick(std::false_type{});
     set_max_dynamic_smem(kern, smem);
@@ -998,8 +1008,10 @@ void launch_raster_plan(const RasterGeom& geo, const PlanSource& src, int Z,
 
 void launch_raster_patterns(const RasterGeom& geo, const PatternSource& src,
                             const RasterOut& out, int* err, cudaStream_t st) {
-    PatternLoader ld{src};
-    launch_raster(geo, ld, src.n_items, out, err, st, kKRasterPatterns);
+    if (aligned8(out.xs))
+        launch_raster(geo, PatternLoader{src}, src.n_items, out, err, st, kKRasterPatterns);
+    else
+        launch_raster(geo, PatternLoaderXs4{{src}}, src.n_items, out, err, st, kKRasterPatterns);
 }
 
 // Shell-major rows [item][Spad][Fs] -> frequency-major [item][F][Spad], shells k0 on
@@ -1053,13 +1065,13 @@ void launch_rows_to_fmajor(const acom_plan_s* p, const float* sre, const float* 
 
 // shell-major rows [item][Spad][Fs] -> [item][S][F][2] interleaved
 __global__ void k_spectra_export(const float* __restrict__ sre, const float* __restrict__ sim,
-                                 int64_t rows, int F, int Spad, int S, float2* __restrict__ dst) {
+                                 int64_t rows, int F, int Spad, int S, float* __restrict__ dst) {
     const int Fs = shell_row_stride(F);
     for (int64_t row = blockIdx.x; row < rows; row += gridDim.x) {
         const int64_t item = row / S;
         const int64_t src = (item * Spad + (row - item * S)) * Fs;
         for (int f = threadIdx.x; f < F; f += blockDim.x)
-            dst[row * F + f] = make_float2(sre[src + f], sim[src + f]);
+            store2(dst + 2 * (row * F + f), sre[src + f], sim[src + f], aligned8(dst));
     }
 }
 
@@ -1069,8 +1081,7 @@ void launch_spectra_export(const float* sre, const float* sim, int items, int F,
     const int blocks = (int)std::min<int64_t>(rows, 64 * (int64_t)sm_count());
     if (blocks > 0) {
         prof_begin(kKMisc, st);
-        k_spectra_export<<<blocks, 128, 0, st>>>(sre, sim, rows, F, Spad, S,
-                                                 reinterpret_cast<float2*>(dst));
+        k_spectra_export<<<blocks, 128, 0, st>>>(sre, sim, rows, F, Spad, S, dst);
         prof_end(kKMisc, st);
     }
 }

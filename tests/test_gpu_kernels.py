@@ -220,6 +220,37 @@ def test_weights_near_the_top_of_fp32(precision):
     plan.close()
 
 
+@pytest.mark.parametrize("geometry", [(6.0, 150, 0.01, 360), (6.0, 40, 0.0375, 72),
+                                      (6.0, 33, 0.045, 84)], ids=str)
+def test_spectra_into_an_array_that_is_not_8_byte_aligned(geometry):
+    """The C calls write spectra to any float address: the same values one float further
+    on, and nothing on either side of them."""
+    import ctypes as C
+    import torch
+    from paper_2111_00171_gb300 import acom
+    lib = acom.load_library()
+    plan = au_plan(*geometry)
+    scan = to_dev(synth.random_patterns(13, n_patterns=5))
+    pk = plan._csr(*scan)
+    stream = torch.cuda.current_stream().cuda_stream
+
+    def polar(ptr):
+        assert lib.acom_polar_spectra(plan.handle, C.byref(pk), C.c_void_p(ptr), None,
+                                      C.c_void_p(stream)) == 0
+
+    def spectra(ptr):
+        assert lib.acom_plan_get_spectra(plan.handle, C.c_void_p(ptr), C.c_void_p(stream)) == 0
+
+    for call, want in ((polar, plan.polar_spectra(*scan)[0]), (spectra, plan.spectra())):
+        buf = torch.full((want.numel() + 3,), -7.0, device="cuda")
+        assert buf.data_ptr() % 8 == 0
+        call(buf.data_ptr() + 4)
+        torch.cuda.synchronize()
+        assert torch.equal(buf[1:-2], want.reshape(-1))
+        assert float(buf[0]) == -7.0 and bool((buf[-2:] == -7.0).all())
+    plan.close()
+
+
 @pytest.mark.parametrize("geometry", [(6.0, 150, 0.01, 360), (6.0, 75, 0.02, 180)], ids=str)
 @pytest.mark.parametrize("precision", [1, 2], ids=["bf16", "fp16"])
 def test_sixteen_bit_copies_with_one_and_two_staging_buffers(geometry, precision):
