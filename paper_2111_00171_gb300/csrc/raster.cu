@@ -504,7 +504,9 @@ size_t raster_fft_smem_bytes(int N, int F, size_t peak_bytes) {
 
 // Barrier of the warps' arrivals on a staged tile (below).  Every warp arrives on every
 // tile, so a wait ends; the count only keeps a broken invariant from hanging the GPU.
-__device__ __forceinline__ void tile_wait(uint64_t* bar, uint32_t parity) {
+// False if it gave up (the caller's copy may then hold part of a tile): the kernel sets
+// the error word at the item's end, so that the call reports a time-out.
+__device__ __forceinline__ bool tile_wait(uint64_t* bar, uint32_t parity) {
     const uint32_t b = (uint32_t)__cvta_generic_to_shared(bar);
     for (int i = 0; i < (1 << 22); ++i) {
         uint32_t ok;
@@ -517,8 +519,9 @@ __device__ __forceinline__ void tile_wait(uint64_t* bar, uint32_t parity) {
             : "=r"(ok)
             : "r"(b), "r"(parity)
             : "memory");
-        if (ok) return;
+        if (ok) return true;
     }
+    return false;
 }
 __device__ __forceinline__ void tile_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(
@@ -570,6 +573,8 @@ k_raster_fft(RasterGeom geo, Loader ld, int64_t n_items, RasterOut out, FftRadix
     const int dbl_peaks =
         XB == 0 ? -1
                 : (int)((reinterpret_cast<unsigned char*>(stage2) - smem) / (ptrdiff_t)sizeof(PeakT));
+    // one pair of shells a warp and tile: a warp waits for a buffer and arrives once a tile
+    static_assert(kFftTile / 2 == W, "a staged tile has one pair of shells per warp");
     uint64_t* tile_bar = reinterpret_cast<uint64_t*>(s_int + 32);       // [2]
     if (XB != 0 && threadIdx.x == 0) {
         for (int i = 0; i < 2; ++i)
@@ -579,6 +584,7 @@ k_raster_fft(RasterGeom geo, Loader ld, int64_t n_items, RasterOut out, FftRadix
                          : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    bool lost = false;                   // a tile's wait gave up
     uint32_t tile_ph = 0;                // bit i: parity of buffer i's next use
     if (!pfa)
         for (int i = threadIdx.x; i < N; i += blockDim.x) {
@@ -835,7 +841,7 @@ k_raster_fft(RasterGeom geo, Loader ld, int64_t n_items, RasterOut out, FftRadix
                 if (XB != 0 && stg && dbl) {
                     if (out_t0 >= 0) {               // the tile before this one
                         const int pb = (staged - 1) & 1;
-                        tile_wait(tile_bar + pb, (tile_ph >> pb) & 1u);
+                        lost |= !tile_wait(tile_bar + pb, (tile_ph >> pb) & 1u);
                         tile_ph ^= 1u << pb;
                         copy_tile(pb ? stage2 : stage, out_t0);
                     }
@@ -908,10 +914,11 @@ k_raster_fft(RasterGeom geo, Loader ld, int64_t n_items, RasterOut out, FftRadix
         }
         if (XB != 0 && out_t0 >= 0) {
             const int pb = (staged - 1) & 1;
-            tile_wait(tile_bar + pb, (tile_ph >> pb) & 1u);
+            lost |= !tile_wait(tile_bar + pb, (tile_ph >> pb) & 1u);
             tile_ph ^= 1u << pb;
             copy_tile(pb ? stage2 : stage, out_t0);
         }
+        if (XB != 0 && lost) atomicOr(err, kErrTimeout);
         if (w_lo < w_hi) {
             atomicMin(&s_int[40], w_lo);
             atomicMax(&s_int[41], w_hi);

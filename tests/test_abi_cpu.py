@@ -138,3 +138,27 @@ def test_autotune_and_tile_order_argument_checks_on_host(lib):
         fields = _header_struct_fields(name)
         assert [f for f, _ in mirror._fields_] == fields, name
         assert C.sizeof(mirror) == 4 * len(fields), name
+
+
+def test_bounded_barrier_waits_report_that_they_gave_up():
+    """Every device wait on a shared-memory barrier that is bounded by a count or a budget of
+    its own sets kErrTimeout in the error word when it runs out, itself or where it is called
+    (the waits before a CTA's exit, which only let copies land, call mbar_try and are not
+    meant).  None of them can be made to run out on a GPU without breaking its kernel."""
+    csrc = os.path.join(ROOT, "paper_2111_00171_gb300", "csrc")
+    waits = {}
+    for name in sorted(os.listdir(csrc)):
+        text = open(os.path.join(csrc, name)).read()
+        for m in re.finditer(r"^__device__ __forceinline__ (\w+) (\w+)\([^)]*\) \{\n(.*?)^\}",
+                             text, flags=re.S | re.M):
+            result, wait, body = m.groups()
+            if "for (" in body and ("try_wait" in body or "mbar_try" in body):
+                waits[wait] = (result, body, text)
+    assert {"mbar_wait", "tile_wait"} <= set(waits)
+    for wait, (result, body, text) in waits.items():
+        if "atomicOr(err, kErrTimeout)" in body:
+            continue
+        assert result == "bool", wait
+        calls = re.findall(r"(.*)\b" + wait + r"\(tile_bar", text)
+        assert calls and all(c.strip() == "lost |= !" for c in calls), wait
+        assert re.search(r"lost\) atomicOr\(err, kErrTimeout\);", text), wait
