@@ -114,6 +114,8 @@ constexpr float kFp16Target = 16384.0f;
 // Absolute error of an FP16 operand below the normal range (|x| < 2^-14),
 // whether the value is rounded to a subnormal or flushed to zero
 constexpr double kFp16Eta = 6.103515625e-05;   // 2^-14
+// and of an FP16 pair: half the spacing of the subnormals that the low half takes
+constexpr double kPairEta = 2.98023223876953125e-08;   // 2^-25
 // E4M3 operands: the FP16 operands times 2^-6 (|x| <= 2^8 < 448, exact), so
 // the pattern and plan scales are the FP16 ones times 2^-6; below E4M3's
 // normal range (2^-6) an operand is off by at most 2^-6

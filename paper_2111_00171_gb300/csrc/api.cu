@@ -743,6 +743,26 @@ static float kappa_fp32(const acom_plan_s* p) {
     return (float)((3.0 * (p->Spad + 2) + 2.0 * p->F) * std::ldexp(1.0, -24));
 }
 
+// FP32 operands as FP16 pairs (k_contract_bound_split), in units of 2^-24 ||P^_f|| ||X^_f||.
+// The errors eA .. eD of the four real products add up to |eA + eB| and |eC + eD|, each at
+// most e ||P^_f|| ||X^_f|| when a real product is off by e ||p|| ||x||: a factor sqrt 2.
+//   operands: x = hi + lo + d with |d| <= 2^-22 |x| (two roundings to 11 bits), twice, and
+//     the dropped lo lo, at most 2^-22 |p| |x|: 12 units, 17 with the factor;
+//   accumulation: a step adds 16 exact products to the accumulator, each of the 17 terms
+//     cut below the last FP32 bit of the largest, so by at most 2^-23 ||p|| ||x|| over the
+//     K tile's shells: 34 units a step.  Four hi hi steps a tile (136), eight cross steps
+//     2^-11 as large, and the two tiles' sum (1): 194.  The two tiles' norms add up to no
+//     more than the whole rows' (Cauchy-Schwarz);
+//   magnitude: 8 roundings of the square, half of that in the root, and 2 of the
+//     approximate root: 6;
+//   frequencies: the sum, 2 F as for FP32.
+// 217, taken as 220; the FP32 constant where that is larger (more than 64 shells).  A value
+// so small that its lo is below FP16's normal range is off by up to 2^-25 after scaling
+// (FP16 subnormals are multiplied as they are): select charges that as it does for FP16.
+static float kappa_pairs(const acom_plan_s* p) {
+    return (float)((std::max(3.0 * (p->Spad + 2), 220.0) + 2.0 * p->F) * std::ldexp(1.0, -24));
+}
+
 // BF16 operands: each product carries at most 2^-7 relative rounding, and
 // |Pr|+|Pi| <= sqrt(2)|P^| (same for X^) gives 2^-6 ||P^_f|| ||X^_f|| for the
 // complex spectrum; the tensor-core FP32 accumulation is charged 8x the FP32
@@ -878,9 +898,10 @@ static acom_status match_enqueue(acom_plan p, const acom_peaks_csr* peaks,
                 launch_contract_bound_fp32(p, w.Xr, w.Xi, nb, ts, w.U, w.extra, st);
             }
             launch_select_exact(p, w.Xsr, w.Xsi, w.U, w.extra, ts, w.xfn, w.srange, w.rmask, p->pfmax,
-                                w.xnorm2, nb, tc ? kappa_tc(p) : kappa_fp32(p), refine, *out,
-                                c0, p->err + 1, st, xscale, rescore_top, w.oin, w.onbr,
-                                &taken);
+                                w.xnorm2, nb,
+                                tc ? kappa_tc(p) : (pairs16 ? kappa_pairs(p) : kappa_fp32(p)),
+                                refine, *out, c0, p->err + 1, st, pairs16 ? w.xscale : xscale,
+                                rescore_top, w.oin, w.onbr, &taken);
             if (out->phi3 || out->orient)
                 launch_orient_compose(p, w.oin, w.onbr, nb, refine, *out, c0, st);
         }

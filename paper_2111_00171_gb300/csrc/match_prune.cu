@@ -494,7 +494,7 @@ struct SelectArgs {
     int64_t off;
     int* n_eval;                      // [0] total axes evaluated, [1] patterns taken
     int taken;                        // n_eval[1] when this launch starts
-    const float* xscale;              // [nb] 2^e of FP16 pattern spectra, or nullptr
+    const float* xscale;              // [nb] 2^e of FP16 pattern spectra or pairs, or nullptr
     float inv_pscale;                 // 2^-k of the plan operand's scale
     float xs_mul;                     // the pattern operand holds xscale * xs_mul times X^
     float eta;                        // absolute error of an operand below its normal range
@@ -1437,10 +1437,11 @@ void launch_select_exact(const acom_plan_s* p, const float* Xsr, const float* Xs
     SelectArgs a{p->Psr, p->Psi, Xsr, Xsi, U, extra, ts, xfn, srange, rmask, pfmax, xnorm2, p->za, p->frames,
                  p->nbr_ptr,
                  p->nbr_idx, p->phase_off, p->n_phases, p->Z, p->F, p->N, p->S, p->Spad, nb, refine, kappa,
-                 fft_radices(p->N), out, off, n_eval, *taken, xscale, 1.0f / p->pscale,
+                 fft_radices(p->N), out, off, n_eval, *taken, xscale,
+                 1.0f / (p->Ps ? fp16_plan_scale(p->N) : p->pscale),
                  p->precision == ACOM_PREC_FP8 ? kFp8Shift : 1.0f,
-                 (float)(p->precision == ACOM_PREC_FP8 ? kFp8Eta : kFp16Eta), rescore_top,
-                 p->smask, oin, onbr};
+                 (float)(p->precision == ACOM_PREC_FP8 ? kFp8Eta : (p->Ps ? kPairEta : kFp16Eta)),
+                 rescore_top, p->smask, oin, onbr};
     a.eta_rs = (float)((double)a.eta * std::sqrt((double)p->Spad));
     const size_t smem = select_smem_bytes(p->Z, p->N, p->F, p->Spad);
     const bool pfa = p->N == 360;

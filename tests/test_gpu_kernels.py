@@ -200,6 +200,61 @@ def test_fp16_pairs_in_few_and_in_many_tiles(geometry, patterns):
     plan.close()
 
 
+@pytest.mark.parametrize("geometry", [(3.0, 33, 0.045, 180), (3.0, 60, 0.025, 180),
+                                      (3.0, 75, 0.02, 180)], ids=str)
+def test_margin_of_the_fp16_pairs(geometry):
+    """The search's rounding margin covers what the FP16 pairs can be off by: 220 + 2 F units
+    of 2^-24 (operands 17, accumulation 194, magnitude 6; the sum over frequencies).  An
+    axis that was not evaluated reports its bound plus the margin."""
+    import torch
+    plan = au_plan(*geometry)
+    peaks = to_dev(synth.random_patterns(14, n_patterns=40))
+    U = plan.bounds(*peaks).double()
+    top = plan.match(*peaks, za_scores=True, refine=False)["za_scores"].double()
+    margin = top - U * (1.0 + 1e-5)
+    margin[margin <= 0] = float("nan")                # evaluated: the exact score
+    got = margin.nanmedian(dim=1).values              # (sums in FP32 round by 1 % of it)
+    _, scale = bounds64(plan, peaks)
+    need = (220 + 2 * plan.info["n_freq"]) * 2.0 ** -24 * scale
+    assert (got >= 0.99 * need).all()
+    plan.close()
+
+
+def test_fp16_pairs_of_values_far_below_the_largest():
+    """A peak that no axis' rows reach but 10^6 times as heavy as the others takes the scale
+    of the pairs, so that the others' low halves are FP16 subnormals: their bounds are off
+    by no more than those halves' spacing allows, and the match finds the winners that the
+    patterns have without that peak."""
+    import torch
+    plan = au_plan(3.0, 150, 0.01, 360)
+    scan = synth.random_patterns(15, n_patterns=24)
+    n = np.diff(scan.row_ptr)
+    at = scan.row_ptr[:-1]                            # the heavy peak before each pattern's own
+    heavy = synth.Scan(scan.row_ptr + np.arange(25), np.insert(scan.qx, at, 0.1).astype(np.float32),
+                       np.insert(scan.qy, at, 0.0).astype(np.float32),
+                       np.insert(scan.I, at, scan.I.max() * 1e12).astype(np.float32),
+                       scan.truth, scan.phase, scan.crystals, "a heavy peak")
+    assert (np.diff(heavy.row_ptr) == n + 1).all() and plan.info["k0"] * 0.01 > 0.1 + 0.08
+    peaks = to_dev(heavy)
+    want, _ = bounds64(plan, peaks)
+    P = torch.view_as_complex(plan.spectra()).to(torch.complex128)[:, plan.info["k0"]:]
+    N, F = plan.info["n_phi"], plan.info["n_freq"]
+    w = torch.full((F,), 2.0 / N, dtype=torch.float64, device="cuda")
+    w[0] = w[-1] = 1.0 / N
+    # 2^-25 of a scaled value: the scale is above 2^13 / B, B the sum of the peaks' weights
+    # times the bins that their tents cover, all 360 of them at most
+    q = np.hypot(heavy.qx.astype(float), heavy.qy)
+    B = np.add.reduceat(q * np.sqrt(heavy.I.astype(float)) * 360, heavy.row_ptr[:-1])
+    off = torch.from_numpy(B).cuda() * 2.0 ** -38
+    # four real products, 118 shells
+    tol = 4 * math.sqrt(118.0) * off[:, None] * (w * P.norm(dim=1)).sum(1)[None]
+    tol = tol + 2.0 ** -17 * want
+    assert ((plan.bounds(*peaks).double() - want).abs() <= tol).all()
+    got, alone = plan.match(*peaks), plan.match(*to_dev(scan))
+    assert ((got["score"] - alone["score"]).abs() <= 2e-6 * alone["score"]).all()
+    plan.close()
+
+
 @pytest.mark.parametrize("precision", [0, 2], ids=["fp32", "fp16"])
 def test_weights_near_the_top_of_fp32(precision):
     """Peak weights up to 1e36 (omega 2, so a weight is its intensity times q): the FP16
