@@ -91,8 +91,8 @@ __device__ __forceinline__ float peak_weight(float x, float y, float I, float ga
     return qg * iw;
 }
 
-// 2^x by the hardware's approximation alone (exp2f is the same value, scaled against
-// results below 2^-126; here those are 0, below the last bit of any sum they enter)
+// 2^x by ex2.approx.ftz (PTX: relative error at most 2^-22, subnormal results 0).  A peak's
+// Gaussian that small is below the last bit of any sum it enters.
 __device__ __forceinline__ float exp2_ftz(float x) {
     float r;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
