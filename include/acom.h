@@ -36,10 +36,15 @@ typedef enum {
 
 /* Arithmetic used by the shell contraction and the inverse transform. */
 typedef enum {
-    ACOM_PREC_FP32 = 0,   /* FP32 operands (reference GPU path): the contraction on CUDA
-                             cores, or with each value as a pair of FP16 values on
-                             the tensor cores where that is no less accurate (at
-                             most 128 shells past the plan's first, n_phi >= 180) */
+    ACOM_PREC_FP32 = 0,   /* FP32 operands (reference GPU path).  The contraction of
+                             acom_match and acom_bounds runs on CUDA cores, or with
+                             each value as a pair of FP16 values on the tensor
+                             cores where its error against FP64 is no larger (at
+                             most 128 shells past the plan's first, n_phi >= 180;
+                             peak intensities within a factor of 1e10 of each
+                             other).  A plan that finds no room for the pairs
+                             keeps the CUDA cores.  acom_bounds_static and
+                             exhaustive matches always use them             */
     ACOM_PREC_BF16 = 1,   /* BF16 operands on tcgen05 tensor cores, FP32 accumulate,
                              top candidates re-scored in FP32                       */
     ACOM_PREC_FP16 = 2,   /* FP16 operands on tcgen05 tensor cores, FP32 accumulate;
@@ -499,23 +504,27 @@ acom_status acom_kinematical_score_strain(acom_plan plan, const acom_peaks_csr* 
  * direct and mirror correlation spectra, which is >= max over phi3 of both C
  * and C_mirror (section "Correlation Pattern Matching"; w_0 = w_{N/2} = 1,
  * else 2).  Computed at the plan's precision (FP32, or BF16 / FP16 tensor cores
- * with FP32 accumulation) without any rounding margin.  ``dst``: DEVICE
+ * with FP32 accumulation) without any rounding margin.  The frequencies are summed
+ * in groups that depend on the number of patterns, axes and SMs, so a pattern's
+ * bounds may differ in their last bits between batches.  ``dst``: DEVICE
  * [n_patterns][Z] FP32.  Stream-ordered; synchronises once to read the error word.
  */
 acom_status acom_bounds(acom_plan plan, const acom_peaks_csr* peaks, float* dst,
                         void* cuda_stream);
 
 /*
- * acom_bounds_static - the same result as acom_bounds, computed without
+ * acom_bounds_static - the bounds of acom_bounds, to rounding, computed without
  * allocating any device memory.  The paper has no counterpart: this entry
  * point exists for callers that must not allocate while they run, such as an
  * acquisition loop that reserved its whole device-memory budget up front, or
  * a host process whose device memory is held by another allocator (a
  * cudaMalloc there could fail or stall).  The plan must already exist; the
  * caller passes the peaks and ``dst`` ([n_patterns][Z] FP32, DEVICE), as for
- * acom_bounds.  FP32 and BF16 plans get their own precision's bounds; FP16
- * and FP8 (E4M3) plans get the bounds of the FP32 path (every plan keeps its
- * FP32 spectra), i.e. the values an FP32 plan's acom_bounds returns.  Peak data
+ * acom_bounds.  BF16 plans get their own precision's bounds, all others those
+ * of the FP32 contraction on CUDA cores (every plan keeps its FP32 spectra).
+ * All frequencies are summed in one chain, where acom_bounds may sum them in
+ * groups or multiply FP16 pairs (ACOM_PREC_FP32): the two agree to FP32
+ * rounding, not bit for bit.  Peak data
  * are checked as for acom_bounds (row_ptr[0] == 0, monotone rows, finite values,
  * at most 1024 peaks per pattern): a violation returns ACOM_ERR_BAD_INPUT.
  *
