@@ -122,6 +122,45 @@ def test_refined_axis_with_more_neighbours_than_are_handed_on():
     plan.close()
 
 
+def test_orientation_from_more_neighbours_than_are_handed_on():
+    """Patterns along axes of such a grid, whose winners' neighbours are counted: at least
+    half of them have the oracle's winner (a tie may be resolved the other way), each with
+    more than 32 neighbours, and then its orientation."""
+    from oracle import acom_oracle as O
+    from gpu_common import au_refl
+    from paper_2111_00171_gb300 import acom
+    tri = [[0, 0, 1], [0, 0.1, 1], [0.1, 0.1, 1]]
+    area = 4.0 * (14 * math.radians(2.0)) ** 2 / 8.0
+    plan = acom.Plan(acom.au_crystal(), tri, area, 2.0, 40, 0.0375, 72, lam=LAM)
+    za = O.zone_axis_grid(*tri, 2.0, area)
+    oplan = O.orientation_plan(au_refl(), za, O.PlanParams(40, 0.0375, 72, 0.08, lam=LAM))
+    rng = np.random.default_rng(16)
+    spec = synth.au_fcc()
+    g, F2 = synth.reflection_table(spec, 1.5)
+    lists, truth = [], []
+    for i in rng.choice(len(za), 12, replace=False):
+        m = np.linalg.qr(np.column_stack([za[i], rng.normal(size=(3, 2))]))[0]
+        m = m[:, [1, 2, 0]] * np.sign(m[:, 0] @ za[i])        # the beam along the axis
+        m[:, 0] *= np.sign(np.linalg.det(m))
+        lists.append(synth._sorted_list(g, F2, m, LAM, 0.02))
+        truth.append(m)
+    scan = synth.Scan(*synth._assemble(lists, np.full(12, 30), rng, 0.005, 0.1), np.array(truth),
+                      np.zeros(12, np.int32), (spec,), "axes of a narrow grid")
+    r = plan.match(*to_dev(scan))
+    m = r["orient"].cpu().numpy()
+    same = 0
+    for b in range(scan.n_patterns):
+        mt = O.match_pattern(oplan, *scan.pattern(b))
+        if (int(r["za_idx"][b]), int(r["phi3_bin"][b]), int(r["mirror"][b])) != (mt.za, mt.k, mt.mirror):
+            continue
+        same += 1
+        assert (za @ za[mt.za] >= math.cos(math.radians(3.0))).sum() > 32
+        # FP32 scores weight the mean: 1e-5 relative, over a neighbourhood of 3 degrees
+        np.testing.assert_allclose(m[b], O.refine(mt, za, 2.0).m, atol=1e-4)
+    assert same >= 6
+    plan.close()
+
+
 @pytest.mark.parametrize("precision", [0, 2], ids=["fp32", "fp16"])
 def test_bins_with_a_prime_factor_above_five(precision):
     """84 = 4 * 3 * 7 bins take the direct transform: the certified match finds the
