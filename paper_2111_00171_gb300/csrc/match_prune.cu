@@ -196,25 +196,34 @@ void launch_contract_bound_fp32(const acom_plan_s* p, const float* Xr, const flo
     prof_end(kKContract, st);
 }
 
-// a split tile's later groups onto its first, eight at a time: a small batch's tiles are
-// cut into up to a frequency each, and one chain of that many FP32 additions rounds more
-// than a whole tile's sum (split_shells).  Eight loads go out together: with the 45 later
-// groups of 100 patterns x 231 axes the select kernel takes 34.8 us, 38.9 one by one.
-__device__ __forceinline__ float later_groups(const TileSplit& ts, const float* __restrict__ extra,
-                                              int b, int z, float u) {
-    const int t = ts.groups > 1 ? ts.split_tile(b, z) : -1;
-    if (t >= 0) {
-        const float* p = extra + ts.extra_at(1, t, b, z);
-        const int64_t plane = ts.extra_at(2, t, b, z) - ts.extra_at(1, t, b, z);
-        int left = ts.groups - 1;
-        for (; left >= 8; left -= 8, p += 8 * plane)
-            u += ((p[0] + p[plane]) + (p[2 * plane] + p[3 * plane])) +
-                 ((p[4 * plane] + p[5 * plane]) + (p[6 * plane] + p[7 * plane]));
+// Adds `left` values `plane` apart to u, 32 at a time: their loads go out together, and
+// their sum is a tree of fours, then a chain.
+__device__ __noinline__ float add_groups(const float* __restrict__ p, int64_t plane, int left,
+                                         float u) {
+    for (; left > 0; left -= 32, p += 32 * plane) {
+        float v[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = j < left ? p[j * plane] : 0.f;
         float s = 0.f;
-        for (; left > 0; --left, p += plane) s += *p;
+#pragma unroll
+        for (int j = 0; j < 32; j += 4) s += (v[j] + v[j + 1]) + (v[j + 2] + v[j + 3]);
         u += s;
     }
     return u;
+}
+
+// A split tile's later groups onto its first.  A small batch's tiles are cut into up to a
+// frequency a group, and one chain of that many FP32 additions rounds more than a whole
+// tile's sum (split_shells).  Called and not inlined: most tiles of a large batch are not
+// split, and the select kernel is faster without the code.  Select, in one chain inlined /
+// here: 65,536 patterns x 903 axes 7.78 / 7.76 ms, 16,000 x 3,486 2.47 / 2.43 ms, 100 x 231
+// (45 later groups) 38.4 / 34.8 us, one pattern x 903 (18) the same within 4 %.
+__device__ __forceinline__ float later_groups(const TileSplit& ts, const float* __restrict__ extra,
+                                              int b, int z, float u) {
+    const int t = ts.groups > 1 ? ts.split_tile(b, z) : -1;
+    return t < 0 ? u
+                 : add_groups(extra + ts.extra_at(1, t, b, z),
+                              (int64_t)ts.tiles() << (ts.lb + ts.lz), ts.groups - 1, u);
 }
 
 __global__ void k_sum_groups(TileSplit ts, float* __restrict__ U, const float* __restrict__ extra,

@@ -695,11 +695,11 @@ constexpr size_t tc_smem_bytes() {
 // the cross terms, 2^-11 of the rest, then four hi hi steps; the epilogue adds
 // the two tiles' accumulators of a frequency rounding to nearest, and the sum
 // over frequencies runs in groups of a quarter (a split tile's: a group a unit, added
-// eight at a time).  The bound's error against FP64 is then no larger than the FP32
+// by add_groups).  The bound's error against FP64 is then no larger than the FP32
 // kernel's with its one sum over all frequencies.  Relative 2-norms over whole and split
 // tiles, 8 to 8,000 patterns of three kinds of peak lists, 66 to 1,378 axes: 1.1e-7 to
-// 1.7e-7 against 3.0e-7 to 3.4e-7 on 150 shells and 360 bins, 1.0e-7 to 1.6e-7 against
-// 2.0e-7 to 2.2e-7 on 75 and 180, 0.7e-7 to 1.4e-7 against 2.4e-7 to 3.1e-7 on 100 and 240
+// 1.7e-7 against 3.0e-7 to 3.4e-7 on 150 shells and 360 bins, 0.9e-7 to 1.5e-7 against
+// 2.0e-7 to 2.2e-7 on 75 and 180, 0.6e-7 to 1.4e-7 against 2.4e-7 to 3.1e-7 on 100 and 240
 // and on 117 and 300; the same shares on a hexagonal crystal (split_shells says where not).
 // With the up to 91 groups of a small batch of few axes added in one chain the 75 x 180
 // plan was at 2.6e-7 against 2.0e-7.
@@ -1432,8 +1432,8 @@ void launch_contract_bound_tc(const acom_plan_s* p, const void* map_x, int pt_st
 // against FP64 is not clearly below the FP32 kernel's.  More than two K tiles need more
 // than four hi hi steps per accumulation (eight on all-positive spectra: 4.8e-7 against
 // 2.4e-7).  With few bins the FP32 kernel's sum over the few frequencies rounds as little
-// as the truncation does: up to 1.00 of its error at 100 bins (1.47e-7 against 1.46e-7), 0.93
-// at 72, 0.90 at 144, 0.83 at 160, and at most 0.77 from 180 bins on.
+// as the truncation does: up to 0.99 of its error at 100 bins (1.46e-7 against 1.46e-7), 0.94
+// at 72, 0.87 at 144, 0.81 at 160, and at most 0.72 from 180 bins on.
 int split_shells(const acom_plan_s* p) {
     const int K = (p->S - p->k0 + 15) / 16 * 16;
     const bool smaller_error = K > 0 && K <= 2 * tc::kKT && p->N >= 180;
