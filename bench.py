@@ -735,7 +735,7 @@ def sweep_combos(args, acom, lib, scan, d_in, flush, stream, n_oracle=1000):
             prof = read_profile(lib, acom)
             name = "contract_fp32" if prec == "fp32" else "contract_tc"
             cnt, cms = prof.get(name, (0, 0.0))
-            flops = 8.0 * Z * S * F * B
+            flops = 8.0 * Z * (S - info["k0"]) * F * B
             tflops = flops / (cms / 1e3) / 1e12 if cms else 0.0
             # E4M3's dense rate is twice BF16's (4.5 vs 2.25 PFLOP/s nominal)
             alu = prec == "fp32" and not fp32_on_tensor_cores(S, info["k0"], N)
@@ -837,11 +837,11 @@ def read_profile(lib, acom):
 # the patterns of a launch (then another chunk size is scaled); the
 # contraction's does not (the plan is re-read once per tile wave).
 TRAFFIC_PER_LAUNCH = {
-    "select_exact": (5.341e9 + 20.85e6, 32768, ("match_prune.cu",), "5542e2567c0d4a2d", "fp16",
+    "select_exact": (5.312e9 + 24.53e6, 32768, ("match_prune.cu",), "6fb0bd2336ceadd8", "fp16",
                      "au_scan_256x256_1deg", True),
-    "raster_patterns": (21.56e6 + 8.031e9, 32768, ("raster.cu",), "65f790beeba11713", "fp16",
+    "raster_patterns": (14.77e6 + 8.031e9, 32768, ("raster.cu",), "7ea1939508e2b80a", "fp16",
                         "au_scan_256x256_1deg", True),
-    "contract_tc": (7.005e9 + 115.2e6, 32768, ("match_tc.cu",), "98bbb62117c87ae7", "fp16",
+    "contract_tc": (5.809e9 + 114.8e6, 32768, ("match_tc.cu",), "a32de7d9535773e4", "fp16",
                     "au_scan_256x256_1deg", False),
 }
 
@@ -885,21 +885,22 @@ def kernel_roofline(name, cnt, ms, peaks, src, B, K, nnz, precision, refine_pair
     if name == "contract_tc":
         # the kernel runs for a few ms at a time within a short step, at the
         # maximum SM clock (clocks sampled beside): the burst peak applies
-        work, unit, bound, peak = 8.0 * Z * S * F * pats, "TFLOP/s", "tensor", \
+        work, unit, bound, peak = 8.0 * Z * (S - k0) * F * pats, "TFLOP/s", "tensor", \
             peaks["bf16_tflops"]
-        note = (f"8 Z S F flops per pattern; bf16 burst peak, which FP16 operands "
-                f"share ({src})")
-        if k0:
-            note += (f"; the kernel skips shells 0..{k0 - 1}, where every plan row is zero "
-                     f"(it executes {W['S'] - k0} of the {W['S']} shells counted)")
+        note = (f"8 flops per axis, frequency and shell from the plan's first non-zero one on "
+                f"({S - k0} of {S}); bf16 burst peak, which FP16 operands share ({src})")
     elif name == "contract_fp32" and rows_nz is not None and fp32_on_tensor_cores(S, k0, N):
-        work, unit, bound, peak = 8.0 * Z * S * F * pats, "TFLOP/s", "tensor", \
+        work, unit, bound, peak = 8.0 * Z * (S - k0) * F * pats, "TFLOP/s", "tensor", \
             peaks["bf16_tflops"]
-        note = (f"8 Z S F flops per pattern, each FP32 product taken as three of FP16 halves; "
+        note = (f"8 flops per axis, frequency and shell from the plan's first non-zero one on "
+                f"({S - k0} of {S}), each FP32 product taken as three of FP16 halves; "
                 f"bf16 burst peak ({src})")
     elif name == "contract_fp32":
-        work, unit, bound, peak = 8.0 * Z * S * F * pats, "TFLOP/s", "alu", fp32_peak
-        note = "8 Z S F flops per pattern; FP32 FMA peak 152 SMs x 128 lanes x 2 x max clock"
+        # exhaustive matches multiply every shell
+        used = S if rows_nz is None else S - k0
+        work, unit, bound, peak = 8.0 * Z * used * F * pats, "TFLOP/s", "alu", fp32_peak
+        note = (f"8 flops per axis, frequency and shell ({used} of {S}); "
+                f"FP32 FMA peak 152 SMs x 128 lanes x 2 x max clock")
     elif name == "select_exact":
         # compulsory HBM bytes: each pattern's FP32 shell-major spectra on
         # the shells its peaks reach (rows_nz of S, re/im) read once, and the
