@@ -920,15 +920,18 @@ def kernel_roofline(name, cnt, ms, peaks, src, B, K, nnz, precision, refine_pair
                 "FP32 FMA peak 152 SMs x 128 lanes x 2 x max clock")
     elif name == "raster_patterns":
         # algorithmic bytes: CSR in (8 B row pointer + 12 B per peak) and the
-        # spectra out: the contraction's operand (re/im, F frequencies: 16-bit
-        # on the shells from the plan's first non-zero shell k0 on, which are
-        # all the tensor-core contraction reads; FP32 frequency-major on all S
-        # shells for the FP32 contraction) and the FP32 shell-major rows
-        # select reads, those of the shells the pattern's peaks reach (rows_nz
-        # of S; the raster writes no other row)
+        # spectra out: the contraction's 16-bit operand (re/im, F frequencies, on
+        # the shells from the plan's first non-zero shell k0 on, which are all the
+        # tensor-core contraction reads; FP32 frequency-major on all S shells for
+        # exhaustive matches; FP32 plans' operands are other kernels' output) and
+        # the FP32 shell-major rows select reads, those of the shells the
+        # pattern's peaks reach (rows_nz of S; the raster writes no other row)
         rows = S if rows_nz is None else rows_nz
-        op_shells = S if precision == "fp32" else S - k0
-        out_b = op_shells * F * 2 * (4 if precision == "fp32" else 2) + rows * F * 8
+        if rows_nz is None:
+            op_shells, op_bytes = S, 8
+        else:
+            op_shells, op_bytes = (0, 0) if precision == "fp32" else (S - k0, 4)
+        out_b = op_shells * F * op_bytes + rows * F * 8
         work = (nnz / B * 12 + 8 + out_b) * pats / 1e9
         unit, bound, peak = "GB/s", "hbm", peaks["hbm_gbs"]
         note = (f"CSR in + contraction operand on {op_shells} shells out + FP32 shell-major "
